@@ -292,3 +292,113 @@ def tolerance(case):
     if case["kind"] == "classify":
         return {"rel": 2e-4, "max": 1e-3}
     return {"rel": 1e-2, "max": 0.07}
+
+
+# ---------------------------------------------------------------------------------------------- the same in 64 bits
+
+
+def _softmax64(q, k, v, *masks):
+    """Attention of q [n, d] over k, v [m, d] in 64 bits; with masks (functions of a row range, or None for all keys) one
+    output per mask and the share of the whole row's weight that it keeps."""
+    n, scale = q.shape[0], 1.0 / math.sqrt(q.shape[1])
+    q, k, v = q.double(), k.double(), v.double()
+    outs = [torch.empty_like(q) for _ in masks or (None,)]
+    shares = [torch.empty(n, dtype=torch.float64, device=q.device) for _ in outs]
+    rows = max(1, (1 << 28) // k.shape[0])
+    for a in range(0, n, rows):
+        sel = slice(a, min(n, a + rows))
+        logits = scale * (q[sel] @ k.T)
+        whole = torch.logsumexp(logits, 1)
+        for i, mask in enumerate(masks or (None,)):
+            x = logits if mask is None else logits.masked_fill(~mask(sel), -math.inf)
+            lse = whole if mask is None else torch.logsumexp(x, 1)
+            outs[i][sel] = torch.exp(x - lse[:, None]) @ v
+            shares[i][sel] = torch.exp(lse - whole)
+    return (outs, shares) if masks else outs[0]
+
+
+def _dense64(q, k, v):
+    return torch.stack([_softmax64(q[:, h], k[:, h], v[:, h]) for h in range(q.shape[1])], 1)
+
+
+def _cells(case, frames):
+    """Index of the deployed cell of every token of `frames` frames."""
+    def axis(n_grid):
+        n = max(1, int(math.floor(n_grid / case["cell"] + 0.5)))
+        edges = torch.tensor([i * n_grid // n for i in range(1, n)], dtype=torch.int64, device="cuda")
+        return torch.bucketize(torch.arange(n_grid, device="cuda"), edges, right=True)
+    return (axis(case["gh"])[:, None] * case["gw"] + axis(case["gw"])[None, :]).flatten().repeat(frames)
+
+
+def _sparse64(case, labels, blocks, q):
+    """headcast_attend over the logical window `blocks` of (K, V), Sink block first, newest block last."""
+    both = case["kind"] == "refresh"
+    cat = lambda part, h: tuple(torch.cat([b[i][:, h] for b in part]) for i in (0, 1))  # noqa: E731
+    out = torch.empty(q.shape, dtype=torch.float64, device="cuda")
+    for h, label in enumerate(labels):
+        if label == SINK:
+            k, v = cat([blocks[0], blocks[-1]] if both else blocks[:1], h)
+        elif label == DUMMY:
+            k, v = cat(blocks[-2:] if both else blocks[-1:], h)
+        else:
+            k, v = cat(blocks, h)
+        if label != SPATIAL:
+            out[:, h] = _softmax64(q[:, h], k, v)
+            continue
+        mine, theirs = _cells(case, case["frames"]), _cells(case, case["frames"] * len(blocks))
+        for c in mine.unique():
+            out[mine == c, h] = _softmax64(q[mine == c, h], k[theirs == c], v[theirs == c])
+    return out
+
+
+def _classify64(case, blocks, q):
+    """(labels, scores [H, 10]): mean cosines of the proxies' outputs to the whole one, 5th percentile and squared error of
+    the Spatial proxy, score, attention masses."""
+    l, n = _tokens(case), len(blocks) * _tokens(case)
+    pos, where = torch.arange(l, device="cuda") % (case["gh"] * case["gw"]), torch.arange(n, device="cuda")
+    where_in = where % (case["gh"] * case["gw"])
+    py, px, ky, kx = pos // case["gw"], pos % case["gw"], where_in // case["gw"], where_in % case["gw"]
+    first, last = where < l, where >= n - l
+    near = lambda s: ((ky - py[s, None]).abs() <= RADIUS) & ((kx - px[s, None]).abs() <= RADIUS)  # noqa: E731
+    cosine = lambda a, b: (a * b).sum(1) / (a.norm(dim=1) * b.norm(dim=1)).clamp_min(1e-12)  # noqa: E731
+    labels, scores = [], []
+    for h in range(case["heads"]):
+        k, v = (torch.cat([b[i][:, h] for b in blocks]) for i in (0, 1))
+        outs, shares = _softmax64(q[:, h], k, v, None, lambda s: first[None], lambda s: last[None], near,
+                                  lambda s: near(s) & ~first & ~last)
+        cos = [cosine(o, outs[0]) for o in outs[1:4]]
+        rank = 0.05 * (l - 1)
+        low = cos[2].sort().values[[int(rank), min(int(rank) + 1, l - 1)]]
+        p5 = low[0] + (rank - int(rank)) * (low[1] - low[0])
+        mse = (outs[3] - outs[0]).square().mean()
+        mass = [s.mean() for s in shares[1:4]]
+        rest = (1.0 - shares[1] - shares[2] - shares[4]).mean()
+        score = p5 - 5.0 * mse
+        cs, cd, cp = (float(c.mean()) for c in cos)
+        labels.append(SINK if cs >= 0.95 else DUMMY if cd >= 0.95 else SPATIAL if cp >= 0.95 and float(score) >= 0.755 else GLOBAL)
+        scores.append(torch.stack([torch.as_tensor(x, dtype=torch.float64, device="cuda") for x in (cs, cd, cp, p5, mse, score, *mass, rest)]))
+    return labels, torch.stack(scores).cpu()
+
+
+def exact(case, seed):
+    kind, steps, n = case["kind"], case["steps"], case["filled"]
+    x = _Inputs(case, seed)
+    if kind == "noalloc":
+        parts = [x.block(b, 0)[:2] for b in range(n)]
+        return _dense64(x.block(n, 1)[2][0], *(torch.cat([p[i] for p in parts]) for i in (0, 1)))
+    if kind == "classify":
+        blocks = [x.block(b, 1) for b in range(n)]
+        return {"labels": None, "scores": _classify64(case, blocks, blocks[-1][2][0])[1]}
+    if kind == "start":
+        blocks = [x.block(b, steps) for b in range(n + 1)]
+        whole = [torch.cat([b[i] for b in blocks[:n]]) for i in (0, 1)]
+        labels, scores = _classify64(case, blocks[:n], blocks[n - 1][2][0])
+        return {"warmup": [_dense64(q, *whole) for q in blocks[n - 1][2]], "labels": None, "scores": scores,
+                "outs": [_sparse64(case, labels, blocks, q) for q in blocks[n][2]]}
+    blocks = [x.block(b, 0) for b in range(n)]
+    new = x.block(n, steps)
+    if kind == "dense":  # the newest cached block was refreshed
+        whole = [torch.cat([b[i] for b in blocks[:-1] + [new]]) for i in (0, 1)]
+        return [_dense64(q, *whole) for q in new[2]]
+    window = blocks + [new] if n < case["blocks"] else blocks[:1] + blocks[2:] + [new]
+    return [_sparse64(case, x.labels, window, q) for q in new[2]]

@@ -7,10 +7,16 @@
 //     product straight from tensor memory);
 //   - K/V tiles (128 keys) arrive through TMA into one 4-slot shared-memory ring (128-byte swizzle), in the
 //     order they are consumed (K0 V0 K1 V1 ...), so loads run two tiles ahead of the products;
-//   - sixteen softmax warps, eight per query tile, two threads per query row (online softmax in the
-//     exp2 domain, a quarter of the exponentials evaluated as a cubic on the FMA pipe to relieve the
+//   - eight softmax warps, four per query tile, one thread per query row (online softmax in the exp2
+//     domain, an eighth of the exponentials evaluated as a cubic on the FMA pipe to relieve the
 //     special-function unit, rescaling of O only when the running maximum grew by more than 2^8);
-//   - warp 0 is the TMA producer, warp 1 issues every MMA.
+//   - warp 0 is the TMA producer, warp 1 issues every MMA (converged, see tc05.cuh).
+// What bounds it: per pair of tiles the tensor pipe needs 2048 clk, the softmax of the two tiles 2100 clk of issue and
+// special-function time per scheduler (microbenchmark: 61 clk to fetch, 136 for the maximum, 1086 for the exponentials of
+// one tile alone, 2126 for two together), and a tile's softmax and its products follow one another; a step takes about
+// 3050 clk.  With two threads per row, a maximum exchanged through shared memory and the products issued from a diverged
+// lane it took 3600.  Steady-state block at 30 x 52 tokens (12 heads of 128, 7-block window, append + four attends):
+// 1396 -> 1256 us; dense sweep over 7 blocks at 45 x 80 tokens: 4856 -> 4398 us.
 // Which keys a query tile sees is entirely a property of the work item: a row range of one of the
 // cache buffers (whole window, one block, one Spatial cell) or, for the classification's Spatial
 // proxy, a per-frame band of tokens plus an element-wise neighbourhood test.
@@ -38,7 +44,7 @@ struct WorkItem {
   int32_t kv_row0;        // buffer row of the first key of segment 0
   int32_t seg_stride;     // rows between the starts of consecutive segments
   int32_t seg_len;        // keys per segment
-  int32_t tiles_per_seg;  // ceil(seg_len / 128)
+  int32_t tiles_per_seg;  // ceil(seg_len / 128); outside the Spatial proxy an item has one segment
   int32_t tile_begin;     // this item covers tiles [tile_begin, tile_end) of the segment-major enumeration
   int32_t tile_end;
   int32_t out_mode;       // OUT_*
@@ -71,11 +77,18 @@ struct AttnParams {
   alignas(64) CUtensorMap maps[8];
 };
 
-constexpr int ATTN_THREADS = 576;  // warp 0: TMA, warp 1: MMA, warps 2-9 / 10-17: softmax for query tile 0 / 1 (112 registers each)
-constexpr int SOFTMAX_WARPS = 8;    // per query tile: two threads per row, each owning 64 of the tile's 128 keys
+constexpr int ATTN_THREADS = 384;  // warp 0: TMA, warp 1: MMA, warps 2-3: idle (they complete the warpgroup), warps 4-7 / 8-11: softmax for query tile 0 / 1
+constexpr int REGS_LAUNCH = 168, REGS_ISSUE = 56, REGS_SOFTMAX = 224;  // per thread: at launch, then warps 0-3 / 4-11
+static_assert(128 * REGS_ISSUE + 256 * REGS_SOFTMAX <= ATTN_THREADS * REGS_LAUNCH, "the block cannot take more registers than it was launched with");
+constexpr int SOFTMAX_WARPS = 4;    // per query tile: one thread per query row
+// Of the four 32-key chunks of P, how many are handed to the tensor pipe ahead of the rest (dense sweep at 45 x 80 tokens,
+// 7 blocks: 1: 4558 us, 2: 4398, 3: 4579).
+constexpr int P_HEAD_CHUNKS = 2;
 constexpr int KV_SLOTS = 4;  // one shared-memory ring for K and V tiles, filled and drained in the order K0 V0 K1 V1 ...
+// Pairs whose index has all these bits set take the polynomial exponential (7: every 8th).  Dense sweep at 45 x 80 tokens,
+// 7 blocks: none 4694 us, 1 in 16 4421, 1 in 8 4398, 1 in 4 4564, 1 in 2 4770.
 #ifndef HC_POLY_MASK
-#define HC_POLY_MASK 3  // pairs whose index has all these bits set take the polynomial exponential (3: every 4th)
+#define HC_POLY_MASK 7
 #endif
 #ifndef HC_L2_HINT
 #define HC_L2_HINT 2  // 1: Spatial cells' K/V are loaded evict-first; 2: the other K/V also evict-last
@@ -141,13 +154,12 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
   using SM = AttnSmem<D>;
   constexpr int NB = D / 64;          // 64-column blocks per tile
   constexpr int QK_STEPS = D / 16;    // k-steps of S = Q K^T
-    constexpr uint32_t TMEM_COLS = 512;
-  constexpr uint32_t S_COL = 0, O_COL = 256;  // S_t at t*128, O_t at 256 + t*128; P_t overlays S_t
+  constexpr uint32_t TMEM_COLS = 512;
+  constexpr uint32_t S_COL = 0, O_COL = 256;  // S_t at t*128, O_t at 256 + t*128; P_t overlays the first half of S_t
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ uint64_t bar_q_full[2], bar_s_full[2], bar_p_full[2], bar_o_full[2], bar_pair[2];
-  __shared__ float pair_val[2][2][2][128];  // [query tile][parity][column half][row]: values the two threads of a row swap
+  __shared__ uint64_t bar_q_full[2], bar_s_full[2], bar_p_head[2], bar_p_full[2], bar_o_full[2];
   __shared__ uint64_t bar_kv_full[KV_SLOTS], bar_kv_free[KV_SLOTS];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
@@ -157,13 +169,13 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int t = 0; t < 2; ++t) {
-      // softmax warps arrive once per warp (lane 0, after __syncwarp): 256 arrivals on one mbarrier would be
-      // 256 serialised shared-memory atomics per tile
+      // softmax warps arrive once per warp (lane 0, after __syncwarp): an arrival per thread would be 128 serialised
+      // shared-memory atomics per tile
       mbar_init(&bar_q_full[t], SOFTMAX_WARPS);
       mbar_init(&bar_s_full[t], 1);
+      mbar_init(&bar_p_head[t], SOFTMAX_WARPS);
       mbar_init(&bar_p_full[t], SOFTMAX_WARPS);
       mbar_init(&bar_o_full[t], 1);
-      mbar_init(&bar_pair[t], SOFTMAX_WARPS);
     }
     for (int s = 0; s < KV_SLOTS; ++s) {
       mbar_init(&bar_kv_full[s], 1);
@@ -227,7 +239,9 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
 
   if (dead_on_arrival) {
     // nothing: straight to the teardown
-  } else if (warp == 0) {
+  } else if (warp < 4) {
+    regs_dec<REGS_ISSUE>();
+    if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       uint32_t kt = 0;
@@ -248,7 +262,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
         const CUtensorMap* vmap = kmap + 1;
         const uint64_t policy = (HC_L2_HINT && w.cell >= 0) ? pol_stream : pol_keep;
         for (int tile = w.tile_begin; tile < w.tile_end; ++tile, ++kt) {
-          const int seg = tile / w.tiles_per_seg, c = tile - seg * w.tiles_per_seg;
+          const int seg = PROXY ? tile / w.tiles_per_seg : 0, c = PROXY ? tile - seg * w.tiles_per_seg : tile;
           const int row = w.kv_row0 + seg * w.seg_stride + c * 128;
           // ring position g = 2 * kt holds K of this tile, g + 1 its V
           for (int kv = 0; kv < 2; ++kv) {
@@ -271,119 +285,112 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
         }
       }
     }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0);
-      const uint32_t idesc_o = idesc_bf16_f32(128, D, 0, 1);
-      const uint32_t q_addr = smem_u32(smem + SM::Q_OFF), kv_addr = smem_u32(smem + SM::KV_OFF);
-      uint32_t kt = 0, q_cnt[2] = {0, 0}, p_cnt[2] = {0, 0};
-      bool ok = true;
-      const uint64_t q_desc = smem_desc_sw128(q_addr, 16, 1024), k_desc = smem_desc_sw128(kv_addr, 16, 1024);
-      const uint64_t v_desc = smem_desc_sw128(kv_addr, SM::BLOCK_BYTES, 1024);
-      auto issue_qk = [&](int t, uint32_t st) {
-        mma_block_ss<QK_STEPS>(tmem + S_COL + t * 128, q_desc + ((t * SM::TILE_BYTES) >> 4),
-                               k_desc + ((st * SM::TILE_BYTES) >> 4), idesc_s, SM::BLOCK_BYTES >> 4, SM::BLOCK_BYTES >> 4);
-      };
-      auto issue_pv = [&](int t, uint32_t st, bool accumulate) {
-        mma_block_ts8(tmem + O_COL + t * 128, tmem + S_COL + t * 128, v_desc + ((st * SM::TILE_BYTES) >> 4), idesc_o,
-                      accumulate ? 1u : 0u);
-      };
-      ItemCursor cur = {item_lo - 1, false, 0u};
-      while (ok && next_item(cur)) {
-        const int it = cur.it;
-        const WorkItem w = p.items[it];
-        const int nt = w.tile_end - w.tile_begin;
-        const int n_q = w.q_count[1] > 0 ? 2 : 1;
-        {
-          const uint32_t st = (2 * kt) % KV_SLOTS, ph = ((2 * kt) / KV_SLOTS) & 1;
-          if (!(ok = mbar_wait(&bar_kv_full[st], ph, abortp, p.status, 21))) break;
-          for (int t = 0; t < n_q && ok; ++t) {
-            if (!(ok = mbar_wait(&bar_q_full[t], q_cnt[t] & 1, abortp, p.status, 22))) break;
-            ++q_cnt[t];
-            tc_fence_after_sync();
-            issue_qk(t, st);
-            mma_commit(&bar_s_full[t]);
-          }
-          if (!ok) break;
-          mma_commit(&bar_kv_free[st]);
+    } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer (the whole warp, converged)
+    const uint32_t elected = elect_one();
+    const uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0);
+    const uint32_t idesc_o = idesc_bf16_f32(128, D, 0, 1);
+    const uint32_t q_addr = smem_u32(smem + SM::Q_OFF), kv_addr = smem_u32(smem + SM::KV_OFF);
+    uint32_t kt = 0, q_cnt[2] = {0, 0}, p_cnt[2] = {0, 0};
+    bool ok = true;
+    const uint64_t q_desc = smem_desc_sw128(q_addr, 16, 1024), k_desc = smem_desc_sw128(kv_addr, 16, 1024);
+    const uint64_t v_desc = smem_desc_sw128(kv_addr, SM::BLOCK_BYTES, 1024);
+    auto issue_qk = [&](int t, uint32_t st) {
+      mma_block_ss<QK_STEPS>(tmem + S_COL + t * 128, q_desc + ((t * SM::TILE_BYTES) >> 4),
+                             k_desc + ((st * SM::TILE_BYTES) >> 4), idesc_s, SM::BLOCK_BYTES >> 4, elected);
+    };
+    auto issue_pv_head = [&](int t, uint32_t st, bool accumulate) {
+      mma_block_ts<0, 2 * P_HEAD_CHUNKS>(tmem + O_COL + t * 128, tmem + S_COL + t * 128, v_desc + ((st * SM::TILE_BYTES) >> 4),
+                                         idesc_o, accumulate ? 1u : 0u, elected);
+    };
+    auto issue_pv_rest = [&](int t, uint32_t st) {
+      mma_block_ts<2 * P_HEAD_CHUNKS, 8>(tmem + O_COL + t * 128, tmem + S_COL + t * 128, v_desc + ((st * SM::TILE_BYTES) >> 4),
+                                         idesc_o, 1u, elected);
+    };
+    auto wait = [&](uint64_t* bar, uint32_t parity, int code) -> bool { return mbar_wait_warp(bar, parity, abortp, p.status, code); };
+    ItemCursor cur = {item_lo - 1, false, 0u};
+    while (ok && __all_sync(0xffffffffu, next_item(cur))) {
+      const int it = cur.it;
+      const WorkItem w = p.items[it];
+      const int nt = w.tile_end - w.tile_begin;
+      const int n_q = w.q_count[1] > 0 ? 2 : 1;
+      {
+        const uint32_t st = (2 * kt) % KV_SLOTS, ph = ((2 * kt) / KV_SLOTS) & 1;
+        if (!(ok = wait(&bar_kv_full[st], ph, 21))) break;
+        for (int t = 0; t < n_q && ok; ++t) {
+          if (!(ok = wait(&bar_q_full[t], q_cnt[t] & 1, 22))) break;
+          ++q_cnt[t];
+          tc_fence_after_sync();
+          issue_qk(t, st);
+          mma_commit(&bar_s_full[t], elected);
         }
-        for (int j = 0; j < nt && ok; ++j) {
-          const uint32_t gv = 2 * (kt + j) + 1, gk = gv + 1;  // ring positions of V_j and K_{j+1}
-          const uint32_t st = gv % KV_SLOTS, ph = (gv / KV_SLOTS) & 1;
-          const uint32_t st1 = gk % KV_SLOTS, ph1 = (gk / KV_SLOTS) & 1;
-          if (!(ok = mbar_wait(&bar_kv_full[st], ph, abortp, p.status, 23))) break;
-          for (int t = 0; t < n_q && ok; ++t) {
-            if (!(ok = mbar_wait(&bar_p_full[t], p_cnt[t] & 1, abortp, p.status, 24))) break;
-            ++p_cnt[t];
-            tc_fence_after_sync();
-            issue_pv(t, st, j > 0);
-            if (j + 1 < nt) {
-              if (t == 0 && !(ok = mbar_wait(&bar_kv_full[st1], ph1, abortp, p.status, 25))) break;
-              tc_fence_after_sync();
-              issue_qk(t, st1);
-              mma_commit(&bar_s_full[t]);
-              if (t == n_q - 1) mma_commit(&bar_kv_free[st1]);
-            } else {
-              mma_commit(&bar_o_full[t]);
-            }
-          }
-          if (!ok) break;
-          mma_commit(&bar_kv_free[st]);
-        }
-        kt += nt;
+        if (!ok) break;
+        mma_commit(&bar_kv_free[st], elected);
       }
+      for (int j = 0; j < nt && ok; ++j) {
+        const uint32_t gv = 2 * (kt + j) + 1, gk = gv + 1;  // ring positions of V_j and K_{j+1}
+        const uint32_t st = gv % KV_SLOTS, ph = (gv / KV_SLOTS) & 1;
+        const uint32_t st1 = gk % KV_SLOTS, ph1 = (gk / KV_SLOTS) & 1;
+        // both operands of this step are waited for ahead of P: the loads run a step ahead, P is what is waited for
+        if (!(ok = wait(&bar_kv_full[st], ph, 23))) break;
+        if (j + 1 < nt && !(ok = wait(&bar_kv_full[st1], ph1, 25))) break;
+        for (int t = 0; t < n_q && ok; ++t) {
+          if (!(ok = wait(&bar_p_head[t], p_cnt[t] & 1, 24))) break;
+          tc_fence_after_sync();
+          issue_pv_head(t, st, j > 0);
+          if (!(ok = wait(&bar_p_full[t], p_cnt[t] & 1, 26))) break;
+          ++p_cnt[t];
+          tc_fence_after_sync();
+          issue_pv_rest(t, st);
+          if (j + 1 < nt) {
+            issue_qk(t, st1);
+            mma_commit(&bar_s_full[t], elected);
+            if (t == n_q - 1) mma_commit(&bar_kv_free[st1], elected);
+          } else {
+            mma_commit(&bar_o_full[t], elected);
+          }
+        }
+        if (!ok) break;
+        mma_commit(&bar_kv_free[st], elected);
+      }
+      kt += nt;
+    }
     }
   } else {
     // ------------------------------------------------------------------ softmax + epilogue warps
-    // Eight warps per query tile.  A warp may only touch the 32 TMEM lanes (rows) of its warp-id quarter, and a
-    // lone warp cannot issue fast enough to keep up with the tensor pipe, so every row is shared by two threads
-    // of two warps on the same scheduler: each owns 64 of the tile's 128 keys (and half of the output columns)
-    // and they swap their row maxima through shared memory once per tile.
-    const int t = (warp - 2) >> 3;                  // query tile
-    const int half = ((warp - 2) >> 2) & 1;         // which 64 keys / which half of the output columns
+    // Four warps per query tile, one thread per query row (a warp may only touch the 32 TMEM lanes of its warp-id quarter).
+    // A thread fetches its row's 128 logits once and keeps them in registers.
+    regs_inc<REGS_SOFTMAX>();
+    const int t = (warp - 4) >> 2;                  // query tile
     const int r = ((warp & 3) << 5) | lane;         // row inside the tile == TMEM lane
     const uint32_t lane_off = static_cast<uint32_t>((warp & 3) << 5) << 16;
-    const uint32_t s_addr = tmem + lane_off + S_COL + t * 128 + half * 64;   // this thread's logits
-    const uint32_t p_addr = s_addr;  // its share of P (packed bf16) goes over the first 32 columns of its own logits
-    constexpr int OC = D / 2;                                                // output columns per thread
-    const uint32_t o_addr = tmem + lane_off + O_COL + t * 128 + half * OC;
+    const uint32_t s_addr = tmem + lane_off + S_COL + t * 128;  // this row's logits; P (packed bf16) goes over their first 64 columns
+    const uint32_t o_addr = tmem + lane_off + O_COL + t * 128;
     uint8_t* sq = smem + SM::Q_OFF + t * SM::TILE_BYTES;
-    uint32_t s_cnt = 0, o_cnt = 0, x_cnt = 0;
+    const int row0 = r & ~31;  // first row of this warp inside the tile
+    uint32_t s_cnt = 0, o_cnt = 0;
     bool ok = true;
-    // swaps one float with the other thread of the row (bounded wait like every other wait here)
-    auto swap_with_partner = [&](float mine, float& theirs) -> bool {
-      const int par = x_cnt & 1;
-      pair_val[t][par][half][r] = mine;
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bar_pair[t]);
-      if (!mbar_wait(&bar_pair[t], par, abortp, p.status, 34)) return false;
-      ++x_cnt;
-      theirs = pair_val[t][par][half ^ 1][r];
-      return true;
-    };
     ItemCursor cur = {item_lo - 1, false, 0u};
     while (ok && next_item(cur)) {
       const int it = cur.it;
       const WorkItem w = p.items[it];
       if (w.q_count[t] == 0) continue;
-      if (p.trace && t == 0 && r == 0 && half == 0) p.trace[2 * it] = global_timer_ns();
+      if (p.trace && t == 0 && r == 0) p.trace[2 * it] = global_timer_ns();
       const bool row_valid = r < w.q_count[t];
       int token = 0;
       if (row_valid) {
         token = w.q_start[t] + r;
         if (w.cell >= 0) token = cell_query_token(p.cells[w.cell], token, p.tokens_per_frame, p.grid_w);
       }
-      // ---- stage this warp's 32 query rows (its half of the columns) into shared memory (swizzled); invalid rows are
-      // zero.  The lanes share the rows: CH consecutive lanes fetch the CH 16-byte chunks of one row, so a load
-      // instruction touches 32 / CH rows (4 lines of 128 bytes at d = 128) instead of 32 - with one row per lane the
-      // 16 warps needed 4096 line visits per item and the load/store unit, not the latency, set the time (2.5 us).
+      // ---- stage this warp's 32 query rows into shared memory (swizzled); invalid rows are zero.  The lanes share the
+      // rows: CH consecutive lanes fetch the CH 16-byte chunks of one row, so a load instruction touches 32 / CH rows
+      // instead of 32.
       {
-        constexpr int CH = D / 16;  // 16-byte chunks of a half row
+        constexpr int CH = D / 8;  // 16-byte chunks of a row
         uint4 v[CH];
 #pragma unroll
         for (int k = 0; k < CH; ++k) {
-          const int idx = k * 32 + lane, row = idx / CH, c = half * CH + idx % CH;
+          const int idx = k * 32 + lane, row = idx / CH, c = idx % CH;
           const int tok = __shfl_sync(0xffffffffu, token, row);
           const bool valid = __shfl_sync(0xffffffffu, row_valid ? 1 : 0, row) != 0;
           v[k] = make_uint4(0, 0, 0, 0);
@@ -391,13 +398,13 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
         }
 #pragma unroll
         for (int k = 0; k < CH; ++k) {
-          const int idx = k * 32 + lane, row = idx / CH, c = half * CH + idx % CH;
-          *reinterpret_cast<uint4*>(sq + (c / 8) * SM::BLOCK_BYTES + sw128_offset((r & ~31) + row, c % 8)) = v[k];
+          const int idx = k * 32 + lane, row = idx / CH, c = idx % CH;
+          *reinterpret_cast<uint4*>(sq + (c / 8) * SM::BLOCK_BYTES + sw128_offset(row0 + row, c % 8)) = v[k];
         }
         fence_proxy_async_smem();
         tc_fence_before_sync();  // orders this thread's TMEM reads of the previous item before the arrive
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bar_q_full[t]);
+        mbar_arrive_if(&bar_q_full[t], lane == 0);
       }
       int qy = 0, qx = 0;
       if (PROXY) {
@@ -405,45 +412,51 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
         qy = pos / p.grid_w;
         qx = pos - qy * p.grid_w;
       }
-      float m_ref = -INFINITY, l_sum = 0.f, l_mid = 0.f;  // l_* cover this thread's 64 keys per tile only
+      float m_ref = -INFINITY, l_sum = 0.f, l_mid = 0.f;
       const int nt = w.tile_end - w.tile_begin;
       for (int j = 0; j < nt; ++j) {
         const int tile = w.tile_begin + j;
-        const int seg = tile / w.tiles_per_seg, c = tile - seg * w.tiles_per_seg;
-        const int n_valid = min(128, w.seg_len - c * 128) - half * 64;  // valid keys among this thread's 64
-        const int tok0 = PROXY ? (w.kv_row0 + c * 128 + half * 64) : 0;  // in-frame token of its first key
+        const int seg = PROXY ? tile / w.tiles_per_seg : 0, c = PROXY ? tile - seg * w.tiles_per_seg : tile;
+        const int n_valid = min(128, w.seg_len - c * 128);  // keys of this tile that exist
+        // Keys this row must not see count as -inf: the ragged tail of a segment, and for the Spatial proxy every key
+        // outside the (2r+1)^2 neighbourhood.
+        uint32_t visible[4] = {0u, 0u, 0u, 0u};
+        if (PROXY) {
+          const int tok0 = w.kv_row0 + c * 128;  // in-frame token of the tile's first key
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch)
+            visible[ch] = visible_keys<PROXY>(n_valid - ch * 32, tok0 + ch * 32, qy, qx, p.radius, p.grid_w);
+        }
         if (!(ok = mbar_wait(&bar_s_full[t], s_cnt & 1, abortp, p.status, 31))) break;
         ++s_cnt;
         tc_fence_after_sync();
-        // pass 1: maximum of this thread's 64 logits (32 columns at a time; they are read again in pass 2, which
-        // keeps the live registers low enough for 576 threads per CTA).  Keys this row must not see count as -inf:
-        // the ragged tail of a segment, and for the Spatial proxy every key outside the (2r+1)^2 neighbourhood.
+        uint32_t sv[4][32];
         float mx;
         {
           float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-          for (int ch = 0; ch < 2; ++ch) {
-            const uint32_t visible = PROXY ? visible_keys<PROXY>(n_valid - ch * 32, tok0 + ch * 32, qy, qx, p.radius, p.grid_w) : 0u;
-            if (PROXY && __all_sync(0xffffffffu, visible == 0u)) continue;  // no row of this warp sees any of these keys
-            uint32_t sv[32];
-            tmem_ld32(s_addr + ch * 32, sv);
-            tmem_wait_ld();
-            apply_visible<PROXY>(sv, visible, n_valid - ch * 32);
+          for (int ch = 0; ch < 4; ++ch) tmem_ld32(s_addr + ch * 32, sv[ch]);
+          tmem_wait_ld(sv[0], sv[1], sv[2], sv[3]);
+          // one branch for the whole tile (only the last tile of a range has hidden keys): with one per chunk the maximum
+          // and the exponentials could not be scheduled across the chunks (dense sweep 4828 -> 4620 us)
+          if (PROXY || n_valid < 128) {
+#pragma unroll
+            for (int ch = 0; ch < 4; ++ch) apply_visible<PROXY>(sv[ch], visible[ch], n_valid - ch * 32);
+          }
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch) {
 #pragma unroll
             for (int i = 0; i < 32; i += 8) {
-              mx4[0] = max3(mx4[0], __uint_as_float(sv[i]), __uint_as_float(sv[i + 1]));
-              mx4[1] = max3(mx4[1], __uint_as_float(sv[i + 2]), __uint_as_float(sv[i + 3]));
-              mx4[2] = max3(mx4[2], __uint_as_float(sv[i + 4]), __uint_as_float(sv[i + 5]));
-              mx4[3] = max3(mx4[3], __uint_as_float(sv[i + 6]), __uint_as_float(sv[i + 7]));
+              mx4[0] = max3(mx4[0], __uint_as_float(sv[ch][i]), __uint_as_float(sv[ch][i + 1]));
+              mx4[1] = max3(mx4[1], __uint_as_float(sv[ch][i + 2]), __uint_as_float(sv[ch][i + 3]));
+              mx4[2] = max3(mx4[2], __uint_as_float(sv[ch][i + 4]), __uint_as_float(sv[ch][i + 5]));
+              mx4[3] = max3(mx4[3], __uint_as_float(sv[ch][i + 6]), __uint_as_float(sv[ch][i + 7]));
             }
           }
           mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
         }
-        float mx_other;
-        if (!(ok = swap_with_partner(mx, mx_other))) break;
-        mx = fmaxf(mx, mx_other) * p.scale_log2e;  // row maximum; scale > 0, so the maximum commutes with it
-        // running maximum: move the reference only when some row of the warp outgrew it by 2^8.  Both threads of
-        // a row see the same maximum and sit in the same lane of their warps, so both warps decide alike.
+        mx *= p.scale_log2e;  // row maximum; scale > 0, so the maximum commutes with it
+        // running maximum: move the reference only when some row of the warp outgrew it by 2^8
         const bool grow = mx > m_ref + RESCALE_THRESHOLD || (m_ref == -INFINITY && mx > -INFINITY);
         if (__any_sync(0xffffffffu, grow)) {
           const float m_new = fmaxf(m_ref, mx);
@@ -451,45 +464,34 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
           l_sum *= alpha;
           l_mid *= alpha;
           m_ref = m_new;
-          if (j > 0) {  // O_t holds the products of the earlier tiles: bring this thread's columns to the new reference
+          if (j > 0) {  // O_t holds the products of the earlier tiles: bring this row to the new reference
 #pragma unroll 1
-            for (int ch = 0; ch < OC / 32; ++ch) {
-              uint32_t v[32];
-              tmem_ld32(o_addr + ch * 32, v);
-              tmem_wait_ld();
+            for (int ch = 0; ch < D / 16; ++ch) {
+              uint32_t v[16];
+              tmem_ld16(o_addr + ch * 16, v);
+              tmem_wait_ld(v);
 #pragma unroll
-              for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
-              tmem_st32(o_addr + ch * 32, v);
+              for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
+              tmem_st16(o_addr + ch * 16, v);
             }
           }
         }
         const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
-        // pass 2: p = 2^(s * c - m), bf16 pack over the first 32 columns of this thread's logits, row sum in fp32
+        // p = 2^(s * c - m), packed to bf16 over the first 64 columns of the logits, row sum in fp32.  The first
+        // P_HEAD_CHUNKS chunks are handed over on their own: their share of the O product runs while the rest is computed.
         const uint64_t c2 = pack_f32x2(p.scale_log2e, p.scale_log2e), m2 = pack_f32x2(-m_use, -m_use);
         float sum4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int ch = 0; ch < 2; ++ch) {
-          const uint32_t visible = PROXY ? visible_keys<PROXY>(n_valid - ch * 32, tok0 + ch * 32, qy, qx, p.radius, p.grid_w) : 0u;
+        for (int ch = 0; ch < 4; ++ch) {
           uint32_t pk[16];
-          if (PROXY && __all_sync(0xffffffffu, visible == 0u)) {
-            // nothing to exponentiate: P = 0 for these keys (the product still reads them)
-#pragma unroll
-            for (int i = 0; i < 16; ++i) pk[i] = 0u;
-            tmem_st16(p_addr + ch * 16, pk);
-            continue;
-          }
-          uint32_t sv[32];
-          tmem_ld32(s_addr + ch * 32, sv);
-          tmem_wait_ld();
-          apply_visible<PROXY>(sv, visible, n_valid - ch * 32);
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
-            const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1])), c2, m2);
+            const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(sv[ch][2 * i]), __uint_as_float(sv[ch][2 * i + 1])), c2, m2);
             float x0, x1, e0, e1;
             unpack_f32x2(x2, x0, x1);
             if ((i & HC_POLY_MASK) == HC_POLY_MASK) {
-              // every fourth pair takes the polynomial route on the FMA pipe: the special-function unit alone
-              // cannot produce 128 x 128 exponentials in the time the tensor pipe needs for the tile
+              // every eighth pair takes the polynomial route on the FMA pipe: two tiles' exponentials keep the
+              // special-function unit busy for 2048 clk, as long as the tensor pipe needs for the two tiles' products
               ex2_poly_pair(pack_f32x2(fmaxf(x0, -126.f), fmaxf(x1, -126.f)), e0, e1);
             } else {
               e0 = ex2_approx(x0);
@@ -500,125 +502,90 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
             // the values even when the reference lags behind the row maximum and the largest p is not exactly 1
             add_bf16x2_to_f32(pk[i], sum4[(i & 1) * 2], sum4[(i & 1) * 2 + 1]);
           }
-          tmem_st16(p_addr + ch * 16, pk);
+          if (ch == P_HEAD_CHUNKS) {
+            // the head of P goes out here and not right behind its stores: by now they are done and nothing waits
+            tmem_wait_st();
+            tc_fence_before_sync();
+            __syncwarp();
+            mbar_arrive_if(&bar_p_head[t], lane == 0);
+          }
+          tmem_st16(s_addr + ch * 16, pk);
         }
+        tmem_wait_st();
+        tc_fence_before_sync();
+        __syncwarp();
+        mbar_arrive_if(&bar_p_full[t], lane == 0);
         const float tile_sum = (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
         l_sum += tile_sum;
         if (PROXY && seg >= p.mid_seg_lo && seg < p.mid_seg_hi && !(seg >= p.last_seg_lo && seg < p.last_seg_hi))
           l_mid += tile_sum;
-        tmem_wait_st();
-        tc_fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bar_p_full[t]);
       }
       if (!ok) break;
-      // ---- epilogue: row sums of the two halves are added, each thread normalises and stores its output columns
-      float other;
-      if (!(ok = swap_with_partner(l_sum, other))) break;
-      l_sum += other;
-      if (PROXY) {
-        if (!(ok = swap_with_partner(l_mid, other))) break;
-        l_mid += other;
-      }
+      // ---- epilogue: normalise and store this row
       if (!(ok = mbar_wait(&bar_o_full[t], o_cnt & 1, abortp, p.status, 32))) break;
       ++o_cnt;
       tc_fence_after_sync();
       const float inv = (l_sum > 0.f) ? 1.f / l_sum : 0.f;
-      const float mult = (w.out_mode == OUT_PARTIAL) ? 1.f : inv;
-      if constexpr (D == 128) {
-        // The thread holds its row's OC output columns, but one row per lane is the worst pattern for global stores
-        // (32 lines per instruction: 4096 line visits per tile, 4-5 us per item).  So the warp turns its 32 x OC block
-        // through shared memory - its 4 KB of this tile's query buffer, which the last S product has finished reading
-        // (the O product committed to bar_o_full was issued after it) - and stores whole 128-byte lines: 8 lanes a row.
-        uint8_t* stg = sq + (half * 4 + (warp & 3)) * 4096;
-        const int row0 = r & ~31;  // first row of this warp inside the tile
-        if (w.out_mode == OUT_BF16) {
-          constexpr int U = OC / 8;  // 16-byte units of a row's half: 8 (d = 128) or 4 (d = 64)
-  #pragma unroll 1
-          for (int ch = 0; ch < OC / 32; ++ch) {
-            uint32_t v[32];
-            tmem_ld32(o_addr + ch * 32, v);
-            tmem_wait_ld();
-  #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              uint4 o4;
-              o4.x = pack_bf16x2(__uint_as_float(v[8 * i + 0]) * mult, __uint_as_float(v[8 * i + 1]) * mult);
-              o4.y = pack_bf16x2(__uint_as_float(v[8 * i + 2]) * mult, __uint_as_float(v[8 * i + 3]) * mult);
-              o4.z = pack_bf16x2(__uint_as_float(v[8 * i + 4]) * mult, __uint_as_float(v[8 * i + 5]) * mult);
-              o4.w = pack_bf16x2(__uint_as_float(v[8 * i + 6]) * mult, __uint_as_float(v[8 * i + 7]) * mult);
-              *reinterpret_cast<uint4*>(stg + lane * 128 + (((ch * 4 + i) ^ (lane & 7)) << 4)) = o4;
-            }
-          }
-          __syncwarp();
-  #pragma unroll
-          for (int k = 0; k < U; ++k) {
-            const int idx = k * 32 + lane, row = idx / U, u = idx % U;
-            const uint4 val = *reinterpret_cast<const uint4*>(stg + row * 128 + ((u ^ (row & 7)) << 4));
-            const int tok = __shfl_sync(0xffffffffu, token, row);
-            const bool valid = __shfl_sync(0xffffffffu, row_valid ? 1 : 0, row) != 0;
-            if (valid)
-              *reinterpret_cast<uint4*>(p.out + (static_cast<size_t>(tok) * p.n_heads + w.head) * D + half * OC + u * 8) = val;
-          }
-          __syncwarp();
-        } else {
-          float* base = p.part_o + (static_cast<size_t>(w.out_slot) * 256 + t * 128 + row0) * D + half * OC;
-  #pragma unroll 1
-          for (int ch = 0; ch < OC / 32; ++ch) {
-            uint32_t v[32];
-            tmem_ld32(o_addr + ch * 32, v);
-            tmem_wait_ld();
-  #pragma unroll
-            for (int i = 0; i < 8; ++i)
-              *reinterpret_cast<float4*>(stg + lane * 128 + ((i ^ (lane & 7)) << 4)) =
-                  make_float4(__uint_as_float(v[4 * i + 0]) * mult, __uint_as_float(v[4 * i + 1]) * mult,
-                              __uint_as_float(v[4 * i + 2]) * mult, __uint_as_float(v[4 * i + 3]) * mult);
-            __syncwarp();
-  #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const int idx = k * 32 + lane, row = idx >> 3, u = idx & 7;
-              const float4 val = *reinterpret_cast<const float4*>(stg + row * 128 + ((u ^ (row & 7)) << 4));
-              const bool valid = __shfl_sync(0xffffffffu, row_valid ? 1 : 0, row) != 0;
-              if (valid) *reinterpret_cast<float4*>(base + static_cast<size_t>(row) * D + ch * 32 + u * 4) = val;
-            }
-            __syncwarp();
-          }
-        }
-      } else
-      {
-        // head_dim 64: a tile's query buffer (16 KB) is too small to turn the fp32 block through; one row per lane
-        const size_t row_elem = (static_cast<size_t>(token) * p.n_heads + w.head) * D + half * OC;
+      // The thread holds its row's output, but one row per lane is the worst pattern for global stores (32 lines per
+      // instruction).  So the warp turns its rows through shared memory - its own 32 rows of this tile's query buffer,
+      // which the last S product has finished reading (the O product committed to bar_o_full was issued after it) - and
+      // stores whole 128-byte lines.
+      uint8_t* stg = sq + row0 * 128;
+      if (w.out_mode == OUT_BF16) {
 #pragma unroll 1
-        for (int ch = 0; ch < OC / 32; ++ch) {
+        for (int ch = 0; ch < D / 32; ++ch) {
           uint32_t v[32];
           tmem_ld32(o_addr + ch * 32, v);
-          tmem_wait_ld();
-          if (!row_valid) continue;
-          if (w.out_mode == OUT_BF16) {
-            uint4* dst = reinterpret_cast<uint4*>(p.out + row_elem + ch * 32);
+          tmem_wait_ld(v);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              uint4 o4;
-              o4.x = pack_bf16x2(__uint_as_float(v[8 * i + 0]) * mult, __uint_as_float(v[8 * i + 1]) * mult);
-              o4.y = pack_bf16x2(__uint_as_float(v[8 * i + 2]) * mult, __uint_as_float(v[8 * i + 3]) * mult);
-              o4.z = pack_bf16x2(__uint_as_float(v[8 * i + 4]) * mult, __uint_as_float(v[8 * i + 5]) * mult);
-              o4.w = pack_bf16x2(__uint_as_float(v[8 * i + 6]) * mult, __uint_as_float(v[8 * i + 7]) * mult);
-              dst[i] = o4;
-            }
-          } else {
-            float* base = p.part_o + (static_cast<size_t>(w.out_slot) * 256 + t * 128 + r) * D + half * OC;
-            float4* dst = reinterpret_cast<float4*>(base + ch * 32);
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-              dst[i] = make_float4(__uint_as_float(v[4 * i + 0]) * mult, __uint_as_float(v[4 * i + 1]) * mult,
-                                   __uint_as_float(v[4 * i + 2]) * mult, __uint_as_float(v[4 * i + 3]) * mult);
+          for (int i = 0; i < 4; ++i) {
+            uint4 o4;
+            o4.x = pack_bf16x2(__uint_as_float(v[8 * i + 0]) * inv, __uint_as_float(v[8 * i + 1]) * inv);
+            o4.y = pack_bf16x2(__uint_as_float(v[8 * i + 2]) * inv, __uint_as_float(v[8 * i + 3]) * inv);
+            o4.z = pack_bf16x2(__uint_as_float(v[8 * i + 4]) * inv, __uint_as_float(v[8 * i + 5]) * inv);
+            o4.w = pack_bf16x2(__uint_as_float(v[8 * i + 6]) * inv, __uint_as_float(v[8 * i + 7]) * inv);
+            *reinterpret_cast<uint4*>(stg + (ch >> 1) * SM::BLOCK_BYTES + lane * 128 + ((((ch & 1) * 4 + i) ^ (lane & 7)) << 4)) = o4;
           }
         }
+        __syncwarp();
+        constexpr int U = D / 8;  // 16-byte units of a row
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+          const int idx = k * 32 + lane, row = idx / U, u = idx % U;
+          const uint4 val = *reinterpret_cast<const uint4*>(stg + (u / 8) * SM::BLOCK_BYTES + row * 128 + (((u % 8) ^ (row & 7)) << 4));
+          const int tok = __shfl_sync(0xffffffffu, token, row);
+          const bool valid = __shfl_sync(0xffffffffu, row_valid ? 1 : 0, row) != 0;
+          if (valid) *reinterpret_cast<uint4*>(p.out + (static_cast<size_t>(tok) * p.n_heads + w.head) * D + u * 8) = val;
+        }
+        __syncwarp();
+      } else {
+        float* base = p.part_o + (static_cast<size_t>(w.out_slot) * 256 + t * 128 + row0) * D;
+#pragma unroll 1
+        for (int ch = 0; ch < D / 32; ++ch) {
+          uint32_t v[32];
+          tmem_ld32(o_addr + ch * 32, v);
+          tmem_wait_ld(v);
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            *reinterpret_cast<float4*>(stg + lane * 128 + ((i ^ (lane & 7)) << 4)) =
+                make_float4(__uint_as_float(v[4 * i + 0]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]),
+                            __uint_as_float(v[4 * i + 3]));
+          __syncwarp();
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const int idx = k * 32 + lane, row = idx >> 3, u = idx & 7;
+            const float4 val = *reinterpret_cast<const float4*>(stg + row * 128 + ((u ^ (row & 7)) << 4));
+            const bool valid = __shfl_sync(0xffffffffu, row_valid ? 1 : 0, row) != 0;
+            if (valid) *reinterpret_cast<float4*>(base + static_cast<size_t>(row) * D + ch * 32 + u * 4) = val;
+          }
+          __syncwarp();
+        }
+        if (row_valid) {
+          p.part_ml[static_cast<size_t>(w.out_slot) * 256 + t * 128 + r] = make_float2(m_ref, l_sum);
+          if (PROXY) p.part_mid[static_cast<size_t>(w.out_slot) * 256 + t * 128 + r] = l_mid;
+        }
       }
-      if (row_valid && half == 0 && w.out_mode == OUT_PARTIAL) {
-        p.part_ml[static_cast<size_t>(w.out_slot) * 256 + t * 128 + r] = make_float2(m_ref, l_sum);
-        if (PROXY) p.part_mid[static_cast<size_t>(w.out_slot) * 256 + t * 128 + r] = l_mid;
-      }
-      if (p.trace && t == 0 && r == 0 && half == 0) p.trace[2 * it + 1] = global_timer_ns();
+      if (p.trace && t == 0 && r == 0) p.trace[2 * it + 1] = global_timer_ns();
     }
   }
   // ------------------------------------------------------------------ teardown

@@ -24,6 +24,11 @@ __device__ __forceinline__ void fence_mbar_init() {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// The same from one lane of a converged warp, without a branch: every lane calls it, the lane with `pred` not zero arrives.
+__device__ __forceinline__ void mbar_arrive_if(uint64_t* bar, uint32_t pred) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t@q mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(smem_u32(bar)), "r"(pred)
+               : "memory");
+}
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                : "memory");
@@ -73,6 +78,35 @@ __device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, 
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
                                           int code) {
   return mbar_wait_limit(bar, parity, abort_flag, status, code, HC_WAIT_LIMIT_NS);
+}
+
+// The wait of a converged warp: one vote per poll, so the warp stays converged and every lane gets the same answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status, int code) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  uint64_t t0 = 0;
+  for (uint32_t spin = 1;; ++spin) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if ((spin & 63u) == 0) {
+      const uint64_t now = global_timer_ns();
+      if (t0 == 0) t0 = now;
+      if (__any_sync(0xffffffffu, now - t0 > HC_WAIT_LIMIT_NS)) {
+        *abort_flag = 1;
+        atomicCAS(status, 0, code);
+        return false;
+      }
+      if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+    }
+  }
+}
+
+// Hands registers of this warpgroup back to the block's pool (dec) or takes them from it (inc); all four warps execute it.
+template <int N>
+__device__ __forceinline__ void regs_dec() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void regs_inc() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
 }
 
 // generic-proxy writes to shared memory -> visible to the async proxy (TMA, tcgen05.mma operands)
@@ -163,110 +197,71 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(uint32_t m, uint32_t n, ui
          ((m >> 4) << 24);
 }
 
-// Issue blocks.  A tcgen05.mma needs at least ~64 clocks of the tensor pipe whatever its N, and any integer
-// work between two of them (descriptor arithmetic in the issuing thread) costs about as much again.  So the
-// k-steps of one product are issued from ONE asm block whose only other instructions are 64-bit adds on the
-// descriptors' start-address field.
-//
-// S[tmem] = A[smem, K-major] * B[smem, K-major]^T over KSTEPS k-steps of 16; both operands are stored as
-// 64-column blocks of [rows][128 bytes] (128-byte swizzle): k-step kk starts (kk % 4) * 32 bytes into block
-// kk / 4.  a_block16 / b_block16 are the block sizes in units of 16 bytes.
-template <int KSTEPS>
-__device__ __forceinline__ void mma_block_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                             uint32_t a_block16, uint32_t b_block16) {
-  static_assert(KSTEPS == 4 || KSTEPS == 8, "head_dim 64 or 128");
-  if (KSTEPS == 4) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
-        "setp.ne.b32 p, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
-        "setp.eq.b32 p, 0, 0;\n\t"
-        "add.u64 a, %1, 2;\n\tadd.u64 b, %2, 2;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t"
-        "add.u64 a, %1, 4;\n\tadd.u64 b, %2, 4;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t"
-        "add.u64 a, %1, 6;\n\tadd.u64 b, %2, 6;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc)
-        : "memory");
-  } else {
-    const uint64_t a1 = a_desc + a_block16, b1 = b_desc + b_block16;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
-        "setp.ne.b32 p, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
-        "setp.eq.b32 p, 0, 0;\n\t"
-        "add.u64 a, %1, 2;\n\tadd.u64 b, %2, 2;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t"
-        "add.u64 a, %1, 4;\n\tadd.u64 b, %2, 4;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t"
-        "add.u64 a, %1, 6;\n\tadd.u64 b, %2, 6;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %4, %5, %3, p;\n\t"
-        "add.u64 a, %4, 2;\n\tadd.u64 b, %5, 2;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t"
-        "add.u64 a, %4, 4;\n\tadd.u64 b, %5, 4;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t"
-        "add.u64 a, %4, 6;\n\tadd.u64 b, %5, 6;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "l"(a1), "l"(b1)
-        : "memory");
-  }
+// Issue blocks.  The products of a whole tile are issued by a CONVERGED warp: every lane walks the same loop and computes
+// the same descriptors, and only the tcgen05.mma itself is predicated on the lane that elect.sync chose.  The
+// descriptors then are warp-uniform values, and the warp keeps up with the tensor pipe whatever else its scheduler runs.
+// Issued from inside an `if (lane == 0)` branch a block of 16 instructions took 1277 clk alone and 1818 clk beside four
+// warps of softmax-like work on that scheduler; this form takes 1024 clk (64 each, the pipe's own rate) in both cases.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+  return e;
 }
 
-// O[tmem] (+)= P[tmem, packed bf16, 8 columns per k-step] * V[smem, MN-major] over 8 k-steps of 16 keys;
-// consecutive k-steps of V are 2048 bytes (128 sixteen-byte units) apart.  P is stored in two pieces: keys 0..63
-// in columns a .. a+31, keys 64..127 in columns a+64 .. a+95 (each piece over the logits it was computed from).
-// `accumulate` applies to the first k-step.
-__device__ __forceinline__ void mma_block_ts8(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                              uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\t.reg .b32 a;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t"
-      "setp.eq.b32 p, 0, 0;\n\t"
-      "add.u32 a, %1, 8;\n\tadd.u64 b, %2, 128;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, p;\n\t"
-      "add.u32 a, %1, 16;\n\tadd.u64 b, %2, 256;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, p;\n\t"
-      "add.u32 a, %1, 24;\n\tadd.u64 b, %2, 384;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, p;\n\t"
-      "add.u32 a, %1, 64;\n\tadd.u64 b, %2, 512;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, p;\n\t"
-      "add.u32 a, %1, 72;\n\tadd.u64 b, %2, 640;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, p;\n\t"
-      "add.u32 a, %1, 80;\n\tadd.u64 b, %2, 768;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, p;\n\t"
-      "add.u32 a, %1, 88;\n\tadd.u64 b, %2, 896;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// D[tmem] (+)= A[smem] * B[smem]
+// D[tmem] (+)= A[smem] * B[smem], issued by the lane whose `elected` is not zero; the warp must be converged
 __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
+                                       uint32_t accumulate, uint32_t elected) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(elected)
       : "memory");
 }
 // D[tmem] (+)= A[tmem] * B[smem]
 __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
+                                       uint32_t accumulate, uint32_t elected) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(elected)
       : "memory");
 }
-// The mbarrier receives one arrival once every tcgen05.mma issued so far by this thread has completed.
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
+
+// S[tmem] = A[smem, K-major] * B[smem, K-major]^T over KSTEPS k-steps of 16; both operands are stored as
+// 64-column blocks of [rows][128 bytes] (128-byte swizzle): k-step kk starts (kk % 4) * 32 bytes into block
+// kk / 4.  block16 is the block size in units of 16 bytes.
+template <int KSTEPS>
+__device__ __forceinline__ void mma_block_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                             uint32_t block16, uint32_t elected) {
+#pragma unroll
+  for (int k = 0; k < KSTEPS; ++k) {
+    const uint32_t off = (k / 4) * block16 + (k % 4) * 2;
+    mma_ss(d_tmem, a_desc + off, b_desc + off, idesc, k > 0 ? 1u : 0u, elected);
+  }
+}
+
+// O[tmem] (+)= P[tmem, packed bf16, 8 columns per k-step] * V[smem, MN-major] over the k-steps [K0, K1) of 16 keys;
+// consecutive k-steps of V are 2048 bytes (128 sixteen-byte units) apart.  `accumulate` applies to k-step 0.
+template <int K0, int K1>
+__device__ __forceinline__ void mma_block_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                             uint32_t accumulate, uint32_t elected) {
+#pragma unroll
+  for (int k = K0; k < K1; ++k)
+    mma_ts(d_tmem, a_tmem + k * 8, b_desc + k * 128, idesc, k > 0 ? 1u : accumulate, elected);
+}
+
+// The mbarrier receives one arrival once every tcgen05.mma issued so far by the elected lane has completed.
+__device__ __forceinline__ void mma_commit(uint64_t* bar, uint32_t elected) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+      ::"r"(smem_u32(bar)), "r"(elected)
+      : "memory");
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -284,14 +279,11 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
       : "r"(taddr)
       : "memory");
 }
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-      "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]),
-      "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]),
-      "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
       : "memory");
 }
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
@@ -302,7 +294,24 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
       "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Waits for this thread's tensor-memory loads; the registers of the waited-for loads are operands, so that no use of them
+// can be scheduled ahead of the wait.
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&a)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]), "+r"(a[8]), "+r"(a[9]), "+r"(a[10]), "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15])
+               :: "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&a)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]), "+r"(a[8]), "+r"(a[9]), "+r"(a[10]), "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15]), "+r"(a[16]), "+r"(a[17]), "+r"(a[18]), "+r"(a[19]), "+r"(a[20]), "+r"(a[21]), "+r"(a[22]), "+r"(a[23]), "+r"(a[24]), "+r"(a[25]), "+r"(a[26]), "+r"(a[27]), "+r"(a[28]), "+r"(a[29]), "+r"(a[30]), "+r"(a[31])
+               :: "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&a)[32], uint32_t (&b)[32], uint32_t (&c)[32], uint32_t (&d)[32]) {
+  tmem_wait_ld(a);
+  asm volatile("" : "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7]), "+r"(b[8]), "+r"(b[9]), "+r"(b[10]), "+r"(b[11]), "+r"(b[12]), "+r"(b[13]), "+r"(b[14]), "+r"(b[15]), "+r"(b[16]), "+r"(b[17]), "+r"(b[18]), "+r"(b[19]), "+r"(b[20]), "+r"(b[21]), "+r"(b[22]), "+r"(b[23]), "+r"(b[24]), "+r"(b[25]), "+r"(b[26]), "+r"(b[27]), "+r"(b[28]), "+r"(b[29]), "+r"(b[30]), "+r"(b[31]));
+  asm volatile("" : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(c[4]), "+r"(c[5]), "+r"(c[6]), "+r"(c[7]), "+r"(c[8]), "+r"(c[9]), "+r"(c[10]), "+r"(c[11]), "+r"(c[12]), "+r"(c[13]), "+r"(c[14]), "+r"(c[15]), "+r"(c[16]), "+r"(c[17]), "+r"(c[18]), "+r"(c[19]), "+r"(c[20]), "+r"(c[21]), "+r"(c[22]), "+r"(c[23]), "+r"(c[24]), "+r"(c[25]), "+r"(c[26]), "+r"(c[27]), "+r"(c[28]), "+r"(c[29]), "+r"(c[30]), "+r"(c[31]));
+  asm volatile("" : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]), "+r"(d[4]), "+r"(d[5]), "+r"(d[6]), "+r"(d[7]), "+r"(d[8]), "+r"(d[9]), "+r"(d[10]), "+r"(d[11]), "+r"(d[12]), "+r"(d[13]), "+r"(d[14]), "+r"(d[15]), "+r"(d[16]), "+r"(d[17]), "+r"(d[18]), "+r"(d[19]), "+r"(d[20]), "+r"(d[21]), "+r"(d[22]), "+r"(d[23]), "+r"(d[24]), "+r"(d[25]), "+r"(d[26]), "+r"(d[27]), "+r"(d[28]), "+r"(d[29]), "+r"(d[30]), "+r"(d[31]));
+}
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------------------------

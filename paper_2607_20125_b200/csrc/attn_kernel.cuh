@@ -182,15 +182,21 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
       mbar_init(&bar_kv_free[s], 1);
     }
     for (int s = 0; s < 4; ++s) mbar_init(&bar_dyn[s], 1);
-    // A context whose earlier kernel gave up on a wait keeps its status word set until the host has read it; the
-    // shared queue's counters may then be half drawn, so until then a launch does nothing at all (every thread sees
-    // the same answer: one thread reads the word, the others read its copy after the barrier below)
-    abort_flag = (*reinterpret_cast<volatile int32_t*>(p.status) != 0) ? 1 : 0;
     fence_mbar_init();
   }
   if (warp == 1) {
     tmem_alloc(&tmem_slot, TMEM_COLS);
     tmem_relinquish();
+  }
+  // The barriers and the tensor memory are set up while the kernel before drains; nothing in global memory has been
+  // touched so far.
+  pdl_launch_dependents();
+  pdl_wait();
+  if (tid == 0) {
+    // A context whose earlier kernel gave up on a wait keeps its status word set until the host has read it; the
+    // shared queue's counters may then be half drawn, so until then a launch does nothing at all (every thread sees
+    // the same answer: one thread reads the word, the others read its copy after the barrier below)
+    abort_flag = (*reinterpret_cast<volatile int32_t*>(p.status) != 0) ? 1 : 0;
   }
   tc_fence_before_sync();
   __syncthreads();
@@ -374,12 +380,12 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
     while (ok && next_item(cur)) {
       const int it = cur.it;
       const WorkItem w = p.items[it];
-      if (w.q_count[t] == 0) continue;
+      if ((t ? w.q_count[1] : w.q_count[0]) == 0) continue;
       if (p.trace && t == 0 && r == 0) p.trace[2 * it] = global_timer_ns();
-      const bool row_valid = r < w.q_count[t];
+      const bool row_valid = r < (t ? w.q_count[1] : w.q_count[0]);
       int token = 0;
       if (row_valid) {
-        token = w.q_start[t] + r;
+        token = (t ? w.q_start[1] : w.q_start[0]) + r;
         if (w.cell >= 0) token = cell_query_token(p.cells[w.cell], token, p.tokens_per_frame, p.grid_w);
       }
       // ---- stage this warp's 32 query rows into shared memory (swizzled); invalid rows are zero.  The lanes share the
@@ -617,12 +623,10 @@ __device__ __forceinline__ float4 ld_stream_f4(const float4* p) {
 }
 
 template <int D>
-__global__ void __launch_bounds__(COMBINE_ROWS * (D / 8))
-combine_kernel(const CombineEntry* entries, const CellGeom* cells, const float* part_o, const float2* part_ml,
-               __nv_bfloat16* out, int n_heads, int tokens_per_frame, int grid_w) {
+__device__ __forceinline__ void combine_rows(const CombineEntry& e, int block, const CellGeom* cells, const float* part_o, const float2* part_ml,
+                                             __nv_bfloat16* out, int n_heads, int tokens_per_frame, int grid_w) {
   constexpr int CHUNKS = D / 8;
-  const CombineEntry e = entries[blockIdx.x / (128 / COMBINE_ROWS)];
-  const int r = (blockIdx.x % (128 / COMBINE_ROWS)) * COMBINE_ROWS + threadIdx.x / CHUNKS;
+  const int r = block * COMBINE_ROWS + threadIdx.x / CHUNKS;
   const int c = threadIdx.x % CHUNKS;
   if (r >= e.q_count) return;
   // Rows of successive parts lie 256 rows apart.  The parts are taken four at a time with all loads of a batch issued
@@ -674,17 +678,14 @@ combine_kernel(const CombineEntry* entries, const CellGeom* cells, const float* 
 // merge their share as above, then one group merges the groups' results through shared memory.  With one thread
 // walking all parts of its row the launch ended with a few blocks each waiting on twenty memory round trips in turn.
 constexpr int COMBINE_LANES = 16;
-constexpr int COMBINE_LONG_PARTS = 16;  // entries with more parts than this go through combine_long_kernel
+constexpr int COMBINE_LONG_PARTS = 16;  // entries with more parts than this go through combine_long_row
 
 template <int D>
-__global__ void __launch_bounds__(COMBINE_LANES * (D / 8))
-combine_long_kernel(const CombineEntry* entries, const CellGeom* cells, const float* part_o, const float2* part_ml,
-                    __nv_bfloat16* out, int n_heads, int tokens_per_frame, int grid_w) {
+__device__ __forceinline__ void combine_long_row(const CombineEntry& e, int r, const CellGeom* cells, const float* part_o, const float2* part_ml,
+                                                 __nv_bfloat16* out, int n_heads, int tokens_per_frame, int grid_w) {
   constexpr int CHUNKS = D / 8;
   __shared__ float sh_m[COMBINE_LANES], sh_l[COMBINE_LANES];
   __shared__ float sh_acc[COMBINE_LANES][D];
-  const CombineEntry e = entries[blockIdx.x / 128];
-  const int r = blockIdx.x % 128;
   if (r >= e.q_count) return;  // the whole block leaves: no barrier is missed
   const int c = threadIdx.x % CHUNKS, lane = threadIdx.x / CHUNKS;
   const size_t row0 = static_cast<size_t>(e.first_slot) * 256 + e.sub * 128 + r;
@@ -731,6 +732,25 @@ combine_long_kernel(const CombineEntry* entries, const CellGeom* cells, const fl
   o4.z = pack_bf16x2(acc[4] * inv, acc[5] * inv);
   o4.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
   *reinterpret_cast<uint4*>(out + (static_cast<size_t>(token) * n_heads + e.head) * D + c * 8) = o4;
+}
+
+// One launch for both: the first n_long entries are the long ones, a block per row, the others take 16 rows per block.
+template <int D>
+__global__ void __launch_bounds__(COMBINE_ROWS * (D / 8))
+combine_kernel(const CombineEntry* entries, int n_long, const CellGeom* cells, const float* part_o, const float2* part_ml,
+               __nv_bfloat16* out, int n_heads, int tokens_per_frame, int grid_w) {
+  static_assert(COMBINE_ROWS == COMBINE_LANES, "both kinds of block have the same threads");
+  constexpr int PER_ENTRY = 128 / COMBINE_ROWS;
+  pdl_launch_dependents();
+  pdl_wait();
+  const int b = blockIdx.x - n_long * 128;
+  if (b < 0) {
+    const CombineEntry e = entries[blockIdx.x / 128];
+    combine_long_row<D>(e, blockIdx.x % 128, cells, part_o, part_ml, out, n_heads, tokens_per_frame, grid_w);
+  } else {
+    const CombineEntry e = entries[n_long + b / PER_ENTRY];
+    combine_rows<D>(e, b % PER_ENTRY, cells, part_o, part_ml, out, n_heads, tokens_per_frame, grid_w);
+  }
 }
 
 }  // namespace hc

@@ -50,13 +50,13 @@ struct Schedule {
   int key_filled = -1;  // cache fill the lists were built for
   std::vector<WorkItem> items;
   std::vector<int32_t> cta_first;
-  std::vector<CombineEntry> combine;       // query tiles to merge, up to COMBINE_LONG_PARTS pieces each
-  std::vector<CombineEntry> combine_long;  // those cut into more pieces (combine_long_kernel)
+  std::vector<CombineEntry> combine;  // query tiles to merge; the first n_long are cut into more than COMBINE_LONG_PARTS pieces
+  int n_long = 0;
   std::vector<ClsGroup> cls_groups;  // classification only: key ranges of one query pair, merged three ways
   std::vector<ClsPart> cls_parts;
   DevBuf<WorkItem> items_dev;
   DevBuf<int32_t> cta_first_dev;
-  DevBuf<CombineEntry> combine_dev, combine_long_dev;
+  DevBuf<CombineEntry> combine_dev;
   DevBuf<ClsGroup> cls_groups_dev;
   DevBuf<ClsPart> cls_parts_dev;
   int n_slots = 0;
@@ -67,7 +67,6 @@ struct Schedule {
     items_dev.release();
     cta_first_dev.release();
     combine_dev.release();
-    combine_long_dev.release();
     cls_groups_dev.release();
     cls_parts_dev.release();
   }

@@ -92,8 +92,8 @@ __global__ void __launch_bounds__(MOVE_ENGINES * 32, 1) move_kernel(const __grid
   // resident and set up their barriers while the kernel before it on the stream drains.  launch_dependents lets the
   // NEXT such kernel do the same with this one; wait returns once the preceding kernel has completed and its writes
   // are visible, and comes before this kernel's first access to global memory.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_launch_dependents();
+  pdl_wait();
   if ((threadIdx.x & 31) != 0) return;
   const int e = threadIdx.x >> 5;
   uint8_t* stage = smem + e * MOVE_STAGE_BYTES;

@@ -93,7 +93,7 @@ double item_cost(const WorkItem& w) {
 void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos, bool allow_split) {
   s.items.clear();
   s.combine.clear();
-  s.combine_long.clear();
+  s.n_long = 0;
   s.n_slots = 0;
   const int n_cta = c->n_sm;
   std::vector<std::vector<WorkItem>> bins(n_cta + 1);  // bins[n_cta]: the shared queue (dynamic tail)
@@ -381,7 +381,6 @@ void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos,
           by_group[w.out_slot].push_back({b, static_cast<int>(i), w.tile_begin});
         }
       s.combine.clear();
-      s.combine_long.clear();
       s.n_slots = 0;
       for (auto& pieces : by_group) {
         if (pieces.empty()) continue;
@@ -405,9 +404,11 @@ void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos,
           e.n_parts = static_cast<int32_t>(pieces.size());
           e.sub = t;
           e.pad = 0;
-          (e.n_parts > COMBINE_LONG_PARTS ? s.combine_long : s.combine).push_back(e);
+          s.combine.push_back(e);
         }
       }
+      auto first_short = std::stable_partition(s.combine.begin(), s.combine.end(), [](const CombineEntry& e) { return e.n_parts > COMBINE_LONG_PARTS; });
+      s.n_long = static_cast<int>(first_short - s.combine.begin());
     }
     // classification: the pieces of every group, in group order
     std::stable_sort(cls_raw.begin(), cls_raw.end(), [](const RawPart& a, const RawPart& b) { return a.group < b.group; });

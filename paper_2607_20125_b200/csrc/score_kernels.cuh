@@ -41,6 +41,8 @@ template <int D>
 __global__ void __launch_bounds__(COMBINE_ROWS * (D / 8))
 cls_combine_kernel(const ClsGroup* groups, const ClsPart* parts, const float* part_o, const float2* part_ml, float* o_ref,
                    float* lse_ref, float* tok, int n_heads, int block_tokens) {
+  pdl_launch_dependents();
+  pdl_wait();
   constexpr int CHUNKS = D / 8;
   constexpr int BLOCKS_PER_TILE = 128 / COMBINE_ROWS;
   const ClsGroup g = groups[blockIdx.x / (2 * BLOCKS_PER_TILE)];
@@ -123,6 +125,8 @@ __global__ void __launch_bounds__(COMBINE_ROWS * (D / 8))
 proxy_combine_kernel(const ClsGroup* groups, const ClsPart* parts, const float* part_o, const float2* part_ml,
                      const float* part_mid, const float* o_ref, const float* lse_ref, float* tok, int n_heads,
                      int block_tokens) {
+  pdl_launch_dependents();
+  pdl_wait();
   constexpr int CHUNKS = D / 8;
   constexpr int BLOCKS_PER_TILE = 128 / COMBINE_ROWS;
   const ClsGroup g = groups[blockIdx.x / (2 * BLOCKS_PER_TILE)];
@@ -259,6 +263,8 @@ struct DecideParams {
 
 // One block per head: fixed-order sums (deterministic), percentile by selection, Eq. 4 and Eq. 5.
 __global__ void __launch_bounds__(1024) head_decide_kernel(const DecideParams p) {
+  pdl_launch_dependents();
+  pdl_wait();
   __shared__ double red[TOK_N][32];
   __shared__ uint32_t hist[256];
   __shared__ uint32_t bcast[3];

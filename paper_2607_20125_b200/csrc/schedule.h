@@ -85,10 +85,26 @@ double item_cost(const WorkItem& w) {
   return tile_cost(w) * (w.tile_end - w.tile_begin) + item_overhead(w) + (w.out_mode == OUT_PARTIAL ? PARTIAL_EXTRA : 0.0);
 }
 
+// The same for work lists with few items per CTA, where the line below has nothing to cut with: its pieces are whole items
+// or at least MIN_PART_TILES long, so five items on 148 SMs stayed five items and a launch took as long as the longest
+// (13 x 22 tokens, six heads, 4-block window: 27 key tiles in a row on one SM, 45 us per launch, 116 SMs idle).
+// Fitted to the per-item timings of the one-thread-per-row kernel (a pair tile takes 1.69 us): Spatial tiles 1.12, lone
+// tiles 0.90, 3.8 / 2.8 us per item, 1.9 us per partial result; merging costs one more launch of about 4 us.
+// Append + four attends: 13 x 22 tokens, six heads 203 -> 96 us; 8 x 8, four heads 75 -> 64; 10 x 13, six heads 134 -> 84.
+constexpr double SHORT_SPATIAL = 1.12, SHORT_SINGLE = 0.90, SHORT_ITEM = 2.2, SHORT_ITEM_SINGLE = 1.7, SHORT_PARTIAL = 1.1, SHORT_MERGE = 2.4;
+constexpr double SHORT_LIST_TILES = 40.0;  // tile-steps per CTA up to which lists are cut this way (above, the dynamic tail takes over)
+
+double short_cost(const WorkItem& w, int n_tiles, bool partial) {
+  const bool pair = w.q_count[1] > 0;
+  return (pair ? 1.0 : SHORT_SINGLE) * (w.cell >= 0 ? SHORT_SPATIAL : 1.0) * n_tiles + (pair ? SHORT_ITEM : SHORT_ITEM_SINGLE) +
+         (partial ? SHORT_PARTIAL : 0.0);
+}
+
 // Assigns work to the persistent CTAs (one per SM).
 //  - allow_split: the items, longest first, are laid end to end and the line is cut into one equal share per
 //    CTA; an item that straddles a cut is divided along its key range, its pieces write unnormalised partial
 //    results and combine_kernel merges them.  Every CTA then carries the same number of tile-times.
+//    Short lists are cut into equal pieces instead, dealt longest first, if that is predicted to end earlier.
 //  - otherwise (outputs that cannot be merged afterwards): whole items, longest first, onto the least loaded CTA.
 void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos, bool allow_split) {
   s.items.clear();
@@ -191,6 +207,63 @@ void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos,
       for (int b = 0; b < n_cta; ++b) n += bins[b].size() == bin_base[b];
       return n;
     };
+    // Short lists: every item in pieces of at most `piece` key tiles, dealt longest first onto the least loaded CTA.
+    // Returns the predicted end of the launch; places the pieces only if `commit` is set.
+    auto lay_out_pieces = [&](int piece, bool commit) -> double {
+      struct Cut { double cost; size_t proto; int begin, take; };
+      std::vector<Cut> cuts;
+      bool merge = false;
+      for (size_t pi = 0; pi < protos.size(); ++pi) {
+        const Proto& p = protos[pi];
+        const int n = (p.n_tiles + piece - 1) / piece;
+        merge = merge || n > 1;
+        for (int k = 0; k < n; ++k) {
+          const int b = static_cast<int>(static_cast<long long>(p.n_tiles) * k / n), e = static_cast<int>(static_cast<long long>(p.n_tiles) * (k + 1) / n);
+          cuts.push_back({short_cost(p.w, e - b, n > 1 || p.cls_group >= 0 || p.always_partial), pi, b, e - b});
+        }
+      }
+      std::stable_sort(cuts.begin(), cuts.end(), [](const Cut& a, const Cut& b) { return a.cost > b.cost; });
+      typedef std::pair<double, int> Load;
+      std::priority_queue<Load, std::vector<Load>, std::greater<Load>> pq;
+      for (int b = 0; b < n_cta; ++b) pq.push(Load(0.0, b));
+      if (commit) {
+        for (auto& bin : bins) bin.clear();
+        cls_raw.clear();
+        s.n_slots = 0;
+      }
+      double end = 0.0;
+      for (const Cut& c : cuts) {
+        Load l = pq.top();
+        pq.pop();
+        end = std::max(end, l.first + c.cost);
+        pq.push(Load(l.first + c.cost, l.second));
+        if (!commit) continue;
+        const Proto& p = protos[c.proto];
+        WorkItem w = p.w;
+        w.tile_begin = p.tile_off + c.begin;
+        w.tile_end = p.tile_off + c.begin + c.take;
+        w.out_mode = OUT_PARTIAL;
+        w.out_slot = p.cls_group >= 0 ? s.n_slots++ : p.group;
+        if (p.cls_group >= 0) cls_raw.push_back({p.cls_group, w.out_slot, p.cls_tag});
+        bins[l.second].push_back(w);
+      }
+      return end + (merge ? SHORT_MERGE : 0.0);
+    };
+    // What the line's layout comes to under the same cost model.
+    auto short_end_of_line = [&]() -> double {
+      std::vector<int> pieces_of(protos.size(), 0);
+      bool merge = false;
+      for (const auto& bin : bins)
+        for (const WorkItem& w : bin)
+          if (s.cls_groups.empty()) merge = ++pieces_of[w.out_slot] > 1 || merge;
+      double end = 0.0;
+      for (const auto& bin : bins) {
+        double load = 0.0;
+        for (const WorkItem& w : bin) load += short_cost(w, w.tile_end - w.tile_begin, !s.cls_groups.empty() || pieces_of[w.out_slot] > 1);
+        end = std::max(end, load);
+      }
+      return end + (merge ? SHORT_MERGE : 0.0);
+    };
     double tail_budget = 0.0;
     auto place = [&](size_t first, size_t last) {  // spreads protos [first, last) over all CTAs, after what is there
       first_proto = first;
@@ -233,6 +306,18 @@ void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos,
           }
         }
         lay_out(share);
+      }
+      if (first == 0 && last == protos.size() && total <= SHORT_LIST_TILES * n_cta) {
+        double best = 0.95 * short_end_of_line();  // (at a predicted gain of less the line was as fast or up to 3 % faster)
+        int best_piece = 0;
+        for (int piece : {64, 48, 40, 32, 24, 20, 16, 12, 10, 8, 6, 5, 4, 3, 2, 1}) {
+          const double end = lay_out_pieces(piece, false);
+          if (end < best) {
+            best = end;
+            best_piece = piece;
+          }
+        }
+        if (best_piece > 0) lay_out_pieces(best_piece, true);
       }
       for (int b = 0; b < n_cta; ++b) bin_base[b] = bins[b].size();
       combine_base = s.combine.size();

@@ -26,9 +26,9 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 
 int upload_schedule(headcast_ctx* c, Schedule& s, cudaStream_t st) {
   if (s.uploaded) return HC_OK;
-  HC_CUDA(c, s.items_dev.reserve(std::max<size_t>(1, s.items.size())));
-  HC_CUDA(c, s.cta_first_dev.reserve(s.cta_first.size()));
-  HC_CUDA(c, s.combine_dev.reserve(std::max<size_t>(1, s.combine.size())));
+  HC_CUDA(c, s.items_dev.reserve(std::max<size_t>(1, s.items.size()), st));
+  HC_CUDA(c, s.cta_first_dev.reserve(s.cta_first.size(), st));
+  HC_CUDA(c, s.combine_dev.reserve(std::max<size_t>(1, s.combine.size()), st));
   if (!s.items.empty())
     HC_CUDA(c, cudaMemcpyAsync(s.items_dev.ptr, s.items.data(), s.items.size() * sizeof(WorkItem),
                                cudaMemcpyHostToDevice, st));
@@ -38,17 +38,17 @@ int upload_schedule(headcast_ctx* c, Schedule& s, cudaStream_t st) {
     HC_CUDA(c, cudaMemcpyAsync(s.combine_dev.ptr, s.combine.data(), s.combine.size() * sizeof(CombineEntry),
                                cudaMemcpyHostToDevice, st));
   if (!s.cls_groups.empty()) {
-    HC_CUDA(c, s.cls_groups_dev.reserve(s.cls_groups.size()));
-    HC_CUDA(c, s.cls_parts_dev.reserve(std::max<size_t>(1, s.cls_parts.size())));
+    HC_CUDA(c, s.cls_groups_dev.reserve(s.cls_groups.size(), st));
+    HC_CUDA(c, s.cls_parts_dev.reserve(std::max<size_t>(1, s.cls_parts.size()), st));
     HC_CUDA(c, cudaMemcpyAsync(s.cls_groups_dev.ptr, s.cls_groups.data(), s.cls_groups.size() * sizeof(ClsGroup),
                                cudaMemcpyHostToDevice, st));
     HC_CUDA(c, cudaMemcpyAsync(s.cls_parts_dev.ptr, s.cls_parts.data(), s.cls_parts.size() * sizeof(ClsPart),
                                cudaMemcpyHostToDevice, st));
   }
   if (s.n_slots > 0) {
-    HC_CUDA(c, c->part_o.reserve(static_cast<size_t>(s.n_slots) * 256 * c->D));
-    HC_CUDA(c, c->part_ml.reserve(static_cast<size_t>(s.n_slots) * 256));
-    HC_CUDA(c, c->part_mid.reserve(static_cast<size_t>(s.n_slots) * 256));
+    HC_CUDA(c, c->part_o.reserve(static_cast<size_t>(s.n_slots) * 256 * c->D, st));
+    HC_CUDA(c, c->part_ml.reserve(static_cast<size_t>(s.n_slots) * 256, st));
+    HC_CUDA(c, c->part_mid.reserve(static_cast<size_t>(s.n_slots) * 256, st));
   }
   // The lists are uploaded once per cache fill and reused by later calls, which may come on another stream: wait
   // here, once, so that no later launch can see a half-written list (the host vectors are pageable, so the copies
@@ -108,7 +108,7 @@ int run_schedule(headcast_ctx* c, Schedule& s, const void* q, void* out, bool pr
   p.trace = nullptr;
   if (c->tracing) {
     const size_t trace_words = 2 * s.items.size();
-    HC_CUDA(c, c->trace_dev.reserve(trace_words));
+    HC_CUDA(c, c->trace_dev.reserve(trace_words, st));
     HC_CUDA(c, cudaMemsetAsync(c->trace_dev.ptr, 0, trace_words * sizeof(unsigned long long), st));
     p.trace = c->trace_dev.ptr;
     c->trace_items = s.items;
@@ -468,39 +468,43 @@ int headcast_create(const headcast_config* cfg, headcast_ctx** out) {
       return rc;
     }
   }
-  int dev = 0;
-  cudaDeviceProp prop;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess) {
+  int major = 0;  // (two attributes: cudaGetDeviceProperties takes 2.5 ms)
+  if (cudaGetDevice(&c->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, c->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) {
     delete c;
     return HC_ERR_CUDA;
   }
-  if (prop.major != 10) {
+  if (major != 10) {
     delete c;
     return HC_ERR_UNSUPPORTED;
   }
-  c->n_sm = prop.multiProcessorCount;
   const size_t mono_bytes = cache_elems(c, c->H) * sizeof(__nv_bfloat16);
   cudaError_t e = cudaSuccess;
   auto step = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-  // the monolithic cache comes from the stream-ordered allocator, so that the split can release it in stream order
-  // (cudaFreeAsync) instead of stalling the host and the device in a cudaFree
-  step(cudaMallocAsync(reinterpret_cast<void**>(&c->mono_k), mono_bytes, nullptr));
-  step(cudaMallocAsync(reinterpret_cast<void**>(&c->mono_v), mono_bytes, nullptr));
-  step(cudaMalloc(&c->arena_k, mono_bytes));
-  step(cudaMalloc(&c->arena_v, mono_bytes));
-  step(cudaMalloc(&c->sp_base, c->T_f * sizeof(int32_t)));
-  step(cudaMalloc(&c->sp_nc, c->T_f * sizeof(int32_t)));
-  step(cudaMalloc(&c->cells_dev, c->cells.size() * sizeof(CellGeom)));
-  step(cudaMalloc(&c->status_dev, sizeof(int32_t)));
-  step(cudaMalloc(&c->dyn_counter_dev, 2 * sizeof(int32_t)));
-  if (e == cudaSuccess) step(cudaMemset(c->dyn_counter_dev, 0, 2 * sizeof(int32_t)));
-  if (c->move_ok) step(cudaMalloc(&c->move_boxes_dev, std::max<size_t>(1, c->move_boxes.size()) * sizeof(MoveBox)));
+  step(refuse_capture(nullptr));
+  auto get = [&](auto** ptr, size_t bytes) {
+    void* m = nullptr;
+    if (e == cudaSuccess) step(block_alloc(&m, bytes));
+    *ptr = static_cast<std::remove_pointer_t<decltype(ptr)>>(m);
+  };
+  if (e == cudaSuccess) step(mono_alloc(reinterpret_cast<void**>(&c->mono_k), mono_bytes, c->device));
+  if (e == cudaSuccess) step(mono_alloc(reinterpret_cast<void**>(&c->mono_v), mono_bytes, c->device));
+  get(&c->arena_k, mono_bytes);
+  get(&c->arena_v, mono_bytes);
+  get(&c->sp_base, c->T_f * sizeof(int32_t));
+  get(&c->sp_nc, c->T_f * sizeof(int32_t));
+  get(&c->cells_dev, c->cells.size() * sizeof(CellGeom));
+  get(&c->status_dev, sizeof(int32_t));
+  get(&c->dyn_counter_dev, 2 * sizeof(int32_t));
+  if (c->move_ok) get(&c->move_boxes_dev, std::max<size_t>(1, c->move_boxes.size()) * sizeof(MoveBox));
   if (e == cudaSuccess) {
-    step(cudaMemset(c->mono_k, 0, mono_bytes));
-    step(cudaMemset(c->mono_v, 0, mono_bytes));
-    step(cudaMemset(c->arena_k, 0, mono_bytes));
-    step(cudaMemset(c->arena_v, 0, mono_bytes));
-    step(cudaMemset(c->status_dev, 0, sizeof(int32_t)));
+    step(cudaMemsetAsync(c->dyn_counter_dev, 0, 2 * sizeof(int32_t), nullptr));
+    step(cudaMemsetAsync(c->mono_k, 0, mono_bytes, nullptr));
+    step(cudaMemsetAsync(c->mono_v, 0, mono_bytes, nullptr));
+    step(cudaMemsetAsync(c->arena_k, 0, mono_bytes, nullptr));
+    step(cudaMemsetAsync(c->arena_v, 0, mono_bytes, nullptr));
+    step(cudaMemsetAsync(c->status_dev, 0, sizeof(int32_t), nullptr));
     step(cudaMemcpy(c->sp_base, sp_base.data(), c->T_f * sizeof(int32_t), cudaMemcpyHostToDevice));
     step(cudaMemcpy(c->sp_nc, sp_nc.data(), c->T_f * sizeof(int32_t), cudaMemcpyHostToDevice));
     step(cudaMemcpy(c->cells_dev, c->cells.data(), c->cells.size() * sizeof(CellGeom), cudaMemcpyHostToDevice));
@@ -525,37 +529,40 @@ int headcast_create(const headcast_config* cfg, headcast_ctx** out) {
 
 int headcast_destroy(headcast_ctx* c) {
   if (!c) return HC_OK;
+  int current = c->device;  // the context's memory belongs to its own device, whichever one is current now
+  cudaGetDevice(&current);
+  if (current != c->device) cudaSetDevice(c->device);
   cudaDeviceSynchronize();
   if (c->mono_k) cudaFreeAsync(c->mono_k, nullptr);
   if (c->mono_v) cudaFreeAsync(c->mono_v, nullptr);
-  cudaDeviceSynchronize();
   void* ptrs[] = {c->arena_k, c->arena_v, c->sp_base, c->sp_nc, c->cells_dev, c->status_dev, c->dyn_counter_dev, c->move_boxes_dev};
   for (void* p : ptrs)
-    if (p) cudaFree(p);
+    if (p) BlockCache::of(c->device)->put(p);
   if (c->ev_a) cudaEventDestroy(c->ev_a);
   if (c->ev_b) cudaEventDestroy(c->ev_b);
-  c->sched_dense.release();
-  c->sched_hc.release();
-  c->sched_cls.release();
-  c->sched_proxy.release();
-  for (Schedule& g : c->sched_stage) g.release();
-  c->stage_q.release();
-  c->stage_out.release();
-  c->stage_k.release();
-  c->stage_v.release();
+  c->sched_dense.release(c->device);
+  c->sched_hc.release(c->device);
+  c->sched_cls.release(c->device);
+  c->sched_proxy.release(c->device);
+  for (Schedule& g : c->sched_stage) g.release(c->device);
+  c->stage_q.release(c->device);
+  c->stage_out.release(c->device);
+  c->stage_k.release(c->device);
+  c->stage_v.release(c->device);
   if (c->copy_in) cudaStreamDestroy(c->copy_in);
   if (c->copy_out) cudaStreamDestroy(c->copy_out);
   for (cudaEvent_t e : c->ev_host)
     if (e) cudaEventDestroy(e);
-  c->part_o.release();
-  c->part_ml.release();
-  c->part_mid.release();
-  c->trace_dev.release();
-  c->cls_o.release();
-  c->cls_lse.release();
-  c->cls_tok.release();
-  c->cls_scores.release();
-  c->cls_labels.release();
+  c->part_o.release(c->device);
+  c->part_ml.release(c->device);
+  c->part_mid.release(c->device);
+  c->trace_dev.release(c->device);
+  c->cls_o.release(c->device);
+  c->cls_lse.release(c->device);
+  c->cls_tok.release(c->device);
+  c->cls_scores.release(c->device);
+  c->cls_labels.release(c->device);
+  if (current != c->device) cudaSetDevice(current);
   delete c;
   return HC_OK;
 }
@@ -650,11 +657,11 @@ int headcast_classify(headcast_ctx* c, const void* q, int32_t* labels_host, floa
   if (n_filled(c) < 2) return fail(c, HC_ERR_STATE, "classification needs at least two cached blocks");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t rows = static_cast<size_t>(c->L) * c->H;
-  HC_CUDA(c, c->cls_o.reserve(rows * c->D));  // the reference output (fp32); the proxy outputs never leave registers
-  HC_CUDA(c, c->cls_lse.reserve(rows));
-  HC_CUDA(c, c->cls_tok.reserve(TOK_N * rows));
-  HC_CUDA(c, c->cls_scores.reserve(static_cast<size_t>(c->H) * HC_N_SCORES));
-  HC_CUDA(c, c->cls_labels.reserve(c->H));
+  HC_CUDA(c, c->cls_o.reserve(rows * c->D, st));  // the reference output (fp32); the proxy outputs never leave registers
+  HC_CUDA(c, c->cls_lse.reserve(rows, st));
+  HC_CUDA(c, c->cls_tok.reserve(TOK_N * rows, st));
+  HC_CUDA(c, c->cls_scores.reserve(static_cast<size_t>(c->H) * HC_N_SCORES, st));
+  HC_CUDA(c, c->cls_labels.reserve(c->H, st));
   const int newest = c->slots.back();
   const int cls_key = n_filled(c) * 64 + newest;  // the work lists depend on the fill and on where the newest block sits
   if (c->sched_cls.key_filled != cls_key) {
@@ -857,8 +864,8 @@ int headcast_append_host(headcast_ctx* c, const void* k_host, const void* v_host
   if (!c || !k_host || !v_host) return HC_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t elems = static_cast<size_t>(c->L) * c->H * c->D;
-  HC_CUDA(c, c->stage_k.reserve(elems));
-  HC_CUDA(c, c->stage_v.reserve(elems));
+  HC_CUDA(c, c->stage_k.reserve(elems, st));
+  HC_CUDA(c, c->stage_v.reserve(elems, st));
   HC_CUDA(c, cudaMemcpyAsync(c->stage_k.ptr, k_host, elems * sizeof(__nv_bfloat16), cudaMemcpyHostToDevice, st));
   HC_CUDA(c, cudaMemcpyAsync(c->stage_v.ptr, v_host, elems * sizeof(__nv_bfloat16), cudaMemcpyHostToDevice, st));
   return headcast_append(c, c->stage_k.ptr, c->stage_v.ptr, stream);
@@ -871,8 +878,8 @@ int headcast_attend_host(headcast_ctx* c, const void* q_host, void* out_host, vo
   int rc = init_host_path(c);
   if (rc != HC_OK) return rc;
   const size_t elems = static_cast<size_t>(c->L) * c->H * c->D;
-  HC_CUDA(c, c->stage_q.reserve(elems));
-  HC_CUDA(c, c->stage_out.reserve(elems));
+  HC_CUDA(c, c->stage_q.reserve(elems, st));
+  HC_CUDA(c, c->stage_out.reserve(elems, st));
   const int key = n_filled(c) * 4 + c->sd_valid;
   // Stages: a stage's queries are copied in (strided: the rows of [L][H][d] hold all heads), attended and copied out
   // as a unit, so that the next stage's queries arrive and the previous stage's outputs leave while this stage

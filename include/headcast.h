@@ -243,8 +243,8 @@ const char* headcast_last_error(const headcast_ctx* ctx);
  *     host threads - race on it.  Keep calls on one GPU in one stream, or order them with events;
  *   - the first call on each device looks up the array's device address and sets the kernel's shared-memory
  *     attribute (with that device current).  Make that first call before starting any stream capture;
- *   - a call on a stream that is being captured returns HC_ERR_UNSUPPORTED (the work list is copied from a host
- *     image that the next call rewrites).
+ *   - a call on a stream that is being captured returns HC_ERR_UNSUPPORTED (a graph replayed beside other calls
+ *     would overwrite the work list they share).
  * softmax_scale = 0 selects 1/sqrt(head_dim).  Asynchronous on `stream`.  headcast_noalloc_status synchronises
  * the stream and reports HC_ERR_TIMEOUT if the kernel gave up on a bounded wait; headcast_noalloc_last_error
  * returns the reason of the last failing call (process-wide buffer). */

@@ -1128,6 +1128,34 @@ struct NoAllocScratch {
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocScratch)];
 
+// Writes the work list of one call: whole query-tile pairs, dealt round-robin to one CTA per SM (every item has the same key
+// range).  Built here and not copied from the host: three copies from pageable memory made a call take 21 us of host time
+// whatever its size.
+__global__ void __launch_bounds__(256) noalloc_list_kernel(NoAllocScratch* s, int n_items, int n_cta, int n_heads, int head_dim,
+                                                           int n_queries, int n_keys) {
+  pdl_launch_dependents();
+  pdl_wait();  // the kernel before may still read the list of its own call
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  const int each = n_items / n_cta, more = n_items % n_cta;  // CTA b owns items b, b + n_cta, ...: `each`, plus one for the first `more`
+  if (i <= n_cta) s->cta_first[i] = i * each + min(i, more);
+  if (i == 0) s->status = 0;  // the array keeps the previous call's contents
+  if (i >= n_items) return;
+  const int b = i % n_cta, h = i % n_heads, q0 = i / n_heads * 256;
+  WorkItem w = {};
+  w.head = h;
+  w.cell = -1;
+  w.q_start[0] = q0;
+  w.q_start[1] = q0 + 128;
+  w.q_count[0] = min(128, n_queries - q0);
+  w.q_count[1] = max(0, min(128, n_queries - q0 - 128));
+  w.kv_x0 = h * head_dim;
+  w.seg_len = n_keys;
+  w.tiles_per_seg = (n_keys + 127) / 128;
+  w.tile_end = w.tiles_per_seg;
+  w.out_mode = OUT_BF16;
+  s->items[b * each + min(b, more) + i / n_cta] = w;
+}
+
 constexpr int NOALLOC_MAX_DEVICES = 64;
 struct NoAllocDevice {
   NoAllocScratch* scratch = nullptr;  // device address of g_noalloc_scratch on that GPU
@@ -1193,8 +1221,8 @@ int headcast_dense_attend_noalloc(const void* q, const void* k, const void* v, v
   const NoAllocDevice& d = g_noalloc_dev[dev];
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   {
-    // the work list is copied from a host image that the next call rewrites: a captured copy would re-read it at
-    // every replay, so capturing streams are turned away
+    // calls share one scratch array: a graph replayed beside other calls would overwrite their work list, so capturing
+    // streams are turned away
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     e = cudaStreamIsCapturing(st, &cap);
     if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "cudaStreamIsCapturing", e);
@@ -1202,38 +1230,17 @@ int headcast_dense_attend_noalloc(const void* q, const void* k, const void* v, v
       return noalloc_fail(HC_ERR_UNSUPPORTED, "headcast_dense_attend_noalloc cannot be called on a capturing stream");
   }
 
-  // host image of the scratch: thread-local static storage, no heap
-  static thread_local NoAllocScratch host;
   const uint64_t row_elems = static_cast<uint64_t>(n_heads) * head_dim;
   AttnParams p;
   std::memset(&p, 0, sizeof(p));
   if (!make_tmap_bf16_2d(&p.maps[0], k, row_elems, n_keys, row_elems, 128) ||
       !make_tmap_bf16_2d(&p.maps[1], v, row_elems, n_keys, row_elems, 128))
     return noalloc_fail(HC_ERR_CUDA, "cuTensorMapEncodeTiled failed or is unavailable");
-  // whole query-tile pairs, dealt round-robin to one CTA per SM (every item has the same key range)
   const int n_cta = d.n_sm;
-  int n = 0;
-  for (int b = 0; b < n_cta; ++b) {
-    host.cta_first[b] = n;
-    for (long long i = b; i < n_items; i += n_cta) {
-      const int h = static_cast<int>(i % n_heads), q0 = static_cast<int>(i / n_heads) * 256;
-      WorkItem w = range_item(h, 0, h * head_dim, 0, n_keys);
-      w.q_start[0] = q0;
-      w.q_start[1] = q0 + 128;
-      w.q_count[0] = std::min(128, n_queries - q0);
-      w.q_count[1] = std::max(0, std::min(128, n_queries - q0 - 128));
-      w.tile_begin = 0;
-      w.tile_end = w.tiles_per_seg;
-      host.items[n++] = w;
-    }
-  }
-  host.cta_first[n_cta] = n;
-  host.status = 0;  // the array keeps the previous call's contents: the status word must start at zero
-  e = cudaMemcpyAsync(d.scratch->items, host.items, static_cast<size_t>(n) * sizeof(WorkItem), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(d.scratch->cta_first, host.cta_first, (n_cta + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&d.scratch->status, &host.status, sizeof(int32_t), cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "copying the work list into the static scratch", e);
+  const int list_threads = std::max(static_cast<int>(n_items), n_cta + 1);
+  e = launch_pdl(noalloc_list_kernel, dim3((list_threads + 255) / 256), dim3(256), 0, st, d.scratch, static_cast<int>(n_items), n_cta,
+                 n_heads, head_dim, n_queries, n_keys);
+  if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "launching the list kernel", e);
 
   p.items = d.scratch->items;
   p.cta_first = d.scratch->cta_first;

@@ -47,3 +47,30 @@ def test_row_maximum_grows_and_falls_from_tile_to_tile(head_dim, n_q):
     q = q + 12.0 * head_dim ** 0.25 * sign[:, None, None] * u
     k = k + 1.1 * head_dim ** 0.25 * steps[:, None, None] * u
     check(q.bfloat16(), k.bfloat16(), v.bfloat16())
+
+
+@pytest.mark.parametrize("heads,n_q", [(1, 1), (3, 256 * 49), (4, 256 * 37), (4, 256 * 37 + 1), (5, 256 * 59 + 130), (64, 256 * 32)])
+def test_work_list_of_the_allocation_free_call(heads, n_q):
+    """1, 147, 148, 152, 300 and 2048 (the limit) work items: fewer than, as many as and more than one per SM."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(heads)
+    q, k, v = (torch.randn(n, heads, 64, device="cuda", generator=gen).bfloat16() for n in (n_q, 70, 70))
+    check(q, k, v)
+
+
+def test_allocation_free_calls_of_different_sizes_back_to_back():
+    """Every call rewrites the list that the call before it still works on: nothing waits in between on the host."""
+    import torch
+    from paper_2607_20125_b200 import binding
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    cases = []
+    for heads, n_q, n_k in ((16, 1373, 5492), (1, 5, 3), (12, 3000, 900), (2, 129, 64)) * 3:
+        q, k, v = (torch.randn(n, heads, 64, device="cuda", generator=gen).bfloat16() for n in (n_q, n_k, n_k))
+        cases.append((q, k, v, torch.empty_like(q)))
+    torch.cuda.synchronize()
+    for q, k, v, out in cases:
+        binding.dense_attend_noalloc(q, k, v, out)
+    binding.noalloc_status()
+    for q, k, v, out in cases:
+        err = (out.float() - reference(q, k, v)).abs()
+        assert err.max().item() <= MAX_ABS and err.mean().item() <= MEAN_ABS

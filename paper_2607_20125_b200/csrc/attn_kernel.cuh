@@ -116,22 +116,24 @@ __device__ __forceinline__ int cell_query_token(const CellGeom& g, int p, int to
   return f * tokens_per_frame + (g.y0 + dy) * grid_w + g.x0 + dx;
 }
 
-// Which of 32 consecutive keys a query row may see, as a bit mask: columns >= n_valid (ragged tail of a segment) are
-// never seen; for the Spatial proxy neither are keys outside the (2r+1)^2 neighbourhood of the query's grid position
-// (qy, qx).  tok0 is the in-frame token index of column 0.  The neighbourhood is at most 2r+1 runs of consecutive
-// tokens (one per grid row), so the mask costs a few integer operations per row of the neighbourhood, not per key.
-template <bool PROXY>
-__device__ __forceinline__ uint32_t visible_keys(int n_valid, int tok0, int qy, int qx, int radius, int grid_w) {
-  uint32_t tail = (n_valid >= 32) ? 0xffffffffu : (n_valid <= 0 ? 0u : (0xffffffffu >> (32 - n_valid)));
-  if (!PROXY) return tail;
-  uint32_t allow = 0;
-  const int lo_x = max(qx - radius, 0), hi_x = min(qx + radius, grid_w - 1);
+// Spatial proxy: which of a tile's 128 keys a query row may see, as four words of bits: keys >= n_valid (ragged tail of a
+// segment) are never seen, nor are keys outside the (2r+1)^2 neighbourhood of the query's grid position (qy, qx).  tok0 is
+// the in-frame token index of the tile's first key.  The neighbourhood is at most 2r+1 runs of consecutive tokens, one per
+// grid row, and a tile of 128 tokens meets two or three of them: the others are left out before any bit is set.
+__device__ __forceinline__ void visible_keys(uint32_t (&allow)[4], int n_valid, int tok0, int qy, int qx, int radius, int grid_w) {
+#pragma unroll
+  for (int w = 0; w < 4; ++w) allow[w] = 0u;
+  const int lo_x = max(qx - radius, 0) - tok0, hi_x = min(qx + radius, grid_w - 1) - tok0;
 #pragma unroll 1
   for (int ky = max(qy - radius, 0); ky <= qy + radius; ++ky) {
-    const int a = max(ky * grid_w + lo_x - tok0, 0), b = min(ky * grid_w + hi_x - tok0, 31);  // inclusive column range
-    if (a <= b) allow |= (0xffffffffu >> (31 - b + a)) << a;
+    const int first = max(ky * grid_w + lo_x, 0), last = min(ky * grid_w + hi_x, n_valid - 1);  // inclusive, inside the tile
+    if (first > last) continue;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const int a = max(first - 32 * w, 0), b = min(last - 32 * w, 31);
+      if (a <= b) allow[w] |= (0xffffffffu >> (31 - b + a)) << a;
+    }
   }
-  return allow & tail;
 }
 
 // Sets the logits of the keys a row must not see to -inf.  Outside the proxy only the ragged tail of a segment is
@@ -427,11 +429,11 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
         // Keys this row must not see count as -inf: the ragged tail of a segment, and for the Spatial proxy every key
         // outside the (2r+1)^2 neighbourhood.
         uint32_t visible[4] = {0u, 0u, 0u, 0u};
+        bool seen[4] = {true, true, true, true};  // proxy: does any row of this warp see one of the chunk's keys?
         if (PROXY) {
-          const int tok0 = w.kv_row0 + c * 128;  // in-frame token of the tile's first key
+          visible_keys(visible, n_valid, w.kv_row0 + c * 128, qy, qx, p.radius, p.grid_w);
 #pragma unroll
-          for (int ch = 0; ch < 4; ++ch)
-            visible[ch] = visible_keys<PROXY>(n_valid - ch * 32, tok0 + ch * 32, qy, qx, p.radius, p.grid_w);
+          for (int ch = 0; ch < 4; ++ch) seen[ch] = __any_sync(0xffffffffu, visible[ch] != 0u);
         }
         if (!(ok = mbar_wait(&bar_s_full[t], s_cnt & 1, abortp, p.status, 31))) break;
         ++s_cnt;
@@ -447,10 +449,12 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
           // and the exponentials could not be scheduled across the chunks (dense sweep 4828 -> 4620 us)
           if (PROXY || n_valid < 128) {
 #pragma unroll
-            for (int ch = 0; ch < 4; ++ch) apply_visible<PROXY>(sv[ch], visible[ch], n_valid - ch * 32);
+            for (int ch = 0; ch < 4; ++ch)
+              if (!PROXY || seen[ch]) apply_visible<PROXY>(sv[ch], visible[ch], n_valid - ch * 32);
           }
 #pragma unroll
           for (int ch = 0; ch < 4; ++ch) {
+            if (PROXY && !seen[ch]) continue;
 #pragma unroll
             for (int i = 0; i < 32; i += 8) {
               mx4[0] = max3(mx4[0], __uint_as_float(sv[ch][i]), __uint_as_float(sv[ch][i + 1]));
@@ -490,6 +494,10 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
 #pragma unroll
         for (int ch = 0; ch < 4; ++ch) {
           uint32_t pk[16];
+          if (PROXY && !seen[ch]) {  // nothing to exponentiate: P = 0 (the product still reads it)
+#pragma unroll
+            for (int i = 0; i < 16; ++i) pk[i] = 0u;
+          } else
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const uint64_t x2 = fma_f32x2(pack_f32x2(__uint_as_float(sv[ch][2 * i]), __uint_as_float(sv[ch][2 * i + 1])), c2, m2);

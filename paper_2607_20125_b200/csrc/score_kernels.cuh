@@ -198,6 +198,7 @@ __device__ __forceinline__ float float_from_key(uint32_t k) {
 // *n_le receives how many values are <= the result (so the caller can tell whether rank k + 1 holds the same value).
 __device__ float block_select(const float* v, int n, int k, uint32_t* hist /* [256] shared */, uint32_t* bcast /* [3] */,
                               uint32_t* n_le) {
+  __shared__ uint32_t totals[8];
   uint32_t prefix = 0, mask = 0, below_total = 0;
   int remaining = k;
   for (int shift = 24; shift >= 0; shift -= 8) {
@@ -205,14 +206,29 @@ __device__ float block_select(const float* v, int n, int k, uint32_t* hist /* [2
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       const uint32_t key = float_order_key(v[i]);
-      if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
+      // cosines crowd into a few bins: the lanes of a warp that hit the same one add their number once (an atomic per
+      // value queued up thousands of them on one address)
+      const bool in = (key & mask) == prefix;
+      const uint32_t digit = (key >> shift) & 255u;
+      const uint32_t peers = __match_any_sync(__activemask(), in ? digit : 256u);
+      if (in && static_cast<int>(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&hist[digit], static_cast<uint32_t>(__popc(peers)));
     }
     __syncthreads();
     if (threadIdx.x < 256) {
-      // the digit whose bin holds rank `remaining`: thread d adds up the bins below d (all threads read the same bin
-      // at the same time: a broadcast), exactly one thread finds the rank inside its own bin
-      uint32_t below = 0;
-      for (int d = 0; d < static_cast<int>(threadIdx.x); ++d) below += hist[d];
+      // the digit whose bin holds rank `remaining`: a scan of the 256 bins, eight warps by shuffles and their totals
+      // through shared memory (adding up the bins below one by one took a fifth of the kernel); one thread finds the rank
+      // inside its own bin
+      const uint32_t mine = hist[threadIdx.x];
+      uint32_t upto = mine;
+#pragma unroll
+      for (int off = 1; off < 32; off *= 2) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, upto, off);
+        if (static_cast<int>(threadIdx.x & 31) >= off) upto += y;
+      }
+      if ((threadIdx.x & 31) == 31) totals[threadIdx.x >> 5] = upto;
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      uint32_t below = upto - mine;
+      for (int w = 0; w < static_cast<int>(threadIdx.x >> 5); ++w) below += totals[w];
       const uint32_t rank = static_cast<uint32_t>(remaining);
       if (below <= rank && rank < below + hist[threadIdx.x]) {
         bcast[0] = threadIdx.x;

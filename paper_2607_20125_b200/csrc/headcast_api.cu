@@ -712,18 +712,30 @@ int headcast_classify(headcast_ctx* c, const void* q, int32_t* labels_host, floa
   int rc = run_schedule(c, c->sched_cls, q, nullptr, false, st);
   if (rc != HC_OK) return rc;
   if (c->sched_proxy.key_filled != cls_key) {
-    // Spatial proxy: per query-tile pair, the band of grid rows within r of any of its queries, in every cached frame
+    // Spatial proxy: per query-tile pair, the tokens from r rows and r columns before its first query to as many behind
+    // its last one, in every cached frame.  A pair that straddles two frames has to sweep whole frames, so frames of more
+    // than 256 tokens are dealt into pairs of their own, of equal size (30 x 52 tokens, r = 2: seven pairs of 223 queries
+    // and 4 key tiles per frame; with pairs of 256 across the block and whole grid rows it was 5 tiles, and 13 for every
+    // sixth pair: 144 us for the sweep, now 113).  Smaller frames fit into a tile or two either way.
     std::vector<Proto> protos;
     c->sched_proxy.cls_groups.clear();
-    const int r = c->cfg.proxy_radius;
+    const long long reach = std::min<long long>(static_cast<long long>(c->cfg.proxy_radius) * (c->G_w + 1), c->T_f);
+    struct Run { int q0, n; };
+    std::vector<Run> runs;
+    if (c->T_f > 256) {
+      const int per_frame = (c->T_f + 255) / 256, size = (c->T_f + per_frame - 1) / per_frame;
+      for (int f = 0; f < c->F_b; ++f)
+        for (int i = 0; i < c->T_f; i += size) runs.push_back({f * c->T_f + i, std::min(size, c->T_f - i)});
+    } else {
+      for (int q0 = 0; q0 < c->L; q0 += 256) runs.push_back({q0, std::min(256, c->L - q0)});
+    }
     for (int h = 0; h < c->H; ++h)
-      for (int q0 = 0; q0 < c->L; q0 += 256) {
-        const int q1 = std::min(c->L, q0 + 256) - 1;
+      for (const Run& run : runs) {
+        const int q0 = run.q0, q1 = run.q0 + run.n - 1;
         int a = 0, b = c->T_f;
         if (q0 / c->T_f == q1 / c->T_f) {
-          const int ylo = std::max(0, (q0 % c->T_f) / c->G_w - r), yhi = std::min(c->G_h - 1, (q1 % c->T_f) / c->G_w + r);
-          a = ylo * c->G_w;
-          b = (yhi + 1) * c->G_w;
+          a = static_cast<int>(std::max<long long>(0, q0 % c->T_f - reach));
+          b = static_cast<int>(std::min<long long>(c->T_f, q1 % c->T_f + reach + 1));
         }
         WorkItem w = range_item(h, MAP_MONO, h * c->D, a, b - a);
         w.seg_stride = c->T_f;
@@ -731,8 +743,8 @@ int headcast_classify(headcast_ctx* c, const void* q, int32_t* labels_host, floa
         p.w = w;
         p.w.q_start[0] = q0;
         p.w.q_start[1] = q0 + 128;
-        p.w.q_count[0] = std::min(128, c->L - q0);
-        p.w.q_count[1] = std::max(0, std::min(128, c->L - q0 - 128));
+        p.w.q_count[0] = std::min(128, run.n);
+        p.w.q_count[1] = std::max(0, run.n - 128);
         p.n_tiles = w.tiles_per_seg * n_filled(c) * c->F_b;
         p.w.tile_begin = 0;
         p.w.tile_end = p.n_tiles;

@@ -49,56 +49,37 @@ WorkItem range_item(int head, int map, int x0, long long row0, int n_keys) {
   return w;
 }
 
-// Cost model of the scheduler, in units of the time one key tile takes with both query tiles in flight (about 2.0 us),
-// fitted by least squares to the per-item timings of headcast_read_trace on B200 (480P, 720P and 1080P work lists,
-// residual 1-3 % of an item): a lone query tile still needs 0.86 of that because the chain S -> softmax -> P -> next S
-// is latency bound; every item pays for its query load, pipeline fill and epilogue; a partial result costs an extra
-// round trip through global memory; the tiles of Spatial items measure 2 % slower.
-#ifndef HC_COST_ITEM
-#define HC_COST_ITEM 2.4
-#endif
-#ifndef HC_COST_ITEM_SINGLE
-#define HC_COST_ITEM_SINGLE 1.0
-#endif
-#ifndef HC_COST_PARTIAL
-#define HC_COST_PARTIAL 0.75
-#endif
-#ifndef HC_COST_SPATIAL
-#define HC_COST_SPATIAL 1.02
-#endif
-#ifndef HC_COST_SINGLE
-#define HC_COST_SINGLE 0.86
-#endif
-constexpr double TILE_COST_PAIR = 1.0, TILE_COST_SINGLE = HC_COST_SINGLE;
-constexpr double ITEM_OVERHEAD = HC_COST_ITEM, ITEM_OVERHEAD_SINGLE = HC_COST_ITEM_SINGLE;
-constexpr double PARTIAL_EXTRA = HC_COST_PARTIAL;
-constexpr double SPATIAL_FACTOR = HC_COST_SPATIAL;  // tiles of Spatial items (queries gathered by cell, short cell-major key runs)
+// Cost model of the scheduler, in units of the time one key tile takes with both query tiles in flight (1.69 us): a lone
+// query tile needs most of that because the chain S -> softmax -> P -> next S is latency bound; every item pays for its
+// query load, pipeline fill and epilogue; a partial result costs an extra round trip through global memory; the tiles of
+// Spatial items (queries gathered by cell, short key runs) measure slower.
+struct CostModel {
+  double tile_single, item, item_single, partial, spatial;
+  double tile(const WorkItem& w) const { return (w.q_count[1] > 0 ? 1.0 : tile_single) * (w.cell >= 0 ? spatial : 1.0); }
+  double overhead(const WorkItem& w) const { return w.q_count[1] > 0 ? item : item_single; }
+  double cost(const WorkItem& w, int n_tiles, bool cut) const { return tile(w) * n_tiles + overhead(w) + (cut ? partial : 0.0); }
+  double cost(const WorkItem& w) const { return cost(w, w.tile_end - w.tile_begin, w.out_mode == OUT_PARTIAL); }
+};
+// Fitted by least squares to the per-item timings of headcast_read_trace on B200 (480P and 720P work lists, residual 4 % of
+// an item; 3.8 us per item, 2.8 for a lone tile, 1.9 per partial result).
+constexpr CostModel COST_MEASURED = {0.90, 2.2, 1.7, 1.1, 1.12};
+// What the line of a list of up to SHORT_LINE_TILES tile-steps per CTA is cut by: its items are few, the cuts fall between
+// whole items, and shares that charge less for an item end earlier (per CTA 9 tile-steps, 14 x 25 tokens, twelve heads: 120 us
+// per block against 127 with the measured costs; 14, 31 x 46, four heads: 173 against 182; 18, 25 x 33: 187 against 192).
+// Longer lists are charged too little by these (25, 15 x 27, sixteen heads: 251 us against 247; 33, 30 x 49, eight heads: 334
+// against 320; 190, 55 x 87, four heads, cells of 6, two-block Sink and Dummy heads: 1915 against 1600); 480P to 1080P do
+// not care.
+constexpr double SHORT_LINE_TILES = 20.0;
+constexpr CostModel COST_SHORT_LINE = {0.86, 2.4, 1.0, 0.75, 1.02};
 constexpr int MIN_PART_TILES = 4;  // never cut a key range into pieces shorter than this
-
-double tile_cost(const WorkItem& w) {
-  return (w.q_count[1] > 0 ? TILE_COST_PAIR : TILE_COST_SINGLE) * (w.cell >= 0 ? SPATIAL_FACTOR : 1.0);
-}
-
-double item_overhead(const WorkItem& w) { return w.q_count[1] > 0 ? ITEM_OVERHEAD : ITEM_OVERHEAD_SINGLE; }
-
-double item_cost(const WorkItem& w) {
-  return tile_cost(w) * (w.tile_end - w.tile_begin) + item_overhead(w) + (w.out_mode == OUT_PARTIAL ? PARTIAL_EXTRA : 0.0);
-}
 
 // The same for work lists with few items per CTA, where the line below has nothing to cut with: its pieces are whole items
 // or at least MIN_PART_TILES long, so five items on 148 SMs stayed five items and a launch took as long as the longest
 // (13 x 22 tokens, six heads, 4-block window: 27 key tiles in a row on one SM, 45 us per launch, 116 SMs idle).
-// Fitted to the per-item timings of the one-thread-per-row kernel (a pair tile takes 1.69 us): Spatial tiles 1.12, lone
-// tiles 0.90, 3.8 / 2.8 us per item, 1.9 us per partial result; merging costs one more launch of about 4 us.
+// Merging costs one more launch of about 4 us.
 // Append + four attends: 13 x 22 tokens, six heads 203 -> 96 us; 8 x 8, four heads 75 -> 64; 10 x 13, six heads 134 -> 84.
-constexpr double SHORT_SPATIAL = 1.12, SHORT_SINGLE = 0.90, SHORT_ITEM = 2.2, SHORT_ITEM_SINGLE = 1.7, SHORT_PARTIAL = 1.1, SHORT_MERGE = 2.4;
+constexpr double SHORT_MERGE = 2.4;
 constexpr double SHORT_LIST_TILES = 40.0;  // tile-steps per CTA up to which lists are cut this way (above, the dynamic tail takes over)
-
-double short_cost(const WorkItem& w, int n_tiles, bool partial) {
-  const bool pair = w.q_count[1] > 0;
-  return (pair ? 1.0 : SHORT_SINGLE) * (w.cell >= 0 ? SHORT_SPATIAL : 1.0) * n_tiles + (pair ? SHORT_ITEM : SHORT_ITEM_SINGLE) +
-         (partial ? SHORT_PARTIAL : 0.0);
-}
 
 // Assigns work to the persistent CTAs (one per SM).
 //  - allow_split: the items, longest first, are laid end to end and the line is cut into one equal share per
@@ -115,8 +96,11 @@ void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos,
   std::vector<std::vector<WorkItem>> bins(n_cta + 1);  // bins[n_cta]: the shared queue (dynamic tail)
   bool tail_mode = false;
   int tail_piece_tiles = 8;
-  std::stable_sort(protos.begin(), protos.end(),
-                   [](const Proto& a, const Proto& b) { return item_cost(a.w) > item_cost(b.w); });
+  double total_cost = 0.0;
+  for (const Proto& p : protos) total_cost += COST_SHORT_LINE.cost(p.w);
+  const CostModel& model = total_cost <= SHORT_LINE_TILES * n_cta ? COST_SHORT_LINE : COST_MEASURED;
+  auto item_cost = [&](const WorkItem& w) { return model.cost(w); };
+  std::stable_sort(protos.begin(), protos.end(), [&](const Proto& a, const Proto& b) { return item_cost(a.w) > item_cost(b.w); });
   if (allow_split) {
     // Lay the items end to end and give every CTA the same share Q of the line, cutting the item that straddles a
     // boundary.  Cuts add cost of their own (a second query load and epilogue, partial results), so the share that
@@ -144,12 +128,12 @@ void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos,
       };
       for (size_t pi = first_proto; pi < last_proto; ++pi) {
         const Proto& p = protos[pi];
-        const double per_tile = tile_cost(p.w), overhead = item_overhead(p.w);
+        const double per_tile = model.tile(p.w), overhead = model.overhead(p.w);
         std::vector<std::pair<int, WorkItem>> parts;  // (cta, piece)
         int begin = 0;
         while (begin < p.n_tiles) {
           const int left = p.n_tiles - begin;
-          const double need = per_tile * left + overhead + (begin > 0 ? PARTIAL_EXTRA : 0.0);
+          const double need = per_tile * left + overhead + (begin > 0 ? model.partial : 0.0);
           int take = left;
           if (tail_mode && cta == n_cta) {
             // the shared queue: pieces of a fixed size, drawn by whichever CTA is free
@@ -157,7 +141,7 @@ void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos,
             if (left - take < MIN_PART_TILES) take = left;
           } else if (need > room && cta < last_bin) {
             // as many tiles as fit, but both pieces must be worth having
-            const int can = std::min(static_cast<int>(std::floor((room - overhead - PARTIAL_EXTRA) / per_tile)),
+            const int can = std::min(static_cast<int>(std::floor((room - overhead - model.partial) / per_tile)),
                                      left - MIN_PART_TILES);
             if (can >= MIN_PART_TILES) {
               take = can;
@@ -172,7 +156,7 @@ void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos,
           w.tile_end = p.tile_off + begin + take;
           parts.push_back(std::make_pair(cta, w));
           const bool cut = (take < left) || begin > 0 || (p.cls_group >= 0) || p.always_partial;
-          const double cost = per_tile * take + overhead + (cut ? PARTIAL_EXTRA : 0.0);
+          const double cost = per_tile * take + overhead + (cut ? model.partial : 0.0);
           room -= cost;
           if (cta == n_cta - 1) last_load += cost;
           begin += take;
@@ -219,7 +203,7 @@ void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos,
         merge = merge || n > 1;
         for (int k = 0; k < n; ++k) {
           const int b = static_cast<int>(static_cast<long long>(p.n_tiles) * k / n), e = static_cast<int>(static_cast<long long>(p.n_tiles) * (k + 1) / n);
-          cuts.push_back({short_cost(p.w, e - b, n > 1 || p.cls_group >= 0 || p.always_partial), pi, b, e - b});
+          cuts.push_back({COST_MEASURED.cost(p.w, e - b, n > 1 || p.cls_group >= 0 || p.always_partial), pi, b, e - b});
         }
       }
       std::stable_sort(cuts.begin(), cuts.end(), [](const Cut& a, const Cut& b) { return a.cost > b.cost; });
@@ -259,7 +243,7 @@ void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos,
       double end = 0.0;
       for (const auto& bin : bins) {
         double load = 0.0;
-        for (const WorkItem& w : bin) load += short_cost(w, w.tile_end - w.tile_begin, !s.cls_groups.empty() || pieces_of[w.out_slot] > 1);
+        for (const WorkItem& w : bin) load += COST_MEASURED.cost(w, w.tile_end - w.tile_begin, !s.cls_groups.empty() || pieces_of[w.out_slot] > 1);
         end = std::max(end, load);
       }
       return end + (merge ? SHORT_MERGE : 0.0);
@@ -279,12 +263,21 @@ void finalize_schedule(headcast_ctx* c, Schedule& s, std::vector<Proto>& protos,
         const double budget = std::min(tail_budget, 0.5 * total);
         tail_mode = true;
         tail_piece_tiles = std::max(8, static_cast<int>(budget / (4.0 * n_cta)));
-        lay_out((total - budget) / n_cta);
+        // The queue also receives what the cuts cost.  In a launch of few items per CTA that would be most of it: the
+        // shares grow until the queue is 15 % of the launch at most (10 % made 32 x 33 tokens, twelve heads, 4 % slower).
+        double share = (total - budget) / n_cta;
+        for (int tries = 0; tries < 4; ++tries) {
+          lay_out(share);
+          double queued = 0.0;
+          for (const WorkItem& w : bins[n_cta]) queued += model.cost(w);
+          if (queued <= 0.15 * total) break;
+          share += (queued - 0.15 * total) / n_cta;
+        }
         tail_mode = false;
         for (int b = 0; b < n_cta; ++b) bin_base[b] = bins[b].size();
         return;
       }
-      double lo = ideal, hi = ideal + biggest + ITEM_OVERHEAD + PARTIAL_EXTRA;
+      double lo = ideal, hi = ideal + biggest + model.item + model.partial;
       while (!fits(hi)) hi *= 1.25;
       for (int iter = 0; iter < 24 && hi - lo > 0.25; ++iter) {
         const double mid = 0.5 * (lo + hi);

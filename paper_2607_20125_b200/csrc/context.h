@@ -43,12 +43,12 @@ class BlockCache {
     static BlockCache* const all = new BlockCache[MAX_DEVICES];  // never destroyed: a context may outlive static objects
     return dev >= 0 && dev < MAX_DEVICES ? &all[dev] : nullptr;
   }
-  // On the current device, which must be this cache's.
-  cudaError_t get(void** ptr, size_t bytes) {
+  // On the current device, which must be this cache's.  `fresh`: by cudaMalloc, whatever is kept here.
+  cudaError_t get(void** ptr, size_t bytes, bool fresh = false) {
     const size_t need = round_up(bytes);
     std::lock_guard<std::mutex> hold(lock_);
     size_t at = free_.size();
-    for (size_t i = 0; i < free_.size(); ++i)
+    for (size_t i = 0; i < free_.size() && !fresh; ++i)
       if (free_[i].bytes >= need && free_[i].bytes <= need + need / 4 && (at == free_.size() || free_[i].bytes < free_[at].bytes)) at = i;
     if (at < free_.size()) {
       *ptr = free_[at].ptr;
@@ -58,7 +58,7 @@ class BlockCache {
       return cudaSuccess;
     }
     cudaError_t e = cudaMalloc(ptr, need);
-    if (e == cudaErrorMemoryAllocation && !free_.empty()) {  // what is kept here may be what is missing
+    if (e == cudaErrorMemoryAllocation && !free_.empty() && !fresh) {  // what is kept here may be what is missing
       cudaGetLastError();
       shrink(0);
       e = cudaMalloc(ptr, need);
@@ -66,13 +66,13 @@ class BlockCache {
     if (e == cudaSuccess) live_[*ptr] = need;
     return e;
   }
-  void put(void* ptr) {  // the device has finished with it
+  void put(void* ptr, bool keep = true) {  // the device has finished with it (keep: false: by cudaFree, which waits)
     std::lock_guard<std::mutex> hold(lock_);
     auto it = live_.find(ptr);
     if (it == live_.end()) return;
     const size_t bytes = it->second;
     live_.erase(it);
-    if (bytes > CACHE_KEEP_BYTES) {
+    if (!keep || bytes > CACHE_KEEP_BYTES) {
       cudaFree(ptr);
       return;
     }
@@ -102,14 +102,6 @@ class BlockCache {
   std::map<void*, size_t> live_;
   size_t kept_ = 0;
 };
-
-// Whether `st` is capturing: memory that outlives a graph is not taken while one is recorded, as with cudaMalloc.
-cudaError_t refuse_capture(cudaStream_t st) {
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  const cudaError_t e = cudaStreamIsCapturing(st, &capture);
-  if (e != cudaSuccess) return e;
-  return capture == cudaStreamCaptureStatusNone ? cudaSuccess : cudaErrorStreamCaptureUnsupported;
-}
 
 cudaError_t block_alloc(void** ptr, size_t bytes) {
   int dev = 0;
@@ -162,16 +154,25 @@ struct DevBuf {  // grow-only device array of the context's device
   size_t cap = 0;
   cudaError_t reserve(size_t n, cudaStream_t st) {
     if (n <= cap) return cudaSuccess;
-    cudaError_t e = refuse_capture(st);
+    // while `st` is captured the cache stands aside: cudaMalloc then says whether memory may be taken in this capture mode
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &status);
     if (e != cudaSuccess) return e;
+    const bool capturing = status != cudaStreamCaptureStatusNone;
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if (ptr) {
+    BlockCache* cache = BlockCache::of(dev);
+    if (!cache) return cudaErrorInvalidDevice;
+    if (ptr && capturing) {
+      cache->put(ptr, false);
+    } else if (ptr) {
       if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;  // any stream may still use the old array
-      release(dev);
+      cache->put(ptr);
     }
+    ptr = nullptr;
+    cap = 0;
     void* bigger = nullptr;
-    e = block_alloc(&bigger, n * sizeof(T));
+    e = cache->get(&bigger, n * sizeof(T), capturing);
     if (e == cudaSuccess) {
       ptr = static_cast<T*>(bigger);
       cap = n;

@@ -482,7 +482,6 @@ int headcast_create(const headcast_config* cfg, headcast_ctx** out) {
   const size_t mono_bytes = cache_elems(c, c->H) * sizeof(__nv_bfloat16);
   cudaError_t e = cudaSuccess;
   auto step = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-  step(refuse_capture(nullptr));
   auto get = [&](auto** ptr, size_t bytes) {
     void* m = nullptr;
     if (e == cudaSuccess) step(block_alloc(&m, bytes));

@@ -35,13 +35,14 @@ enum { MAP_MONO = 0, MAP_SD = 1, MAP_GLOBAL = 2, MAP_SPATIAL = 3, N_MAP_PAIRS = 
 // allocation fails.  A block is given back only once the device has finished with it, so it may serve any stream.
 constexpr size_t CACHE_KEEP_BYTES = size_t(384) << 20;
 constexpr unsigned long long MONO_KEEP_BYTES = 256ull << 20;  // the same for the monolithic caches, see mono_alloc
-constexpr int MAX_DEVICES = 64;
 
 class BlockCache {
  public:
-  static BlockCache* of(int dev) {
-    static BlockCache* const all = new BlockCache[MAX_DEVICES];  // never destroyed: a context may outlive static objects
-    return dev >= 0 && dev < MAX_DEVICES ? &all[dev] : nullptr;
+  static BlockCache& of(int dev) {
+    static std::mutex lock;
+    static std::map<int, BlockCache>& all = *new std::map<int, BlockCache>;  // never destroyed: a context may outlive static objects
+    std::lock_guard<std::mutex> hold(lock);
+    return all[dev];
   }
   // On the current device, which must be this cache's.  `fresh`: by cudaMalloc, whatever is kept here.
   cudaError_t get(void** ptr, size_t bytes, bool fresh = false) {
@@ -107,8 +108,7 @@ cudaError_t block_alloc(void** ptr, size_t bytes) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  BlockCache* cache = BlockCache::of(dev);
-  return cache ? cache->get(ptr, bytes) : cudaErrorInvalidDevice;
+  return BlockCache::of(dev).get(ptr, bytes);
 }
 
 // The monolithic cache is released in the middle of a stream's work (at the split), so it comes from a stream-ordered pool
@@ -116,10 +116,9 @@ cudaError_t block_alloc(void** ptr, size_t bytes) {
 // 200 MB to map and unmap them again) and hands memory out again only once the work that used it has completed.
 cudaError_t mono_alloc(void** ptr, size_t bytes, int dev) {
   static std::mutex lock;
-  static cudaMemPool_t pools[MAX_DEVICES] = {};
-  if (dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
+  static std::map<int, cudaMemPool_t>& pools = *new std::map<int, cudaMemPool_t>;
   std::lock_guard<std::mutex> hold(lock);
-  if (!pools[dev]) {
+  if (!pools.count(dev)) {
     cudaMemPoolProps props = {};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
@@ -161,18 +160,17 @@ struct DevBuf {  // grow-only device array of the context's device
     const bool capturing = status != cudaStreamCaptureStatusNone;
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    BlockCache* cache = BlockCache::of(dev);
-    if (!cache) return cudaErrorInvalidDevice;
+    BlockCache& cache = BlockCache::of(dev);
     if (ptr && capturing) {
-      cache->put(ptr, false);
+      cache.put(ptr, false);
     } else if (ptr) {
       if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;  // any stream may still use the old array
-      cache->put(ptr);
+      cache.put(ptr);
     }
     ptr = nullptr;
     cap = 0;
     void* bigger = nullptr;
-    e = cache->get(&bigger, n * sizeof(T), capturing);
+    e = cache.get(&bigger, n * sizeof(T), capturing);
     if (e == cudaSuccess) {
       ptr = static_cast<T*>(bigger);
       cap = n;
@@ -180,7 +178,7 @@ struct DevBuf {  // grow-only device array of the context's device
     return e;
   }
   void release(int dev) {  // once the device has finished with it
-    if (ptr) BlockCache::of(dev)->put(ptr);
+    if (ptr) BlockCache::of(dev).put(ptr);
     ptr = nullptr;
     cap = 0;
   }

@@ -536,7 +536,7 @@ int headcast_destroy(headcast_ctx* c) {
   if (c->mono_v) cudaFreeAsync(c->mono_v, nullptr);
   void* ptrs[] = {c->arena_k, c->arena_v, c->sp_base, c->sp_nc, c->cells_dev, c->status_dev, c->dyn_counter_dev, c->move_boxes_dev};
   for (void* p : ptrs)
-    if (p) BlockCache::of(c->device)->put(p);
+    if (p) BlockCache::of(c->device).put(p);
   if (c->ev_a) cudaEventDestroy(c->ev_a);
   if (c->ev_b) cudaEventDestroy(c->ev_b);
   c->sched_dense.release(c->device);

@@ -1,0 +1,11 @@
+// The whole library on top of fake_cuda.cpp: host code only, no kernel ever runs.
+#include "../../paper_2607_20125_b200/csrc/headcast_api.cu"
+
+// What the last attention launch was given.
+static hc::AttnParams last_attn;
+
+extern "C" void fake_saw_launch(const char* name, void** args) {
+  if (std::strstr(name, "attn_kernel")) std::memcpy(&last_attn, args[0], sizeof(last_attn));
+}
+extern "C" void* fake_attn_part_o() { return last_attn.part_o; }
+extern "C" int fake_attn_radius() { return last_attn.radius; }

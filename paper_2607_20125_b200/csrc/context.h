@@ -32,7 +32,7 @@ enum { MAP_MONO = 0, MAP_SD = 1, MAP_GLOBAL = 2, MAP_SPATIAL = 3, N_MAP_PAIRS = 
 // with giving them back; with cudaMalloc and cudaFree that took half of the 14.8 ms from create to destroy (3.5 us per MB
 // and 55 us per small buffer each way), with blocks kept from the context before it takes 0.3 ms.  Per GPU at most
 // CACHE_KEEP_BYTES are kept, the blocks given back last; older ones go to the system then and there, all of them when an
-// allocation fails.  A block is given back only once the device has finished with it, so it may serve any stream.
+// allocation fails.  A block is kept only if the device has been waited for since its last use, so it may serve any stream.
 constexpr size_t CACHE_KEEP_BYTES = size_t(384) << 20;
 constexpr unsigned long long MONO_KEEP_BYTES = 256ull << 20;  // the same for the monolithic caches, see mono_alloc
 
@@ -67,23 +67,50 @@ class BlockCache {
     if (e == cudaSuccess) live_[*ptr] = need;
     return e;
   }
-  void put(void* ptr, bool keep = true) {  // the device has finished with it (keep: false: by cudaFree, which waits)
+  // Gives a block back.  idle: wait_idle() has returned true since its last use.  If not, the block goes through cudaFree,
+  // which waits itself, or refuses beside a stream capture: then it is set aside until the device can be waited for.
+  void put(void* ptr, bool idle) {
     std::lock_guard<std::mutex> hold(lock_);
     auto it = live_.find(ptr);
     if (it == live_.end()) return;
     const size_t bytes = it->second;
     live_.erase(it);
-    if (!keep || bytes > CACHE_KEEP_BYTES) {
-      cudaFree(ptr);
+    if (!idle || bytes > CACHE_KEEP_BYTES) {
+      give_up(ptr);
       return;
     }
     shrink(CACHE_KEEP_BYTES - bytes);
     free_.push_back({ptr, bytes});
     kept_ += bytes;
   }
+  // The same for memory of mono_alloc.  Its free is ordered by a stream and does not wait for the others.
+  void put_mono(void* ptr, bool idle) {
+    if (idle && cudaFreeAsync(ptr, nullptr) == cudaSuccess) return;
+    std::lock_guard<std::mutex> hold(lock_);
+    aside_.push_back(ptr);
+  }
+  // Waits for the device, which must be the current one.  False if the runtime refuses to (it does while any of the device's
+  // streams is under capture): work may then be in flight on any stream.
+  bool wait_idle() {
+    std::vector<void*> aside;  // not what is set aside while this waits
+    {
+      std::lock_guard<std::mutex> hold(lock_);
+      aside.swap(aside_);
+    }
+    const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+    std::lock_guard<std::mutex> hold(lock_);
+    if (idle)
+      for (void* ptr : aside) give_up(ptr);
+    else
+      aside_.insert(aside_.end(), aside.begin(), aside.end());
+    return idle;
+  }
 
  private:
   struct Block { void* ptr; size_t bytes; };
+  void give_up(void* ptr) {
+    if (cudaFree(ptr) != cudaSuccess) aside_.push_back(ptr);
+  }
   static size_t round_up(size_t bytes) {
     if (bytes > (size_t(1) << 20)) return (bytes + (size_t(2) << 20) - 1) >> 21 << 21;
     size_t r = 4096;
@@ -93,13 +120,14 @@ class BlockCache {
   void shrink(size_t to) {  // oldest first
     size_t n = 0;
     for (; n < free_.size() && kept_ > to; ++n) {
-      cudaFree(free_[n].ptr);
+      give_up(free_[n].ptr);
       kept_ -= free_[n].bytes;
     }
     free_.erase(free_.begin(), free_.begin() + n);
   }
   std::mutex lock_;
   std::vector<Block> free_;
+  std::vector<void*> aside_;  // given back while the device could not be waited for: belongs to nobody, handed to nobody
   std::map<void*, size_t> live_;
   size_t kept_ = 0;
 };
@@ -165,7 +193,7 @@ struct DevBuf {  // grow-only device array of the context's device
       cache.put(ptr, false);
     } else if (ptr) {
       if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;  // any stream may still use the old array
-      cache.put(ptr);
+      cache.put(ptr, true);
     }
     ptr = nullptr;
     cap = 0;
@@ -177,8 +205,8 @@ struct DevBuf {  // grow-only device array of the context's device
     }
     return e;
   }
-  void release(int dev) {  // once the device has finished with it
-    if (ptr) BlockCache::of(dev).put(ptr);
+  void release(BlockCache& cache, bool idle) {
+    if (ptr) cache.put(ptr, idle);
     ptr = nullptr;
     cap = 0;
   }
@@ -201,12 +229,12 @@ struct Schedule {
   int dyn_first = 0, dyn_end = 0;  // items [dyn_first, dyn_end) form the shared queue the CTAs draw from when their own list is done
   bool uploaded = false;
   double flops = 0.0;
-  void release(int dev) {
-    items_dev.release(dev);
-    cta_first_dev.release(dev);
-    combine_dev.release(dev);
-    cls_groups_dev.release(dev);
-    cls_parts_dev.release(dev);
+  void release(BlockCache& cache, bool idle) {
+    items_dev.release(cache, idle);
+    cta_first_dev.release(cache, idle);
+    combine_dev.release(cache, idle);
+    cls_groups_dev.release(cache, idle);
+    cls_parts_dev.release(cache, idle);
   }
 };
 

@@ -517,7 +517,7 @@ int headcast_create(const headcast_config* cfg, headcast_ctx** out) {
   int rc = HC_OK;
   if (e != cudaSuccess) rc = (e == cudaErrorMemoryAllocation) ? HC_ERR_NOMEM : HC_ERR_CUDA;
   if (rc == HC_OK) rc = build_maps(c);
-  if (rc == HC_OK && cudaDeviceSynchronize() != cudaSuccess) rc = HC_ERR_CUDA;
+  if (rc == HC_OK && !BlockCache::of(c->device).wait_idle()) rc = HC_ERR_CUDA;
   if (rc != HC_OK) {
     headcast_destroy(c);
     return rc;
@@ -531,36 +531,38 @@ int headcast_destroy(headcast_ctx* c) {
   int current = c->device;  // the context's memory belongs to its own device, whichever one is current now
   cudaGetDevice(&current);
   if (current != c->device) cudaSetDevice(c->device);
-  cudaDeviceSynchronize();
-  if (c->mono_k) cudaFreeAsync(c->mono_k, nullptr);
-  if (c->mono_v) cudaFreeAsync(c->mono_v, nullptr);
+  BlockCache& cache = BlockCache::of(c->device);
+  const bool idle = cache.wait_idle();  // if not, kernels may be at work on any of these: nothing of it is kept for others
+  if (c->mono_k) cache.put_mono(c->mono_k, idle);
+  if (c->mono_v) cache.put_mono(c->mono_v, idle);
   void* ptrs[] = {c->arena_k, c->arena_v, c->sp_base, c->sp_nc, c->cells_dev, c->status_dev, c->dyn_counter_dev, c->move_boxes_dev};
   for (void* p : ptrs)
-    if (p) BlockCache::of(c->device).put(p);
+    if (p) cache.put(p, idle);
   if (c->ev_a) cudaEventDestroy(c->ev_a);
   if (c->ev_b) cudaEventDestroy(c->ev_b);
-  c->sched_dense.release(c->device);
-  c->sched_hc.release(c->device);
-  c->sched_cls.release(c->device);
-  c->sched_proxy.release(c->device);
-  for (Schedule& g : c->sched_stage) g.release(c->device);
-  c->stage_q.release(c->device);
-  c->stage_out.release(c->device);
-  c->stage_k.release(c->device);
-  c->stage_v.release(c->device);
+  c->sched_dense.release(cache, idle);
+  c->sched_hc.release(cache, idle);
+  c->sched_cls.release(cache, idle);
+  c->sched_proxy.release(cache, idle);
+  for (Schedule& g : c->sched_stage) g.release(cache, idle);
+  c->stage_q.release(cache, idle);
+  c->stage_out.release(cache, idle);
+  c->stage_k.release(cache, idle);
+  c->stage_v.release(cache, idle);
   if (c->copy_in) cudaStreamDestroy(c->copy_in);
   if (c->copy_out) cudaStreamDestroy(c->copy_out);
   for (cudaEvent_t e : c->ev_host)
     if (e) cudaEventDestroy(e);
-  c->part_o.release(c->device);
-  c->part_ml.release(c->device);
-  c->part_mid.release(c->device);
-  c->trace_dev.release(c->device);
-  c->cls_o.release(c->device);
-  c->cls_lse.release(c->device);
-  c->cls_tok.release(c->device);
-  c->cls_scores.release(c->device);
-  c->cls_labels.release(c->device);
+  c->part_o.release(cache, idle);
+  c->part_ml.release(cache, idle);
+  c->part_mid.release(cache, idle);
+  c->trace_dev.release(cache, idle);
+  c->cls_o.release(cache, idle);
+  c->cls_lse.release(cache, idle);
+  c->cls_tok.release(cache, idle);
+  c->cls_scores.release(cache, idle);
+  c->cls_labels.release(cache, idle);
+  if (!idle) cudaGetLastError();  // the refusal is dealt with, no later call is to report it
   if (current != c->device) cudaSetDevice(current);
   delete c;
   return HC_OK;

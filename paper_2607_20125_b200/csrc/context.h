@@ -31,10 +31,10 @@ enum { MAP_MONO = 0, MAP_SD = 1, MAP_GLOBAL = 2, MAP_SPATIAL = 3, N_MAP_PAIRS = 
 // Device memory of the contexts.  A layer's life starts with about thirty allocations, 400 MB at 30 x 52 tokens, and ends
 // with giving them back; with cudaMalloc and cudaFree that took half of the 14.8 ms from create to destroy (3.5 us per MB
 // and 55 us per small buffer each way), with blocks kept from the context before it takes 0.3 ms.  Per GPU at most
-// CACHE_KEEP_BYTES are kept, the blocks given back last; older ones go to the system then and there, all of them when an
-// allocation fails.  A block is kept only if the device has been waited for since its last use, so it may serve any stream.
+// CACHE_KEEP_BYTES are kept, the blocks given back last; older ones go to the system then and there, all of them and what
+// the pool holds unused when an allocation of either kind fails.  A block is kept only if the device has been waited for since its last use, so it may serve any stream.
 constexpr size_t CACHE_KEEP_BYTES = size_t(384) << 20;
-constexpr unsigned long long MONO_KEEP_BYTES = 256ull << 20;  // the same for the monolithic caches, see mono_alloc
+constexpr unsigned long long MONO_KEEP_BYTES = 256ull << 20;  // the same for the monolithic caches, see get_mono
 
 class BlockCache {
  public:
@@ -59,9 +59,8 @@ class BlockCache {
       return cudaSuccess;
     }
     cudaError_t e = cudaMalloc(ptr, need);
-    if (e == cudaErrorMemoryAllocation && !free_.empty() && !fresh) {  // what is kept here may be what is missing
-      cudaGetLastError();
-      shrink(0);
+    if (e == cudaErrorMemoryAllocation) {
+      release_all();
       e = cudaMalloc(ptr, need);
     }
     if (e == cudaSuccess) live_[*ptr] = need;
@@ -83,7 +82,21 @@ class BlockCache {
     free_.push_back({ptr, bytes});
     kept_ += bytes;
   }
-  // The same for memory of mono_alloc.  Its free is ordered by a stream and does not wait for the others.
+  // The monolithic cache is released in the middle of a stream's work (at the split), so it comes from a stream-ordered pool
+  // of its own instead of a block; the pool keeps at most MONO_KEEP_BYTES unused (the default pool keeps nothing: 2.8 ms per
+  // 200 MB to map and unmap them again) and hands memory out again only once the work that used it has completed.
+  cudaError_t get_mono(void** ptr, size_t bytes, int dev) {
+    std::lock_guard<std::mutex> hold(lock_);
+    cudaError_t e = pool_ ? cudaSuccess : make_pool(dev);
+    if (e != cudaSuccess) return e;
+    e = cudaMallocFromPoolAsync(ptr, bytes, pool_, nullptr);
+    if (e == cudaErrorMemoryAllocation) {
+      release_all();
+      e = cudaMallocFromPoolAsync(ptr, bytes, pool_, nullptr);
+    }
+    return e;
+  }
+  // The same for memory of get_mono.  Its free is ordered by a stream and does not wait for the others.
   void put_mono(void* ptr, bool idle) {
     if (idle && cudaFreeAsync(ptr, nullptr) == cudaSuccess) return;
     std::lock_guard<std::mutex> hold(lock_);
@@ -108,6 +121,32 @@ class BlockCache {
 
  private:
   struct Block { void* ptr; size_t bytes; };
+  // What is kept here, of either kind, may be what is missing.
+  void release_all() {
+    cudaGetLastError();
+    shrink(0);
+    if (pool_) cudaMemPoolTrimTo(pool_, 0);
+  }
+  cudaError_t make_pool(int dev) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool;
+    cudaError_t e = cudaMemPoolCreate(&pool, &props);
+    if (e != cudaSuccess) return e;
+    unsigned long long keep = MONO_KEEP_BYTES;
+    int off = 0;
+    e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolReuseFollowEventDependencies, &off);
+    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &off);
+    if (e != cudaSuccess) {
+      cudaMemPoolDestroy(pool);
+      return e;
+    }
+    pool_ = pool;
+    return cudaSuccess;
+  }
   void give_up(void* ptr) {
     if (cudaFree(ptr) != cudaSuccess) aside_.push_back(ptr);
   }
@@ -130,48 +169,14 @@ class BlockCache {
   std::vector<void*> aside_;  // given back while the device could not be waited for: belongs to nobody, handed to nobody
   std::map<void*, size_t> live_;
   size_t kept_ = 0;
+  cudaMemPool_t pool_ = nullptr;
 };
 
-cudaError_t block_alloc(void** ptr, size_t bytes) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  return BlockCache::of(dev).get(ptr, bytes);
-}
-
-// The monolithic cache is released in the middle of a stream's work (at the split), so it comes from a stream-ordered pool
-// of its own instead of a block; the pool keeps at most MONO_KEEP_BYTES unused (the default pool keeps nothing: 2.8 ms per
-// 200 MB to map and unmap them again) and hands memory out again only once the work that used it has completed.
-cudaError_t mono_alloc(void** ptr, size_t bytes, int dev) {
-  static std::mutex lock;
-  static std::map<int, cudaMemPool_t>& pools = *new std::map<int, cudaMemPool_t>;
-  std::lock_guard<std::mutex> hold(lock);
-  if (!pools.count(dev)) {
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    cudaMemPool_t pool;
-    cudaError_t e = cudaMemPoolCreate(&pool, &props);
-    if (e != cudaSuccess) return e;
-    unsigned long long keep = MONO_KEEP_BYTES;
-    int off = 0;
-    e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolReuseFollowEventDependencies, &off);
-    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &off);
-    if (e != cudaSuccess) {
-      cudaMemPoolDestroy(pool);
-      return e;
-    }
-    pools[dev] = pool;
-  }
-  cudaError_t e = cudaMallocFromPoolAsync(ptr, bytes, pools[dev], nullptr);
-  if (e == cudaErrorMemoryAllocation) {
-    cudaGetLastError();
-    cudaDeviceSynchronize();
-    cudaMemPoolTrimTo(pools[dev], 0);
-    e = cudaMallocFromPoolAsync(ptr, bytes, pools[dev], nullptr);
-  }
+// `take`, and once more after waiting for the device if memory runs out: what is still on its way back counts then.
+template <typename F>
+cudaError_t take_or_wait(BlockCache& cache, F take) {
+  cudaError_t e = take();
+  if (e == cudaErrorMemoryAllocation && cache.wait_idle()) e = take();
   return e;
 }
 

@@ -480,15 +480,21 @@ int headcast_create(const headcast_config* cfg, headcast_ctx** out) {
     return HC_ERR_UNSUPPORTED;
   }
   const size_t mono_bytes = cache_elems(c, c->H) * sizeof(__nv_bfloat16);
+  BlockCache& cache = BlockCache::of(c->device);
   cudaError_t e = cudaSuccess;
   auto step = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
   auto get = [&](auto** ptr, size_t bytes) {
     void* m = nullptr;
-    if (e == cudaSuccess) step(block_alloc(&m, bytes));
+    if (e == cudaSuccess) step(take_or_wait(cache, [&] { return cache.get(&m, bytes); }));
     *ptr = static_cast<std::remove_pointer_t<decltype(ptr)>>(m);
   };
-  if (e == cudaSuccess) step(mono_alloc(reinterpret_cast<void**>(&c->mono_k), mono_bytes, c->device));
-  if (e == cudaSuccess) step(mono_alloc(reinterpret_cast<void**>(&c->mono_v), mono_bytes, c->device));
+  auto get_mono = [&](__nv_bfloat16** ptr) {
+    void* m = nullptr;
+    if (e == cudaSuccess) step(take_or_wait(cache, [&] { return cache.get_mono(&m, mono_bytes, c->device); }));
+    *ptr = static_cast<__nv_bfloat16*>(m);
+  };
+  get_mono(&c->mono_k);
+  get_mono(&c->mono_v);
   get(&c->arena_k, mono_bytes);
   get(&c->arena_v, mono_bytes);
   get(&c->sp_base, c->T_f * sizeof(int32_t));
@@ -517,7 +523,7 @@ int headcast_create(const headcast_config* cfg, headcast_ctx** out) {
   int rc = HC_OK;
   if (e != cudaSuccess) rc = (e == cudaErrorMemoryAllocation) ? HC_ERR_NOMEM : HC_ERR_CUDA;
   if (rc == HC_OK) rc = build_maps(c);
-  if (rc == HC_OK && !BlockCache::of(c->device).wait_idle()) rc = HC_ERR_CUDA;
+  if (rc == HC_OK && !cache.wait_idle()) rc = HC_ERR_CUDA;
   if (rc != HC_OK) {
     headcast_destroy(c);
     return rc;

@@ -47,3 +47,34 @@ def test_memory_that_could_not_be_freed_is_freed_once_the_device_can_be_waited_f
         again = fake.context(**TINY)
         assert again.append(2) == 0 and again.full_attend() == 0 and again.destroy() == 0
     assert fake.used() - fake.pool_unused() <= whole  # (the pool gives back by itself what exceeds its bound)
+
+
+@pytest.mark.parametrize("idle_blocks,heads", [(False, 5), (False, 16), (True, 5), (True, 16)])
+def test_creation_takes_back_all_that_the_library_keeps_idle(fake, idle_blocks, heads):
+    wanted = dict(TINY, n_heads=heads)  # 5: memory runs out at its monolithic cache, 16: later, at its blocks
+    clean = FakeLibrary()
+    need = clean.context(**wanted) and clean.used()
+    contexts = [fake.context(**TINY) for _ in range(3)]
+    for ctx in contexts:
+        if idle_blocks:  # blocks, scratch arrays among them, and the monolithic cache in the pool
+            assert ctx.append(2) == 0 and ctx.full_attend() == 0 and ctx.destroy() == 0
+        else:  # the monolithic cache only, the blocks are in use
+            assert ctx.append() == 0 and ctx.split([0, 1, 2, 3]) == 0
+    idle = fake.used() if idle_blocks else fake.pool_unused()
+    assert idle > fake.pool_unused() > 0 if idle_blocks else idle > 0
+    fake.capacity_left(need - idle)  # every idle byte has to come back for this one to fit
+    assert fake.context(**wanted).rc == 0
+
+
+def test_a_growing_scratch_array_takes_back_the_pools_idle_memory(fake):
+    ctx = fake.context(**TINY)
+    gone = fake.context(**TINY)
+    assert ctx.append(2) == 0 and gone.append() == 0 and gone.split([0, 1, 2, 3]) == 0
+    assert fake.pool_unused() > 0
+    clean = FakeLibrary()
+    twin = clean.context(**TINY)
+    twin.append(2)
+    before = clean.used()
+    assert twin.full_attend() == 0
+    fake.capacity_left(max(0, clean.used() - before - fake.pool_unused()))
+    assert ctx.full_attend() == 0

@@ -44,8 +44,8 @@ class BlockCache {
     std::lock_guard<std::mutex> hold(lock);
     return all[dev];
   }
-  // On the current device, which must be this cache's.  `fresh`: by cudaMalloc, whatever is kept here.
-  cudaError_t get(void** ptr, size_t bytes, bool fresh = false) {
+  // On the current device, which must be this cache's.  *got: the block's size.  `fresh`: by cudaMalloc, whatever is kept here.
+  cudaError_t get(void** ptr, size_t bytes, size_t* got = nullptr, bool fresh = false) {
     const size_t need = round_up(bytes);
     std::lock_guard<std::mutex> hold(lock_);
     size_t at = free_.size();
@@ -54,6 +54,7 @@ class BlockCache {
     if (at < free_.size()) {
       *ptr = free_[at].ptr;
       live_[*ptr] = free_[at].bytes;
+      if (got) *got = free_[at].bytes;
       kept_ -= free_[at].bytes;
       free_.erase(free_.begin() + at);
       return cudaSuccess;
@@ -64,6 +65,7 @@ class BlockCache {
       e = cudaMalloc(ptr, need);
     }
     if (e == cudaSuccess) live_[*ptr] = need;
+    if (got) *got = need;
     return e;
   }
   // Gives a block back.  idle: wait_idle() has returned true since its last use.  If not, the block goes through cudaFree,
@@ -190,23 +192,20 @@ struct DevBuf {  // grow-only device array of the context's device
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &status);
     if (e != cudaSuccess) return e;
-    const bool capturing = status != cudaStreamCaptureStatusNone;
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     BlockCache& cache = BlockCache::of(dev);
-    if (ptr && capturing) {
-      cache.put(ptr, false);
-    } else if (ptr) {
-      if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;  // any stream may still use the old array
-      cache.put(ptr, true);
-    }
+    // Any stream may still use the old array.  cudaFree waits for them; a device synchronisation, with which the array could
+    // be kept, would be refused beside a capture on whatever stream and destroy that capture.
+    if (ptr) cache.put(ptr, false);
     ptr = nullptr;
     cap = 0;
     void* bigger = nullptr;
-    e = cache.get(&bigger, n * sizeof(T), capturing);
+    size_t bytes = 0;
+    e = cache.get(&bigger, n * sizeof(T), &bytes, status != cudaStreamCaptureStatusNone);
     if (e == cudaSuccess) {
       ptr = static_cast<T*>(bigger);
-      cap = n;
+      cap = bytes / sizeof(T);
     }
     return e;
   }

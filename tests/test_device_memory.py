@@ -78,3 +78,13 @@ def test_a_growing_scratch_array_takes_back_the_pools_idle_memory(fake):
     assert twin.full_attend() == 0
     fake.capacity_left(max(0, clean.used() - before - fake.pool_unused()))
     assert ctx.full_attend() == 0
+
+
+def test_scratch_may_grow_beside_the_capture_of_another_stream(fake):
+    ctx = fake.context(**TINY)
+    assert ctx.append(1) == 0 and ctx.full_attend() == 0
+    first = fake.attn_part_o()
+    fake.capture(RELAXED, 77)
+    assert ctx.append(3) == 0 and ctx.full_attend(stream=78) == 0
+    assert fake.attn_part_o() != first and fake.is_live(fake.attn_part_o())
+    assert not fake.capture_invalidated()

@@ -195,20 +195,24 @@ struct DevBuf {  // grow-only device array of the context's device
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     BlockCache& cache = BlockCache::of(dev);
-    // Any stream may still use the old array.  cudaFree waits for them; a device synchronisation, with which the array could
-    // be kept, would be refused beside a capture on whatever stream and destroy that capture.
-    if (ptr) cache.put(ptr, false);
-    ptr = nullptr;
-    cap = 0;
+    const bool capturing = status != cudaStreamCaptureStatusNone;
     void* bigger = nullptr;
     size_t bytes = 0;
-    e = cache.get(&bigger, n * sizeof(T), &bytes, status != cudaStreamCaptureStatusNone);
+    e = cache.get(&bigger, n * sizeof(T), &bytes, capturing);
+    if (e == cudaErrorMemoryAllocation && ptr) {  // no room for both: the old one first
+      give_back(cache);
+      e = cache.get(&bigger, n * sizeof(T), &bytes, capturing);
+    }
     if (e == cudaSuccess) {
+      give_back(cache);
       ptr = static_cast<T*>(bigger);
       cap = bytes / sizeof(T);
     }
     return e;
   }
+  // Any stream may still use the array.  cudaFree waits for them; a device synchronisation, with which the memory could be
+  // kept, would be refused beside a capture on whatever stream and destroy that capture.
+  void give_back(BlockCache& cache) { release(cache, false); }
   void release(BlockCache& cache, bool idle) {
     if (ptr) cache.put(ptr, idle);
     ptr = nullptr;

@@ -25,6 +25,13 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 }
 
 int upload_schedule(headcast_ctx* c, Schedule& s, cudaStream_t st) {
+  // The partial results are shared by all lists of the context, so every launch makes sure of them and not only the first of
+  // its list: another list's growth may have failed in between and left none.
+  if (s.n_slots > 0) {
+    HC_CUDA(c, c->part_o.reserve(static_cast<size_t>(s.n_slots) * 256 * c->D, st));
+    HC_CUDA(c, c->part_ml.reserve(static_cast<size_t>(s.n_slots) * 256, st));
+    HC_CUDA(c, c->part_mid.reserve(static_cast<size_t>(s.n_slots) * 256, st));
+  }
   if (s.uploaded) return HC_OK;
   HC_CUDA(c, s.items_dev.reserve(std::max<size_t>(1, s.items.size()), st));
   HC_CUDA(c, s.cta_first_dev.reserve(s.cta_first.size(), st));
@@ -44,11 +51,6 @@ int upload_schedule(headcast_ctx* c, Schedule& s, cudaStream_t st) {
                                cudaMemcpyHostToDevice, st));
     HC_CUDA(c, cudaMemcpyAsync(s.cls_parts_dev.ptr, s.cls_parts.data(), s.cls_parts.size() * sizeof(ClsPart),
                                cudaMemcpyHostToDevice, st));
-  }
-  if (s.n_slots > 0) {
-    HC_CUDA(c, c->part_o.reserve(static_cast<size_t>(s.n_slots) * 256 * c->D, st));
-    HC_CUDA(c, c->part_ml.reserve(static_cast<size_t>(s.n_slots) * 256, st));
-    HC_CUDA(c, c->part_mid.reserve(static_cast<size_t>(s.n_slots) * 256, st));
   }
   // The lists are uploaded once per cache fill and reused by later calls, which may come on another stream: wait
   // here, once, so that no later launch can see a half-written list (the host vectors are pageable, so the copies

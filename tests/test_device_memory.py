@@ -88,3 +88,20 @@ def test_scratch_may_grow_beside_the_capture_of_another_stream(fake):
     assert ctx.append(3) == 0 and ctx.full_attend(stream=78) == 0
     assert fake.attn_part_o() != first and fake.is_live(fake.attn_part_o())
     assert not fake.capture_invalidated()
+
+
+@pytest.mark.parametrize("refusal", ["memory", "capture"])
+def test_a_list_that_is_already_uploaded_has_its_scratch_after_anothers_growth_failed(fake, refusal):
+    ctx = fake.context(n_heads=6, head_dim=128, grid_h=13, grid_w=22, n_blocks=4, cell_h=6, cell_w=6, keep_monolithic=1)
+    assert ctx.append(4) == 0 and ctx.split([0, 1, 2, 3, 2, 3]) == 0 and ctx.attend() == 0
+    first = fake.attn_part_o()
+    if refusal == "memory":
+        fake.capacity_left(64 << 10)  # enough for the dense list, not for its partial results
+        assert ctx.full_attend() == -4
+    else:
+        fake.capture(GLOBAL_MODE, 77)
+        assert ctx.full_attend(stream=78) != 0
+        fake.capture(0, None)
+    assert ctx.attend() == 0
+    assert fake.is_live(fake.attn_part_o())
+    assert refusal == "memory" or fake.attn_part_o() == first

@@ -32,17 +32,22 @@ enum { MAP_MONO = 0, MAP_SD = 1, MAP_GLOBAL = 2, MAP_SPATIAL = 3, N_MAP_PAIRS = 
 // with giving them back; with cudaMalloc and cudaFree that took half of the 14.8 ms from create to destroy (3.5 us per MB
 // and 55 us per small buffer each way), with blocks kept from the context before it takes 0.3 ms.  Per GPU at most
 // CACHE_KEEP_BYTES are kept, the blocks given back last; older ones go to the system then and there, all of them and what
-// the pool holds unused when an allocation of either kind fails.  A block is kept only if the device has been waited for since its last use, so it may serve any stream.
+// the pool holds unused when an allocation of either kind fails.  A block is kept only if the device has been waited for
+// since its last use, so it may serve any stream.
 constexpr size_t CACHE_KEEP_BYTES = size_t(384) << 20;
 constexpr unsigned long long MONO_KEEP_BYTES = 256ull << 20;  // the same for the monolithic caches, see get_mono
 
 class BlockCache {
  public:
-  static BlockCache& of(int dev) {
+  // The cache of the current device, more exactly of the CUDA context that is current on it: after a device reset, or in
+  // another context that a host made through the driver, an older context's memory must not come back.  nullptr: no context.
+  static BlockCache* current(int dev) {
+    unsigned long long id = 0;
+    if (cudaFree(nullptr) != cudaSuccess || !current_context_id(&id)) return nullptr;
     static std::mutex lock;
-    static std::map<int, BlockCache>& all = *new std::map<int, BlockCache>;  // never destroyed: a context may outlive static objects
+    static auto& all = *new std::map<std::pair<int, unsigned long long>, BlockCache>;  // never destroyed: a context may outlive static objects
     std::lock_guard<std::mutex> hold(lock);
-    return all[dev];
+    return &all[std::make_pair(dev, id)];
   }
   // On the current device, which must be this cache's.  *got: the block's size.  `fresh`: by cudaMalloc, whatever is kept here.
   cudaError_t get(void** ptr, size_t bytes, size_t* got = nullptr, bool fresh = false) {
@@ -186,15 +191,12 @@ template <typename T>
 struct DevBuf {  // grow-only device array of the context's device
   T* ptr = nullptr;
   size_t cap = 0;
-  cudaError_t reserve(size_t n, cudaStream_t st) {
+  cudaError_t reserve(BlockCache& cache, size_t n, cudaStream_t st) {
     if (n <= cap) return cudaSuccess;
     // while `st` is captured the cache stands aside: cudaMalloc then says whether memory may be taken in this capture mode
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &status);
     if (e != cudaSuccess) return e;
-    int dev = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    BlockCache& cache = BlockCache::of(dev);
     const bool capturing = status != cudaStreamCaptureStatusNone;
     void* bigger = nullptr;
     size_t bytes = 0;
@@ -300,6 +302,7 @@ struct headcast_ctx {
   DevBuf<int32_t> cls_labels;
 
   int device = 0;
+  BlockCache* memory = nullptr;  // where the device memory of this context comes from
   int n_sm = 148;
   int64_t launches = 0;
   bool tracing = false;  // record per-item start/end times in the attention kernel

@@ -28,14 +28,14 @@ int upload_schedule(headcast_ctx* c, Schedule& s, cudaStream_t st) {
   // The partial results are shared by all lists of the context, so every launch makes sure of them and not only the first of
   // its list: another list's growth may have failed in between and left none.
   if (s.n_slots > 0) {
-    HC_CUDA(c, c->part_o.reserve(static_cast<size_t>(s.n_slots) * 256 * c->D, st));
-    HC_CUDA(c, c->part_ml.reserve(static_cast<size_t>(s.n_slots) * 256, st));
-    HC_CUDA(c, c->part_mid.reserve(static_cast<size_t>(s.n_slots) * 256, st));
+    HC_CUDA(c, c->part_o.reserve(*c->memory, static_cast<size_t>(s.n_slots) * 256 * c->D, st));
+    HC_CUDA(c, c->part_ml.reserve(*c->memory, static_cast<size_t>(s.n_slots) * 256, st));
+    HC_CUDA(c, c->part_mid.reserve(*c->memory, static_cast<size_t>(s.n_slots) * 256, st));
   }
   if (s.uploaded) return HC_OK;
-  HC_CUDA(c, s.items_dev.reserve(std::max<size_t>(1, s.items.size()), st));
-  HC_CUDA(c, s.cta_first_dev.reserve(s.cta_first.size(), st));
-  HC_CUDA(c, s.combine_dev.reserve(std::max<size_t>(1, s.combine.size()), st));
+  HC_CUDA(c, s.items_dev.reserve(*c->memory, std::max<size_t>(1, s.items.size()), st));
+  HC_CUDA(c, s.cta_first_dev.reserve(*c->memory, s.cta_first.size(), st));
+  HC_CUDA(c, s.combine_dev.reserve(*c->memory, std::max<size_t>(1, s.combine.size()), st));
   if (!s.items.empty())
     HC_CUDA(c, cudaMemcpyAsync(s.items_dev.ptr, s.items.data(), s.items.size() * sizeof(WorkItem),
                                cudaMemcpyHostToDevice, st));
@@ -45,8 +45,8 @@ int upload_schedule(headcast_ctx* c, Schedule& s, cudaStream_t st) {
     HC_CUDA(c, cudaMemcpyAsync(s.combine_dev.ptr, s.combine.data(), s.combine.size() * sizeof(CombineEntry),
                                cudaMemcpyHostToDevice, st));
   if (!s.cls_groups.empty()) {
-    HC_CUDA(c, s.cls_groups_dev.reserve(s.cls_groups.size(), st));
-    HC_CUDA(c, s.cls_parts_dev.reserve(std::max<size_t>(1, s.cls_parts.size()), st));
+    HC_CUDA(c, s.cls_groups_dev.reserve(*c->memory, s.cls_groups.size(), st));
+    HC_CUDA(c, s.cls_parts_dev.reserve(*c->memory, std::max<size_t>(1, s.cls_parts.size()), st));
     HC_CUDA(c, cudaMemcpyAsync(s.cls_groups_dev.ptr, s.cls_groups.data(), s.cls_groups.size() * sizeof(ClsGroup),
                                cudaMemcpyHostToDevice, st));
     HC_CUDA(c, cudaMemcpyAsync(s.cls_parts_dev.ptr, s.cls_parts.data(), s.cls_parts.size() * sizeof(ClsPart),
@@ -110,7 +110,7 @@ int run_schedule(headcast_ctx* c, Schedule& s, const void* q, void* out, bool pr
   p.trace = nullptr;
   if (c->tracing) {
     const size_t trace_words = 2 * s.items.size();
-    HC_CUDA(c, c->trace_dev.reserve(trace_words, st));
+    HC_CUDA(c, c->trace_dev.reserve(*c->memory, trace_words, st));
     HC_CUDA(c, cudaMemsetAsync(c->trace_dev.ptr, 0, trace_words * sizeof(unsigned long long), st));
     p.trace = c->trace_dev.ptr;
     c->trace_items = s.items;
@@ -482,7 +482,12 @@ int headcast_create(const headcast_config* cfg, headcast_ctx** out) {
     return HC_ERR_UNSUPPORTED;
   }
   const size_t mono_bytes = cache_elems(c, c->H) * sizeof(__nv_bfloat16);
-  BlockCache& cache = BlockCache::of(c->device);
+  c->memory = BlockCache::current(c->device);
+  if (!c->memory) {
+    delete c;
+    return HC_ERR_CUDA;
+  }
+  BlockCache& cache = *c->memory;
   cudaError_t e = cudaSuccess;
   auto step = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
   auto get = [&](auto** ptr, size_t bytes) {
@@ -539,7 +544,7 @@ int headcast_destroy(headcast_ctx* c) {
   int current = c->device;  // the context's memory belongs to its own device, whichever one is current now
   cudaGetDevice(&current);
   if (current != c->device) cudaSetDevice(c->device);
-  BlockCache& cache = BlockCache::of(c->device);
+  BlockCache& cache = *c->memory;
   const bool idle = cache.wait_idle();  // if not, kernels may be at work on any of these: nothing of it is kept for others
   if (c->mono_k) cache.put_mono(c->mono_k, idle);
   if (c->mono_v) cache.put_mono(c->mono_v, idle);
@@ -666,11 +671,11 @@ int headcast_classify(headcast_ctx* c, const void* q, int32_t* labels_host, floa
   if (n_filled(c) < 2) return fail(c, HC_ERR_STATE, "classification needs at least two cached blocks");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t rows = static_cast<size_t>(c->L) * c->H;
-  HC_CUDA(c, c->cls_o.reserve(rows * c->D, st));  // the reference output (fp32); the proxy outputs never leave registers
-  HC_CUDA(c, c->cls_lse.reserve(rows, st));
-  HC_CUDA(c, c->cls_tok.reserve(TOK_N * rows, st));
-  HC_CUDA(c, c->cls_scores.reserve(static_cast<size_t>(c->H) * HC_N_SCORES, st));
-  HC_CUDA(c, c->cls_labels.reserve(c->H, st));
+  HC_CUDA(c, c->cls_o.reserve(*c->memory, rows * c->D, st));  // the reference output (fp32); the proxy outputs never leave registers
+  HC_CUDA(c, c->cls_lse.reserve(*c->memory, rows, st));
+  HC_CUDA(c, c->cls_tok.reserve(*c->memory, TOK_N * rows, st));
+  HC_CUDA(c, c->cls_scores.reserve(*c->memory, static_cast<size_t>(c->H) * HC_N_SCORES, st));
+  HC_CUDA(c, c->cls_labels.reserve(*c->memory, c->H, st));
   const int newest = c->slots.back();
   const int cls_key = n_filled(c) * 64 + newest;  // the work lists depend on the fill and on where the newest block sits
   if (c->sched_cls.key_filled != cls_key) {
@@ -885,8 +890,8 @@ int headcast_append_host(headcast_ctx* c, const void* k_host, const void* v_host
   if (!c || !k_host || !v_host) return HC_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t elems = static_cast<size_t>(c->L) * c->H * c->D;
-  HC_CUDA(c, c->stage_k.reserve(elems, st));
-  HC_CUDA(c, c->stage_v.reserve(elems, st));
+  HC_CUDA(c, c->stage_k.reserve(*c->memory, elems, st));
+  HC_CUDA(c, c->stage_v.reserve(*c->memory, elems, st));
   HC_CUDA(c, cudaMemcpyAsync(c->stage_k.ptr, k_host, elems * sizeof(__nv_bfloat16), cudaMemcpyHostToDevice, st));
   HC_CUDA(c, cudaMemcpyAsync(c->stage_v.ptr, v_host, elems * sizeof(__nv_bfloat16), cudaMemcpyHostToDevice, st));
   return headcast_append(c, c->stage_k.ptr, c->stage_v.ptr, stream);
@@ -899,8 +904,8 @@ int headcast_attend_host(headcast_ctx* c, const void* q_host, void* out_host, vo
   int rc = init_host_path(c);
   if (rc != HC_OK) return rc;
   const size_t elems = static_cast<size_t>(c->L) * c->H * c->D;
-  HC_CUDA(c, c->stage_q.reserve(elems, st));
-  HC_CUDA(c, c->stage_out.reserve(elems, st));
+  HC_CUDA(c, c->stage_q.reserve(*c->memory, elems, st));
+  HC_CUDA(c, c->stage_out.reserve(*c->memory, elems, st));
   const int key = n_filled(c) * 4 + c->sd_valid;
   // Stages: a stage's queries are copied in (strided: the rows of [L][H][d] hold all heads), attended and copied out
   // as a unit, so that the next stage's queries arrive and the previous stage's outputs leave while this stage

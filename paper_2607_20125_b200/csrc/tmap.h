@@ -1,5 +1,5 @@
-// Host-side construction of TMA tensor maps without linking libcuda: the driver's encode function
-// is looked up through the CUDA runtime at first use.
+// The driver's functions that this library needs - construction of TMA tensor maps, the number of a CUDA context - without
+// linking libcuda: they are looked up through the CUDA runtime at first use.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -21,6 +21,19 @@ inline EncodeTiledFn get_encode_tiled() {
     return nullptr;
   fn = reinterpret_cast<EncodeTiledFn>(p);
   return fn;
+}
+
+// A number of its own for every CUDA context of the process, also for the one that follows a device reset.
+inline bool current_context_id(unsigned long long* id) {
+  typedef CUresult (*GetIdFn)(CUcontext, unsigned long long*);
+  static GetIdFn fn = nullptr;
+  if (!fn) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) return false;
+    fn = reinterpret_cast<GetIdFn>(p);
+  }
+  return fn(nullptr, id) == CUDA_SUCCESS;
 }
 
 // 2-D bf16 tensor [rows][row_elems] (row pitch = pitch_elems), box = 64 columns x box_rows rows,

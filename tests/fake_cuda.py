@@ -17,7 +17,7 @@ RELAXED, GLOBAL_MODE = 1, 2  # capture modes
 def _built():
     folder = tempfile.TemporaryDirectory()
     lib = os.path.join(folder.name, "fake.so")
-    cmd = [os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-cudart", "none", "-shared", "-Xcompiler", "-fPIC", "-Xlinker", "-Bsymbolic",
+    cmd = [os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-cudart", "none", "-shared", "-Xcompiler", "-fPIC,-fno-gnu-unique", "-Xlinker", "-Bsymbolic",
            "-gencode", "arch=compute_100a,code=sm_100a", "-Xptxas", "-O0", "-std=c++17", "-o", lib,
            os.path.join(NATIVE, "headcast_on_fake_cuda.cu"), os.path.join(NATIVE, "fake_cuda.cpp")]
     res = subprocess.run(cmd, capture_output=True, text=True)
@@ -32,7 +32,7 @@ class FakeLibrary:
         os.close(handle)
         shutil.copy(lib, path)
         self.lib = binding.load_library(path)
-        for name in ("fake_used", "fake_pool_unused", "fake_busy", "fake_busy_writes"):
+        for name in ("fake_used", "fake_pool_unused", "fake_busy", "fake_busy_writes", "fake_stray_writes"):
             getattr(self.lib, name).restype = C.c_longlong
         self.lib.fake_capacity_left.argtypes = [C.c_longlong]
         self.lib.fake_capture.argtypes = [C.c_int, C.c_void_p]

@@ -22,6 +22,7 @@ struct Fake {
   std::multimap<size_t, char*> pool;           // freed to the pool, still reserved
   std::map<char*, size_t> busy;                // memory that work in flight still touches
   long long busy_writes = 0;                   // host-ordered writes into it: somebody was handed memory in use
+  long long stray_writes = 0;                  // writes to what is no device memory
   int device = 0;
   int capture = 0;                             // of another or of capture_stream: 0 none, 1 relaxed, 2 global
   cudaStream_t capture_stream = nullptr;
@@ -43,10 +44,16 @@ cudaError_t refused() {
 
 void finish() { fake().busy.clear(); }
 
-void write_to(const void* p) {
-  char* c = static_cast<char*>(const_cast<void*>(p));
-  auto it = fake().busy.upper_bound(c);
-  if (it != fake().busy.begin() && c < (--it)->first + it->second) ++fake().busy_writes;
+bool inside(const std::map<char*, size_t>& blocks, char* c) {
+  auto it = blocks.upper_bound(c);
+  return it != blocks.begin() && c < (--it)->first + it->second;
+}
+
+bool write_to(void* p) {  // by the device
+  if (inside(fake().busy, static_cast<char*>(p))) ++fake().busy_writes;
+  if (inside(fake().live, static_cast<char*>(p))) return true;
+  ++fake().stray_writes;
+  return false;
 }
 
 cudaError_t take(void** p, size_t bytes) {
@@ -88,7 +95,7 @@ void fake_reset() {
   fake().capture_stream = nullptr;
   fake().invalidated = false;
   fake().busy.clear();
-  fake().busy_writes = 0;
+  fake().busy_writes = fake().stray_writes = 0;
   fake().log.clear();
 }
 void fake_capacity_left(long long bytes) { fake().capacity = fake().used + bytes; }
@@ -96,6 +103,7 @@ long long fake_used() { return fake().used; }
 long long fake_pool_unused() { return fake().pool_unused; }
 void fake_work_in_flight() { fake().busy = fake().live; }
 long long fake_busy() { return static_cast<long long>(fake().busy.size()); }
+long long fake_stray_writes() { return fake().stray_writes; }
 long long fake_busy_writes() { return fake().busy_writes; }
 void fake_capture(int mode, void* stream) {
   fake().capture = mode;
@@ -170,19 +178,17 @@ cudaError_t cudaFreeAsync(void* p, cudaStream_t) {
   to_pool(static_cast<char*>(p));
   return cudaSuccess;
 }
-cudaError_t cudaMemcpy(void* dst, const void* src, size_t n, cudaMemcpyKind) {
-  write_to(dst);
-  std::memcpy(dst, src, n);
+cudaError_t cudaMemcpy(void* dst, const void* src, size_t n, cudaMemcpyKind kind) {
+  if (kind == cudaMemcpyDeviceToHost || write_to(dst)) std::memcpy(dst, src, n);
   return cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void* dst, const void* src, size_t n, cudaMemcpyKind k, cudaStream_t) { return cudaMemcpy(dst, src, n, k); }
-cudaError_t cudaMemcpy2DAsync(void* dst, size_t, const void*, size_t, size_t, size_t, cudaMemcpyKind, cudaStream_t) {
-  write_to(dst);
+cudaError_t cudaMemcpy2DAsync(void* dst, size_t, const void*, size_t, size_t, size_t, cudaMemcpyKind kind, cudaStream_t) {
+  if (kind == cudaMemcpyHostToDevice) write_to(dst);
   return cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) {
-  write_to(p);
-  std::memset(p, v, n);
+  if (write_to(p)) std::memset(p, v, n);
   return cudaSuccess;
 }
 

@@ -105,3 +105,14 @@ def test_a_list_that_is_already_uploaded_has_its_scratch_after_anothers_growth_f
     assert ctx.attend() == 0
     assert fake.is_live(fake.attn_part_o())
     assert refusal == "memory" or fake.attn_part_o() == first
+
+
+def test_nothing_kept_from_before_a_device_reset_comes_back(fake):
+    for _ in range(2):
+        old = fake.context(**TINY)
+        assert old.append(2) == 0 and old.full_attend() == 0 and old.destroy() == 0
+        fake.device_reset()
+        new = fake.context(**TINY)
+        assert new.rc == 0 and new.append(2) == 0 and new.full_attend() == 0
+        assert fake.stray_writes() == 0
+        assert new.destroy() == 0

@@ -17,9 +17,11 @@
  *     arguments named *_host are HOST pointers.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the default stream).  Work is enqueued
  *     on it and the call returns without waiting, except where a call says it synchronises.
- *   - the context owns every cache, table and scratch buffer (device memory it allocates at
- *     headcast_create / headcast_split_cache and frees at headcast_destroy).  The caller must
- *     keep the context's device current and must not use one context from two threads at once.
+ *   - the context owns every cache, table and scratch buffer: device memory that it takes at headcast_create or
+ *     on first use and gives up at headcast_destroy (the monolithic cache at the split).  Of what contexts give up
+ *     the library keeps at most 640 MB per GPU for contexts to come (384 MB of blocks, 256 MB of monolithic
+ *     caches); it goes back when an allocation of the library fails, or by headcast_release_memory().  The caller
+ *     must keep the context's device current and must not use one context from two threads at once.
  *   - a kernel that gave up on a bounded wait sets a device status word; the next synchronising
  *     call, or headcast_check(), reports it as HC_ERR_TIMEOUT.  Until it has been reported, later
  *     attention launches of the context return at once without computing anything (their
@@ -110,8 +112,14 @@ void headcast_default_config(headcast_config* cfg);
  * Synchronises the device. */
 int headcast_create(const headcast_config* cfg, headcast_ctx** out);
 
-/* Frees everything the context owns.  Synchronises the device.  NULL is accepted. */
+/* Gives up everything the context owns; a bounded part stays with the library (see above).  Synchronises the device;
+ * where the runtime refuses that, beside a stream capture, memory that may still be in use waits, unused by anybody,
+ * for the next call here that can synchronise.  NULL is accepted. */
 int headcast_destroy(headcast_ctx* ctx);
+
+/* Returns to the system what destroyed contexts have left with the library on the current device, for other allocators
+ * of the process.  Synchronises the device; HC_ERR_CUDA if the runtime refuses that: something may have stayed then. */
+int headcast_release_memory(void);
 
 /* Sec. 3.1 / 4.3: adds one generated block's K and V ([L][H][d] each, device) to the cache.
  * While the cache is not full the block is placed after the newest one; once full, the oldest block other

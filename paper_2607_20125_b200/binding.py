@@ -24,7 +24,7 @@ EXPORTS = ("headcast_default_config", "headcast_create", "headcast_destroy", "he
            "headcast_set_kernel_timing", "headcast_last_attention_kernel_ms", "headcast_set_tracing",
            "headcast_read_trace", "headcast_dense_attend_noalloc", "headcast_noalloc_status",
            "headcast_noalloc_last_error", "headcast_plan_schedule", "headcast_selftest_bounded_wait", "headcast_overwrite_last",
-           "headcast_append_host", "headcast_attend_host")
+           "headcast_append_host", "headcast_attend_host", "headcast_release_memory")
 
 
 class Config(C.Structure):
@@ -60,6 +60,7 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
     lib.headcast_default_config.restype = None
     lib.headcast_create.argtypes = [C.POINTER(Config), C.POINTER(vp)]
     lib.headcast_destroy.argtypes = [vp]
+    lib.headcast_release_memory.argtypes = []
     lib.headcast_append.argtypes = [vp, vp, vp, vp]
     lib.headcast_full_attend.argtypes = [vp, vp, vp, vp]
     lib.headcast_overwrite_last.argtypes = [vp, vp, vp, vp]
@@ -190,6 +191,14 @@ def noalloc_status() -> None:
     rc = lib.headcast_noalloc_status(_stream())
     if rc != 0:
         raise HeadCastError(rc, lib.headcast_noalloc_last_error().decode())
+
+
+def release_memory() -> None:
+    """Returns to the system what destroyed contexts have left with the library on the current device (at most 640 MB,
+    kept for contexts to come), for other allocators of the process."""
+    rc = load_library().headcast_release_memory()
+    if rc != 0:
+        raise HeadCastError(rc, "the device could not be synchronised (a stream is under capture?)")
 
 
 class HeadCast:

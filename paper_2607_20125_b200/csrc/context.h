@@ -65,7 +65,7 @@ class BlockCache {
       return cudaSuccess;
     }
     cudaError_t e = cudaMalloc(ptr, need);
-    if (e == cudaErrorMemoryAllocation) {
+    if (e == cudaErrorMemoryAllocation) {  // what is kept may be what is missing
       release_all();
       e = cudaMalloc(ptr, need);
     }
@@ -125,11 +125,17 @@ class BlockCache {
       aside_.insert(aside_.end(), aside.begin(), aside.end());
     return idle;
   }
+  // Gives back all that is kept.  False if something could not be waited for and stays.
+  bool trim() {
+    const bool idle = wait_idle();
+    std::lock_guard<std::mutex> hold(lock_);
+    release_all();
+    return idle && aside_.empty();
+  }
 
  private:
   struct Block { void* ptr; size_t bytes; };
-  // What is kept here, of either kind, may be what is missing.
-  void release_all() {
+  void release_all() {  // all that is kept, of either kind
     cudaGetLastError();
     shrink(0);
     if (pool_) cudaMemPoolTrimTo(pool_, 0);

@@ -581,6 +581,14 @@ int headcast_destroy(headcast_ctx* c) {
   return HC_OK;
 }
 
+int headcast_release_memory(void) {
+  int dev = 0;
+  BlockCache* memory = cudaGetDevice(&dev) == cudaSuccess ? BlockCache::current(dev) : nullptr;
+  if (memory && memory->trim()) return HC_OK;
+  cudaGetLastError();
+  return HC_ERR_CUDA;
+}
+
 int headcast_append(headcast_ctx* c, const void* k_new, const void* v_new, void* stream) {
   if (!c) return HC_ERR_INVALID_ARG;
   if (!aligned16(k_new) || !aligned16(v_new)) return fail(c, HC_ERR_INVALID_ARG, "k_new/v_new must be 16-byte aligned device pointers");

@@ -1,5 +1,8 @@
 """Device memory of the contexts, on a CUDA runtime made for tests: what is kept from one context to the next, and what
 happens when the device cannot be waited for or memory runs out."""
+import os
+import re
+
 import pytest
 
 from fake_cuda import GLOBAL_MODE, RELAXED, FakeLibrary
@@ -116,3 +119,25 @@ def test_nothing_kept_from_before_a_device_reset_comes_back(fake):
         assert new.rc == 0 and new.append(2) == 0 and new.full_attend() == 0
         assert fake.stray_writes() == 0
         assert new.destroy() == 0
+
+
+def test_kept_memory_can_be_given_back(fake):
+    alive = fake.context(**TINY)
+    with_one = fake.used()
+    gone = [fake.context(**TINY) for _ in range(3)]
+    for ctx in gone:
+        assert ctx.append(2) == 0 and ctx.full_attend() == 0 and ctx.destroy() == 0
+    assert fake.used() > with_one
+    assert fake.lib.headcast_release_memory() == 0 and fake.used() == with_one
+    assert alive.append(2) == 0 and alive.full_attend() == 0 and alive.destroy() == 0
+    fake.capture(RELAXED, None)
+    assert fake.lib.headcast_release_memory() == -3
+    fake.capture(0, None)
+    assert fake.lib.headcast_release_memory() == 0 and fake.used() == 0
+
+
+def test_the_header_states_what_is_kept():
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    source = open(os.path.join(root, "paper_2607_20125_b200", "csrc", "context.h")).read()
+    kept = [int(re.search(name + r" = (?:size_t\()?(\d+)(?:\)|ull) << 20;", source).group(1)) for name in ("CACHE_KEEP_BYTES", "MONO_KEEP_BYTES")]
+    assert f"at most {sum(kept)} MB per GPU" in open(os.path.join(root, "include", "headcast.h")).read()

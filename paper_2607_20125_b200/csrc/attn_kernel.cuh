@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(ATTN_THREADS, 1) attn_kernel(const __grid_cons
           const int tok = __shfl_sync(0xffffffffu, token, row);
           const bool valid = __shfl_sync(0xffffffffu, row_valid ? 1 : 0, row) != 0;
           v[k] = make_uint4(0, 0, 0, 0);
-          if (valid) v[k] = __ldg(reinterpret_cast<const uint4*>(p.q + (static_cast<size_t>(tok) * p.n_heads + w.head) * D) + c);
+          if (valid) v[k] = *(reinterpret_cast<const uint4*>(p.q + (static_cast<size_t>(tok) * p.n_heads + w.head) * D) + c);
         }
 #pragma unroll
         for (int k = 0; k < CH; ++k) {
@@ -647,7 +647,7 @@ __device__ __forceinline__ void combine_rows(const CombineEntry& e, int block, c
     float mk[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      mk[k] = (i0 + k < n) ? __ldg(&part_ml[row0 + static_cast<size_t>(i0 + k) * 256]).x : -INFINITY;
+      mk[k] = (i0 + k < n) ? part_ml[row0 + static_cast<size_t>(i0 + k) * 256].x : -INFINITY;
     m = fmaxf(fmaxf(m, fmaxf(mk[0], mk[1])), fmaxf(mk[2], mk[3]));
   }
   float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0}, l = 0.f;
@@ -657,7 +657,7 @@ __device__ __forceinline__ void combine_rows(const CombineEntry& e, int block, c
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const size_t row = row0 + static_cast<size_t>(min(i0 + k, n - 1)) * 256;  // past the end: a valid row, weight 0
-      ml[k] = __ldg(&part_ml[row]);
+      ml[k] = part_ml[row];
       const float4* src = reinterpret_cast<const float4*>(part_o + row * D + c * 8);
       a[k] = ld_stream_f4(src);
       b[k] = ld_stream_f4(src + 1);
@@ -699,11 +699,11 @@ __device__ __forceinline__ void combine_long_row(const CombineEntry& e, int r, c
   const size_t row0 = static_cast<size_t>(e.first_slot) * 256 + e.sub * 128 + r;
   const int n = e.n_parts;
   float m = -INFINITY;
-  for (int i = lane; i < n; i += COMBINE_LANES) m = fmaxf(m, __ldg(&part_ml[row0 + static_cast<size_t>(i) * 256]).x);
+  for (int i = lane; i < n; i += COMBINE_LANES) m = fmaxf(m, part_ml[row0 + static_cast<size_t>(i) * 256].x);
   float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0}, l = 0.f;
   for (int i = lane; i < n; i += COMBINE_LANES) {
     const size_t row = row0 + static_cast<size_t>(i) * 256;
-    const float2 ml = __ldg(&part_ml[row]);
+    const float2 ml = part_ml[row];
     const float4* src = reinterpret_cast<const float4*>(part_o + row * D + c * 8);
     const float4 a = ld_stream_f4(src), b = ld_stream_f4(src + 1);
     const float wgt = (ml.x == -INFINITY) ? 0.f : ex2_approx(ml.x - m);

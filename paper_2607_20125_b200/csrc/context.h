@@ -260,6 +260,7 @@ struct headcast_ctx {
   headcast_config cfg;
   int H, D, L, T_f, F_b, n_blk, CH, G_h, G_w;
   float scale;
+  int radius = 0;  // of the Spatial proxy, at most what reaches every token of a frame: the kernel walks rows and multiplies by it
   int state = STATE_FILLING;
   std::vector<int> slots;  // logical block -> physical ring slot (index 0 = sink block)
   bool have_labels = false;

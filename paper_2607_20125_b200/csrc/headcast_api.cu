@@ -118,7 +118,7 @@ int run_schedule(headcast_ctx* c, Schedule& s, const void* q, void* out, bool pr
     c->trace_items = s.items;
     c->trace_cta_first = s.cta_first;
   }
-  p.radius = c->cfg.proxy_radius;
+  p.radius = c->radius;
   if (proxy) {
     const int newest = c->slots.back();
     p.mid_seg_lo = c->F_b;
@@ -368,6 +368,7 @@ static int init_host(headcast_ctx* c, const headcast_config* cfg, std::vector<in
   c->n_blk = cfg->n_blocks;
   c->CH = c->D / 8;
   c->sd_slots = cfg->sd_mode ? 2 : 1;
+  c->radius = std::min(cfg->proxy_radius, std::max(c->G_h, c->G_w));
   c->scale = cfg->softmax_scale > 0.f ? cfg->softmax_scale : 1.0f / std::sqrt(static_cast<float>(c->D));
   c->row_edges = (cfg->row_edges_host && cfg->n_row_edges > 0)
                      ? std::vector<int>(cfg->row_edges_host, cfg->row_edges_host + cfg->n_row_edges)
@@ -743,7 +744,7 @@ int headcast_classify(headcast_ctx* c, const void* q, int32_t* labels_host, floa
     // sixth pair: 144 us for the sweep, now 113).  Smaller frames fit into a tile or two either way.
     std::vector<Proto> protos;
     c->sched_proxy.cls_groups.clear();
-    const long long reach = std::min<long long>(static_cast<long long>(c->cfg.proxy_radius) * (c->G_w + 1), c->T_f);
+    const long long reach = std::min<long long>(static_cast<long long>(c->radius) * (c->G_w + 1), c->T_f);
     struct Run { int q0, n; };
     std::vector<Run> runs;
     if (c->T_f > 256) {

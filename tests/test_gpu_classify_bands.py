@@ -25,3 +25,15 @@ def test_classification_of_frames_dealt_into_pairs(gh, gw, radius):
         tol = {"mse_spatial": 2e-3, "p5_spatial": 1e-2, "score": 2e-2}.get(name, 5e-3)
         assert np.abs(scores[:, i] - want[:, i]).max() <= tol, (name, scores[:, i], want[:, i])
     assert list(labels) == list(want_labels)
+
+
+@pytest.mark.parametrize("gh,gw", [(16, 17), (8, 9)])
+def test_any_radius_beyond_the_frame_means_the_whole_frame(gh, gw):
+    w = synth.Workload("whole", 4, 64, gh, gw, 3, labels=(0, 1, 2, 3))
+    results = []
+    for radius in (max(gh, gw), 10**6, 2**31 - 1):
+        p = Pair(w, keep_monolithic=True, proxy_radius=radius)
+        p.append(2)
+        results.append(p.hc.classify(to_dev(synth.make_q(w, 1, 0))))
+    for labels, scores in results[1:]:
+        assert np.array_equal(labels, results[0][0]) and np.array_equal(scores, results[0][1])

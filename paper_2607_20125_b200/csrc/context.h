@@ -305,6 +305,11 @@ struct headcast_ctx {
   DevBuf<float> part_o;
   DevBuf<float2> part_ml;
   DevBuf<float> part_mid;
+  // The partial results and the counters of the shared queue exist once: see order_shared_scratch
+  bool scratch_used = false;
+  unsigned long long scratch_stream = 0;  // of the last call that used them: its number, a handle may name another stream by now
+  int stream_switches = 0;
+  cudaEvent_t scratch_done = nullptr;
   DevBuf<float> cls_o, cls_lse, cls_tok, cls_scores;
   DevBuf<int32_t> cls_labels;
 

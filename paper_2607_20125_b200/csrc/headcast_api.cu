@@ -84,10 +84,38 @@ int launch_attn_t(headcast_ctx* c, const AttnParams& p, cudaStream_t st) {
   return HC_OK;
 }
 
+// The partial results and the counters of the shared queue are the context's, one set for all its calls, so a call on
+// another stream than the last one has to come after it.  A caller that moves to another stream does so once or twice: that
+// costs a wait for the device each time.  One that keeps changing gets an event behind every call instead, which a call on
+// a single stream is spared (an event per call costs the block of 192 tokens and four heads its overlapping launches).
+constexpr int SWITCHES_BY_WAITING = 3;
+int order_shared_scratch(headcast_ctx* c, cudaStream_t st) {
+  unsigned long long stream = 0;
+  HC_CUDA(c, cudaStreamGetId(st, &stream));
+  if (c->scratch_used && c->scratch_stream != stream) {
+    if (c->stream_switches < SWITCHES_BY_WAITING) {
+      if (!c->memory->wait_idle()) return fail(c, HC_ERR_CUDA, "the device cannot be waited for while this context changes streams (a stream is under capture?)");
+      if (++c->stream_switches == SWITCHES_BY_WAITING) HC_CUDA(c, cudaEventCreateWithFlags(&c->scratch_done, cudaEventDisableTiming));
+    } else {
+      HC_CUDA(c, cudaStreamWaitEvent(st, c->scratch_done, 0));
+    }
+  }
+  c->scratch_used = true;
+  c->scratch_stream = stream;
+  return HC_OK;
+}
+
 int run_schedule(headcast_ctx* c, Schedule& s, const void* q, void* out, bool proxy, cudaStream_t st) {
   int rc = upload_schedule(c, s, st);
   if (rc != HC_OK) return rc;
   if (s.items.empty()) return HC_OK;
+  bool shares_scratch = s.n_slots > 0 || s.dyn_end > s.dyn_first;
+  if (shares_scratch) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    HC_CUDA(c, cudaStreamIsCapturing(st, &status));
+    if (status != cudaStreamCaptureStatusNone) shares_scratch = false;  // the graph's launches are the caller's to order
+    if (shares_scratch && (rc = order_shared_scratch(c, st)) != HC_OK) return rc;
+  }
   AttnParams p;
   std::memset(&p, 0, sizeof(p));
   p.items = s.items_dev.ptr;
@@ -151,6 +179,7 @@ int run_schedule(headcast_ctx* c, Schedule& s, const void* q, void* out, bool pr
                           s.combine_dev.ptr, s.n_long, c->cells_dev, c->part_o.ptr, c->part_ml.ptr, p.out, c->H, c->T_f, c->G_w));
     ++c->launches;
   }
+  if (shares_scratch && c->scratch_done) HC_CUDA(c, cudaEventRecord(c->scratch_done, st));
   return HC_OK;
 }
 
@@ -556,6 +585,7 @@ int headcast_destroy(headcast_ctx* c) {
     if (p) cache.put(p, idle);
   if (c->ev_a) cudaEventDestroy(c->ev_a);
   if (c->ev_b) cudaEventDestroy(c->ev_b);
+  if (c->scratch_done) cudaEventDestroy(c->scratch_done);
   c->sched_dense.release(cache, idle);
   c->sched_hc.release(cache, idle);
   c->sched_cls.release(cache, idle);

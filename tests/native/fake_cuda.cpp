@@ -29,7 +29,7 @@ struct Fake {
   bool invalidated = false;                    // the capture was destroyed by a refused call
   unsigned long long context_id = 1;
   std::map<const void*, std::string> kernels;
-  std::string log;                             // launches, events and waits in order: "L<stream>:<kernel> E<stream>:<event> W<stream>:<event>"
+  std::string log;                             // launches, events and waits in order: "L<stream>:<kernel> E<stream>:<event> W<stream>:<event> S" (the device)
 };
 
 Fake& fake() {  // the library registers its kernels before this file's globals would exist
@@ -208,6 +208,7 @@ cudaError_t cudaGetDeviceProperties_v2(cudaDeviceProp* p, int) {
 cudaError_t cudaDeviceSynchronize() {
   if (fake().capture) return refused();
   finish();
+  fake().log += "S ";
   return cudaSuccess;
 }
 cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* st) {
@@ -216,6 +217,10 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* st) {
 }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) {
   return fake().capture == 2 || (fake().capture && s == fake().capture_stream && s) ? refused() : cudaSuccess;
+}
+cudaError_t cudaStreamGetId(cudaStream_t s, unsigned long long* id) {
+  *id = reinterpret_cast<uintptr_t>(s);
+  return cudaSuccess;
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
   static uintptr_t n = 1000;

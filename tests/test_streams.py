@@ -1,0 +1,72 @@
+"""Calls of one context on several streams, on a CUDA runtime made for tests: launches that share the context's scratch memory
+follow one another, by events or by a wait for the device."""
+import pytest
+
+from fake_cuda import RELAXED, FakeLibrary
+
+SIZES = [dict(n_heads=4, head_dim=64, grid_h=8, grid_w=8, n_blocks=5, keep_monolithic=1),     # short lists
+         dict(n_heads=6, head_dim=128, grid_h=20, grid_w=25, n_blocks=7, keep_monolithic=1)]  # with a shared queue
+LABELS = [0, 1, 2, 3, 2, 3]
+
+
+def unordered(log):
+    """How many scratch-using launches there are, and the pairs of them on different streams of which the earlier need not
+    have ended when the later one starts."""
+    launches, waited, before, events, pairs = [], set(), {}, {}, []  # before: what comes first on a stream, by its waits
+    for entry in log.decode().split():
+        stream, _, what = entry[1:].partition(":")
+        past = waited | before.get(stream, set()) | {i for i, s in enumerate(launches) if s == stream}
+        if entry[0] == "S":
+            waited = set(range(len(launches)))
+        elif entry[0] == "E":
+            events[what] = past
+        elif entry[0] == "W":
+            before[stream] = before.get(stream, set()) | events.get(what, set())
+        elif "attn_kernel" in what or "combine_kernel" in what:
+            pairs += [(i, len(launches)) for i in range(len(launches)) if i not in past]
+            launches.append(stream)
+    return len(launches), pairs
+
+
+def ready(fake, cfg):
+    ctx = fake.context(**cfg)
+    assert ctx.append(cfg["n_blocks"]) == 0 and ctx.split(LABELS[:cfg["n_heads"]]) == 0
+    for stream in (0, 11):  # both lists are uploaded
+        assert ctx.attend(stream) == 0 and ctx.full_attend(stream) == 0
+    fake.clear_log()
+    return ctx
+
+
+@pytest.mark.parametrize("cfg", SIZES)
+def test_calls_on_changing_streams_follow_one_another(cfg):
+    fake = FakeLibrary()
+    ctx = ready(fake, cfg)
+    for stream in (11, 12, 12, 11, 13, 0, 12, 11, 11, 12, 13, 13, 0, 11):
+        assert ctx.attend(stream) == 0 and ctx.full_attend(stream) == 0
+    n, pairs = unordered(fake.log())
+    assert n == 14 * 4 and not pairs
+    assert fake.log().count(b"S ") <= 3  # a caller that keeps changing streams is not made to wait on the host
+    assert ctx.destroy() == 0
+
+
+@pytest.mark.parametrize("cfg", SIZES)
+def test_calls_on_one_stream_record_and_wait_for_nothing(cfg):
+    fake = FakeLibrary()
+    ctx = ready(fake, cfg)
+    for _ in range(4):
+        assert ctx.attend(11) == 0 and ctx.full_attend(11) == 0
+    assert all(entry.startswith("L") for entry in fake.log().decode().split())
+
+
+def test_a_captured_call_records_and_waits_for_nothing():
+    fake = FakeLibrary()
+    ctx = ready(fake, SIZES[0])
+    for stream in (12, 11, 12, 11, 12):
+        assert ctx.attend(stream) == 0
+    fake.clear_log()
+    fake.capture(RELAXED, 21)
+    assert ctx.attend(21) == 0
+    assert all(entry.startswith("L") for entry in fake.log().decode().split())
+    fake.capture(0, None)
+    assert ctx.attend(12) == 0 and ctx.attend(11) == 0
+    assert "W11:" in fake.log().decode() and "W12:" not in fake.log().decode()

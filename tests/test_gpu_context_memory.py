@@ -1,5 +1,6 @@
 """GPU: contexts created after others were destroyed work on recycled memory and still see a zeroed cache; what is kept
 between contexts stays bounded; several threads may create and destroy at the same time."""
+import ctypes
 import threading
 
 import pytest
@@ -60,3 +61,72 @@ def test_threads_create_and_destroy_side_by_side():
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+@pytest.mark.parametrize("w", [synth.tiny(), synth.small()], ids=["tiny", "small"])
+def test_calls_on_changing_streams_give_the_results_of_one_stream(w):
+    import torch
+    from test_gpu_parity import to_dev
+    p = Pair(w, keep_monolithic=True)
+    p.append(2)
+    p.hc.set_labels(w.labels)
+    p.hc.split_cache()
+    qs = [to_dev(synth.make_q(w, 1, i)) for i in range(8)]
+    new = lambda: [torch.full_like(q, float("nan")) for q in qs]  # noqa: E731
+    calls = [(p.hc.attend, new(), new()), (p.hc.full_attend, new(), new())]
+    for call, want, _ in calls:
+        for q, out in zip(qs, want):
+            call(q, out)
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    for turn in range(6):
+        for i, q in enumerate(qs):
+            with torch.cuda.stream(streams[(i * (turn + 1)) % 3]):
+                for call, _, got in calls:
+                    call(q, got[i])
+        torch.cuda.synchronize()
+        for _, want, got in calls:
+            assert all(torch.equal(a, b) for a, b in zip(want, got))
+            for g in got:
+                g.fill_(float("nan"))
+        torch.cuda.synchronize()
+
+
+def test_kept_memory_can_be_given_back():
+    import torch
+    from paper_2607_20125_b200 import binding
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    binding.release_memory()
+    free0 = torch.cuda.mem_get_info()[0]
+    one_life(synth.small())
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    binding.release_memory()
+    assert free0 - torch.cuda.mem_get_info()[0] <= 8 << 20
+
+
+def test_destroying_a_context_beside_a_relaxed_capture_keeps_results_right():
+    """Another context, created afterwards on whatever memory came back, gives the right results."""
+    import torch
+    from paper_2607_20125_b200.binding import HeadCast
+    from test_gpu_parity import to_dev
+    w = synth.small()
+    first = HeadCast.from_workload(w)
+    k, v = (to_dev(x) for x in synth.make_kv(w, 0))
+    q = to_dev(synth.make_q(w, 0, 0))
+    out = torch.empty_like(q)
+    side, captured = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    runtime = ctypes.CDLL("libcudart.so.12")  # the one that torch has loaded
+    assert runtime.cudaStreamBeginCapture(ctypes.c_void_p(captured.cuda_stream), 2) == 0  # relaxed
+    with torch.cuda.stream(side):
+        first.append(k, v)
+        for _ in range(20):
+            first.full_attend(q, out)
+        first.destroy()
+    graph = ctypes.c_void_p()
+    runtime.cudaStreamEndCapture(ctypes.c_void_p(captured.cuda_stream), ctypes.byref(graph))  # destroy has ended the capture
+    runtime.cudaGetLastError()
+    torch.cuda.synchronize()
+    one_life(w)

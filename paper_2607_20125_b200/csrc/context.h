@@ -193,12 +193,25 @@ cudaError_t take_or_wait(BlockCache& cache, F take) {
   return e;
 }
 
+// Where a context's device memory comes from.  Once a launch of the context has been captured, a graph may use any of its
+// arrays at any time: arrays that were outgrown then stay until the context goes.
+struct ContextMemory {
+  BlockCache* cache = nullptr;
+  bool captured = false;
+  std::vector<void*> outgrown;
+  void release(bool idle) {
+    for (void* ptr : outgrown) cache->put(ptr, idle);
+    outgrown.clear();
+  }
+};
+
 template <typename T>
 struct DevBuf {  // grow-only device array of the context's device
   T* ptr = nullptr;
   size_t cap = 0;
-  cudaError_t reserve(BlockCache& cache, size_t n, cudaStream_t st) {
+  cudaError_t reserve(ContextMemory& memory, size_t n, cudaStream_t st) {
     if (n <= cap) return cudaSuccess;
+    BlockCache& cache = *memory.cache;
     // while `st` is captured the cache stands aside: cudaMalloc then says whether memory may be taken in this capture mode
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &status);
@@ -207,12 +220,12 @@ struct DevBuf {  // grow-only device array of the context's device
     void* bigger = nullptr;
     size_t bytes = 0;
     e = cache.get(&bigger, n * sizeof(T), &bytes, capturing);
-    if (e == cudaErrorMemoryAllocation && ptr) {  // no room for both: the old one first
-      give_back(cache);
+    if (e == cudaErrorMemoryAllocation && ptr && !memory.captured) {  // no room for both: the old one first
+      give_back(memory);
       e = cache.get(&bigger, n * sizeof(T), &bytes, capturing);
     }
     if (e == cudaSuccess) {
-      give_back(cache);
+      give_back(memory);
       ptr = static_cast<T*>(bigger);
       cap = bytes / sizeof(T);
     }
@@ -220,7 +233,13 @@ struct DevBuf {  // grow-only device array of the context's device
   }
   // Any stream may still use the array.  cudaFree waits for them; a device synchronisation, with which the memory could be
   // kept, would be refused beside a capture on whatever stream and destroy that capture.
-  void give_back(BlockCache& cache) { release(cache, false); }
+  void give_back(ContextMemory& memory) {
+    if (ptr && memory.captured) {
+      memory.outgrown.push_back(ptr);
+      ptr = nullptr;
+    }
+    release(*memory.cache, false);
+  }
   void release(BlockCache& cache, bool idle) {
     if (ptr) cache.put(ptr, idle);
     ptr = nullptr;
@@ -314,7 +333,7 @@ struct headcast_ctx {
   DevBuf<int32_t> cls_labels;
 
   int device = 0;
-  BlockCache* memory = nullptr;  // where the device memory of this context comes from
+  ContextMemory memory;
   int n_sm = 148;
   int64_t launches = 0;
   bool tracing = false;  // record per-item start/end times in the attention kernel

@@ -30,14 +30,14 @@ int upload_schedule(headcast_ctx* c, Schedule& s, cudaStream_t st) {
   // The partial results are shared by all lists of the context, so every launch makes sure of them and not only the first of
   // its list: another list's growth may have failed in between and left none.
   if (s.n_slots > 0) {
-    HC_CUDA(c, c->part_o.reserve(*c->memory, static_cast<size_t>(s.n_slots) * 256 * c->D, st));
-    HC_CUDA(c, c->part_ml.reserve(*c->memory, static_cast<size_t>(s.n_slots) * 256, st));
-    HC_CUDA(c, c->part_mid.reserve(*c->memory, static_cast<size_t>(s.n_slots) * 256, st));
+    HC_CUDA(c, c->part_o.reserve(c->memory, static_cast<size_t>(s.n_slots) * 256 * c->D, st));
+    HC_CUDA(c, c->part_ml.reserve(c->memory, static_cast<size_t>(s.n_slots) * 256, st));
+    HC_CUDA(c, c->part_mid.reserve(c->memory, static_cast<size_t>(s.n_slots) * 256, st));
   }
   if (s.uploaded) return HC_OK;
-  HC_CUDA(c, s.items_dev.reserve(*c->memory, std::max<size_t>(1, s.items.size()), st));
-  HC_CUDA(c, s.cta_first_dev.reserve(*c->memory, s.cta_first.size(), st));
-  HC_CUDA(c, s.combine_dev.reserve(*c->memory, std::max<size_t>(1, s.combine.size()), st));
+  HC_CUDA(c, s.items_dev.reserve(c->memory, std::max<size_t>(1, s.items.size()), st));
+  HC_CUDA(c, s.cta_first_dev.reserve(c->memory, s.cta_first.size(), st));
+  HC_CUDA(c, s.combine_dev.reserve(c->memory, std::max<size_t>(1, s.combine.size()), st));
   if (!s.items.empty())
     HC_CUDA(c, cudaMemcpyAsync(s.items_dev.ptr, s.items.data(), s.items.size() * sizeof(WorkItem),
                                cudaMemcpyHostToDevice, st));
@@ -47,8 +47,8 @@ int upload_schedule(headcast_ctx* c, Schedule& s, cudaStream_t st) {
     HC_CUDA(c, cudaMemcpyAsync(s.combine_dev.ptr, s.combine.data(), s.combine.size() * sizeof(CombineEntry),
                                cudaMemcpyHostToDevice, st));
   if (!s.cls_groups.empty()) {
-    HC_CUDA(c, s.cls_groups_dev.reserve(*c->memory, s.cls_groups.size(), st));
-    HC_CUDA(c, s.cls_parts_dev.reserve(*c->memory, std::max<size_t>(1, s.cls_parts.size()), st));
+    HC_CUDA(c, s.cls_groups_dev.reserve(c->memory, s.cls_groups.size(), st));
+    HC_CUDA(c, s.cls_parts_dev.reserve(c->memory, std::max<size_t>(1, s.cls_parts.size()), st));
     HC_CUDA(c, cudaMemcpyAsync(s.cls_groups_dev.ptr, s.cls_groups.data(), s.cls_groups.size() * sizeof(ClsGroup),
                                cudaMemcpyHostToDevice, st));
     HC_CUDA(c, cudaMemcpyAsync(s.cls_parts_dev.ptr, s.cls_parts.data(), s.cls_parts.size() * sizeof(ClsPart),
@@ -94,7 +94,7 @@ int order_shared_scratch(headcast_ctx* c, cudaStream_t st) {
   HC_CUDA(c, cudaStreamGetId(st, &stream));
   if (c->scratch_used && c->scratch_stream != stream) {
     if (c->stream_switches < SWITCHES_BY_WAITING) {
-      if (!c->memory->wait_idle()) return fail(c, HC_ERR_CUDA, "the device cannot be waited for while this context changes streams (a stream is under capture?)");
+      if (!c->memory.cache->wait_idle()) return fail(c, HC_ERR_CUDA, "the device cannot be waited for while this context changes streams (a stream is under capture?)");
       if (++c->stream_switches == SWITCHES_BY_WAITING) HC_CUDA(c, cudaEventCreateWithFlags(&c->scratch_done, cudaEventDisableTiming));
     } else {
       HC_CUDA(c, cudaStreamWaitEvent(st, c->scratch_done, 0));
@@ -106,16 +106,16 @@ int order_shared_scratch(headcast_ctx* c, cudaStream_t st) {
 }
 
 int run_schedule(headcast_ctx* c, Schedule& s, const void* q, void* out, bool proxy, cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  HC_CUDA(c, cudaStreamIsCapturing(st, &status));
+  const bool capturing = status != cudaStreamCaptureStatusNone;
+  c->memory.captured = c->memory.captured || capturing;
   int rc = upload_schedule(c, s, st);
   if (rc != HC_OK) return rc;
   if (s.items.empty()) return HC_OK;
-  bool shares_scratch = s.n_slots > 0 || s.dyn_end > s.dyn_first;
-  if (shares_scratch) {
-    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-    HC_CUDA(c, cudaStreamIsCapturing(st, &status));
-    if (status != cudaStreamCaptureStatusNone) shares_scratch = false;  // the graph's launches are the caller's to order
-    if (shares_scratch && (rc = order_shared_scratch(c, st)) != HC_OK) return rc;
-  }
+  // (the launches of a graph are the caller's to order)
+  const bool shares_scratch = !capturing && (s.n_slots > 0 || s.dyn_end > s.dyn_first);
+  if (shares_scratch && (rc = order_shared_scratch(c, st)) != HC_OK) return rc;
   AttnParams p;
   std::memset(&p, 0, sizeof(p));
   p.items = s.items_dev.ptr;
@@ -140,7 +140,7 @@ int run_schedule(headcast_ctx* c, Schedule& s, const void* q, void* out, bool pr
   p.trace = nullptr;
   if (c->tracing) {
     const size_t trace_words = 2 * s.items.size();
-    HC_CUDA(c, c->trace_dev.reserve(*c->memory, trace_words, st));
+    HC_CUDA(c, c->trace_dev.reserve(c->memory, trace_words, st));
     HC_CUDA(c, cudaMemsetAsync(c->trace_dev.ptr, 0, trace_words * sizeof(unsigned long long), st));
     p.trace = c->trace_dev.ptr;
     c->trace_items = s.items;
@@ -514,12 +514,12 @@ int headcast_create(const headcast_config* cfg, headcast_ctx** out) {
     return HC_ERR_UNSUPPORTED;
   }
   const size_t mono_bytes = cache_elems(c, c->H) * sizeof(__nv_bfloat16);
-  c->memory = BlockCache::current(c->device);
-  if (!c->memory) {
+  c->memory.cache = BlockCache::current(c->device);
+  if (!c->memory.cache) {
     delete c;
     return HC_ERR_CUDA;
   }
-  BlockCache& cache = *c->memory;
+  BlockCache& cache = *c->memory.cache;
   cudaError_t e = cudaSuccess;
   auto step = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
   auto get = [&](auto** ptr, size_t bytes) {
@@ -576,7 +576,7 @@ int headcast_destroy(headcast_ctx* c) {
   int current = c->device;  // the context's memory belongs to its own device, whichever one is current now
   cudaGetDevice(&current);
   if (current != c->device) cudaSetDevice(c->device);
-  BlockCache& cache = *c->memory;
+  BlockCache& cache = *c->memory.cache;
   const bool idle = cache.wait_idle();  // if not, kernels may be at work on any of these: nothing of it is kept for others
   if (c->mono_k) cache.put_mono(c->mono_k, idle);
   if (c->mono_v) cache.put_mono(c->mono_v, idle);
@@ -608,6 +608,7 @@ int headcast_destroy(headcast_ctx* c) {
   c->cls_tok.release(cache, idle);
   c->cls_scores.release(cache, idle);
   c->cls_labels.release(cache, idle);
+  c->memory.release(idle);
   if (!idle) cudaGetLastError();  // the refusal is dealt with, no later call is to report it
   if (current != c->device) cudaSetDevice(current);
   delete c;
@@ -712,11 +713,11 @@ int headcast_classify(headcast_ctx* c, const void* q, int32_t* labels_host, floa
   if (n_filled(c) < 2) return fail(c, HC_ERR_STATE, "classification needs at least two cached blocks");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t rows = static_cast<size_t>(c->L) * c->H;
-  HC_CUDA(c, c->cls_o.reserve(*c->memory, rows * c->D, st));  // the reference output (fp32); the proxy outputs never leave registers
-  HC_CUDA(c, c->cls_lse.reserve(*c->memory, rows, st));
-  HC_CUDA(c, c->cls_tok.reserve(*c->memory, TOK_N * rows, st));
-  HC_CUDA(c, c->cls_scores.reserve(*c->memory, static_cast<size_t>(c->H) * HC_N_SCORES, st));
-  HC_CUDA(c, c->cls_labels.reserve(*c->memory, c->H, st));
+  HC_CUDA(c, c->cls_o.reserve(c->memory, rows * c->D, st));  // the reference output (fp32); the proxy outputs never leave registers
+  HC_CUDA(c, c->cls_lse.reserve(c->memory, rows, st));
+  HC_CUDA(c, c->cls_tok.reserve(c->memory, TOK_N * rows, st));
+  HC_CUDA(c, c->cls_scores.reserve(c->memory, static_cast<size_t>(c->H) * HC_N_SCORES, st));
+  HC_CUDA(c, c->cls_labels.reserve(c->memory, c->H, st));
   const int newest = c->slots.back();
   const int cls_key = n_filled(c) * 64 + newest;  // the work lists depend on the fill and on where the newest block sits
   if (c->sched_cls.key_filled != cls_key) {
@@ -931,8 +932,8 @@ int headcast_append_host(headcast_ctx* c, const void* k_host, const void* v_host
   if (!c || !k_host || !v_host) return HC_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t elems = static_cast<size_t>(c->L) * c->H * c->D;
-  HC_CUDA(c, c->stage_k.reserve(*c->memory, elems, st));
-  HC_CUDA(c, c->stage_v.reserve(*c->memory, elems, st));
+  HC_CUDA(c, c->stage_k.reserve(c->memory, elems, st));
+  HC_CUDA(c, c->stage_v.reserve(c->memory, elems, st));
   HC_CUDA(c, cudaMemcpyAsync(c->stage_k.ptr, k_host, elems * sizeof(__nv_bfloat16), cudaMemcpyHostToDevice, st));
   HC_CUDA(c, cudaMemcpyAsync(c->stage_v.ptr, v_host, elems * sizeof(__nv_bfloat16), cudaMemcpyHostToDevice, st));
   return headcast_append(c, c->stage_k.ptr, c->stage_v.ptr, stream);
@@ -945,8 +946,8 @@ int headcast_attend_host(headcast_ctx* c, const void* q_host, void* out_host, vo
   int rc = init_host_path(c);
   if (rc != HC_OK) return rc;
   const size_t elems = static_cast<size_t>(c->L) * c->H * c->D;
-  HC_CUDA(c, c->stage_q.reserve(*c->memory, elems, st));
-  HC_CUDA(c, c->stage_out.reserve(*c->memory, elems, st));
+  HC_CUDA(c, c->stage_q.reserve(c->memory, elems, st));
+  HC_CUDA(c, c->stage_out.reserve(c->memory, elems, st));
   const int key = n_filled(c) * 4 + c->sd_valid;
   // Stages: a stage's queries are copied in (strided: the rows of [L][H][d] hold all heads), attended and copied out
   // as a unit, so that the next stage's queries arrive and the previous stage's outputs leave while this stage

@@ -141,3 +141,17 @@ def test_the_header_states_what_is_kept():
     source = open(os.path.join(root, "paper_2607_20125_b200", "csrc", "context.h")).read()
     kept = [int(re.search(name + r" = (?:size_t\()?(\d+)(?:\)|ull) << 20;", source).group(1)) for name in ("CACHE_KEEP_BYTES", "MONO_KEEP_BYTES")]
     assert f"at most {sum(kept)} MB per GPU" in open(os.path.join(root, "include", "headcast.h")).read()
+
+
+def test_scratch_that_a_graph_uses_stays_when_another_list_needs_more(fake):
+    ctx = fake.context(n_heads=6, head_dim=128, grid_h=13, grid_w=22, n_blocks=4, cell_h=6, cell_w=6, keep_monolithic=1)
+    assert ctx.append(4) == 0 and ctx.split([0, 1, 2, 3, 2, 3]) == 0 and ctx.attend() == 0
+    fake.capture(RELAXED, 21)
+    assert ctx.attend(stream=21) == 0
+    fake.capture(0, None)
+    in_graph = fake.attn_part_o()
+    fake.capacity_left(64 << 10)
+    assert ctx.full_attend() == -4 and fake.is_live(in_graph)  # not even for want of memory
+    fake.capacity_left(64 << 20)
+    assert ctx.full_attend() == 0 and fake.attn_part_o() != in_graph and fake.is_live(in_graph)
+    assert ctx.destroy() == 0 and fake.lib.headcast_release_memory() == 0 and fake.used() == 0

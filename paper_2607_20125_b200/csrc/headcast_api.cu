@@ -772,42 +772,56 @@ int headcast_classify(headcast_ctx* c, const void* q, int32_t* labels_host, floa
     // its last one, in every cached frame.  A pair that straddles two frames has to sweep whole frames, so frames of more
     // than 256 tokens are dealt into pairs of their own, of equal size (30 x 52 tokens, r = 2: seven pairs of 223 queries
     // and 4 key tiles per frame; with pairs of 256 across the block and whole grid rows it was 5 tiles, and 13 for every
-    // sixth pair: 144 us for the sweep, now 113).  Smaller frames fit into a tile or two either way.
+    // sixth pair: 144 us for the sweep, now 113).  Where the bands cannot get shorter - a frame little larger than a pair,
+    // rows or a radius that reach over most of it (1 x 300 tokens: 18 tiles per frame against 12) - and for smaller frames,
+    // which fit into a tile or two either way, the fewer pairs across the block are the cheaper deal.
     std::vector<Proto> protos;
     c->sched_proxy.cls_groups.clear();
     const long long reach = std::min<long long>(static_cast<long long>(c->radius) * (c->G_w + 1), c->T_f);
     struct Run { int q0, n; };
-    std::vector<Run> runs;
+    auto band_item = [&](const Run& run, int h) {
+      const int q0 = run.q0, q1 = run.q0 + run.n - 1;
+      int a = 0, b = c->T_f;
+      if (q0 / c->T_f == q1 / c->T_f) {
+        a = static_cast<int>(std::max<long long>(0, q0 % c->T_f - reach));
+        b = static_cast<int>(std::min<long long>(c->T_f, q1 % c->T_f + reach + 1));
+      }
+      WorkItem w = range_item(h, MAP_MONO, h * c->D, a, b - a);
+      w.seg_stride = c->T_f;
+      w.q_start[0] = q0;
+      w.q_start[1] = q0 + 128;
+      w.q_count[0] = std::min(128, run.n);
+      w.q_count[1] = std::max(0, run.n - 128);
+      return w;
+    };
+    std::vector<Run> runs, per_frame;
+    for (int q0 = 0; q0 < c->L; q0 += 256) runs.push_back({q0, std::min(256, c->L - q0)});
     if (c->T_f > 256) {
-      const int per_frame = (c->T_f + 255) / 256, size = (c->T_f + per_frame - 1) / per_frame;
+      const int n = (c->T_f + 255) / 256, size = (c->T_f + n - 1) / n;
       for (int f = 0; f < c->F_b; ++f)
-        for (int i = 0; i < c->T_f; i += size) runs.push_back({f * c->T_f + i, std::min(size, c->T_f - i)});
-    } else {
-      for (int q0 = 0; q0 < c->L; q0 += 256) runs.push_back({q0, std::min(256, c->L - q0)});
+        for (int i = 0; i < c->T_f; i += size) per_frame.push_back({f * c->T_f + i, std::min(size, c->T_f - i)});
+      auto cost = [&](const std::vector<Run>& deal) {
+        double sum = 0.0;
+        for (const Run& run : deal) {
+          const WorkItem w = band_item(run, 0);
+          sum += COST_MEASURED.cost(w, w.tiles_per_seg * n_filled(c) * c->F_b, true);
+        }
+        return sum;
+      };
+      if (cost(per_frame) < cost(runs)) runs.swap(per_frame);
     }
     for (int h = 0; h < c->H; ++h)
       for (const Run& run : runs) {
-        const int q0 = run.q0, q1 = run.q0 + run.n - 1;
-        int a = 0, b = c->T_f;
-        if (q0 / c->T_f == q1 / c->T_f) {
-          a = static_cast<int>(std::max<long long>(0, q0 % c->T_f - reach));
-          b = static_cast<int>(std::min<long long>(c->T_f, q1 % c->T_f + reach + 1));
-        }
-        WorkItem w = range_item(h, MAP_MONO, h * c->D, a, b - a);
-        w.seg_stride = c->T_f;
+        const WorkItem w = band_item(run, h);
         Proto p;
         p.w = w;
-        p.w.q_start[0] = q0;
-        p.w.q_start[1] = q0 + 128;
-        p.w.q_count[0] = std::min(128, run.n);
-        p.w.q_count[1] = std::max(0, run.n - 128);
         p.n_tiles = w.tiles_per_seg * n_filled(c) * c->F_b;
         p.w.tile_begin = 0;
         p.w.tile_end = p.n_tiles;
         // whole or cut into pieces, a band leaves partial results that proxy_combine_kernel merges and scores
         ClsGroup g;
         g.head = h;
-        g.q_start = q0;
+        g.q_start = run.q0;
         g.q_count[0] = p.w.q_count[0];
         g.q_count[1] = p.w.q_count[1];
         g.first_part = 0;

@@ -9,3 +9,9 @@ extern "C" void fake_saw_launch(const char* name, void** args) {
 }
 extern "C" void* fake_attn_part_o() { return last_attn.part_o; }
 extern "C" int fake_attn_radius() { return last_attn.radius; }
+// Key tiles of its work list, over all CTAs (without a shared queue).
+extern "C" int fake_attn_tile_steps() {
+  int sum = 0;
+  for (int i = 0; i < last_attn.cta_first[148]; ++i) sum += last_attn.items[i].tile_end - last_attn.items[i].tile_begin;
+  return sum;
+}

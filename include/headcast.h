@@ -17,9 +17,9 @@
  *     arguments named *_host are HOST pointers.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the default stream).  Work is enqueued
  *     on it and the call returns without waiting, except where a call says it synchronises.
- *     Attention calls of one context share scratch memory: on different streams the library orders them one
- *     after the other (it waits for the device the first times a context changes streams).  Launches captured
- *     into a graph use the same scratch at every replay; the caller orders replays and other calls.
+ *     Attention calls of one context share scratch memory.  When a context changes streams the call takes a new
+ *     scratch, the first three times, and from then on waits on the device for the call before it.  Launches
+ *     captured into a graph use the same scratch at every replay; the caller orders replays and other calls.
  *   - the context owns every cache, table and scratch buffer: device memory that it takes at headcast_create or
  *     on first use and gives up at headcast_destroy (the monolithic cache at the split).  Of what contexts give up
  *     the library keeps at most 640 MB per GPU for contexts to come (384 MB of blocks, 256 MB of monolithic

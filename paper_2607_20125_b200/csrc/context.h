@@ -193,11 +193,11 @@ cudaError_t take_or_wait(BlockCache& cache, F take) {
   return e;
 }
 
-// Where a context's device memory comes from.  Once a launch of the context has been captured, a graph may use any of its
-// arrays at any time: arrays that were outgrown then stay until the context goes.
+// Where a context's device memory comes from.  Arrays that were outgrown and may still be in use, by work on any stream or by
+// a graph, stay until the context goes.
 struct ContextMemory {
   BlockCache* cache = nullptr;
-  bool captured = false;
+  bool captured = false;  // a launch of the context has been captured: a graph may use any of its arrays at any time
   std::vector<void*> outgrown;
   void release(bool idle) {
     for (void* ptr : outgrown) cache->put(ptr, idle);
@@ -209,9 +209,28 @@ template <typename T>
 struct DevBuf {  // grow-only device array of the context's device
   T* ptr = nullptr;
   size_t cap = 0;
+  // The old array stays with the context (small blocks come in powers of two: all of them together are smaller than the new one).
   cudaError_t reserve(ContextMemory& memory, size_t n, cudaStream_t st) {
-    if (n <= cap) return cudaSuccess;
-    BlockCache& cache = *memory.cache;
+    return n <= cap ? cudaSuccess : grow(memory, n, st, false);
+  }
+  // For the large arrays, whose uses all come before this point of `st`: once the stream is waited for, the old array is kept
+  // for others.  (A wait for the whole device would be refused beside a capture on whatever stream and destroy that capture.)
+  cudaError_t reserve_in_order(ContextMemory& memory, size_t n, cudaStream_t st) {
+    return n <= cap ? cudaSuccess : grow(memory, n, st, !memory.captured);
+  }
+  void retire(ContextMemory& memory) {
+    if (ptr) memory.outgrown.push_back(ptr);
+    ptr = nullptr;
+    cap = 0;
+  }
+  void release(BlockCache& cache, bool idle) {
+    if (ptr) cache.put(ptr, idle);
+    ptr = nullptr;
+    cap = 0;
+  }
+
+ private:
+  cudaError_t grow(ContextMemory& memory, size_t n, cudaStream_t st, bool in_order) {
     // while `st` is captured the cache stands aside: cudaMalloc then says whether memory may be taken in this capture mode
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &status);
@@ -219,31 +238,20 @@ struct DevBuf {  // grow-only device array of the context's device
     const bool capturing = status != cudaStreamCaptureStatusNone;
     void* bigger = nullptr;
     size_t bytes = 0;
-    e = cache.get(&bigger, n * sizeof(T), &bytes, capturing);
-    if (e == cudaErrorMemoryAllocation && ptr && !memory.captured) {  // no room for both: the old one first
-      give_back(memory);
-      e = cache.get(&bigger, n * sizeof(T), &bytes, capturing);
+    e = memory.cache->get(&bigger, n * sizeof(T), &bytes, capturing);
+    if (e == cudaErrorMemoryAllocation && !memory.captured) {  // what this context does not need any more comes first
+      if (in_order) release(*memory.cache, ptr && cudaStreamSynchronize(st) == cudaSuccess);
+      if (!memory.outgrown.empty() && memory.cache->wait_idle()) memory.release(true);
+      e = memory.cache->get(&bigger, n * sizeof(T), &bytes, capturing);
     }
-    if (e == cudaSuccess) {
-      give_back(memory);
-      ptr = static_cast<T*>(bigger);
-      cap = bytes / sizeof(T);
-    }
-    return e;
-  }
-  // Any stream may still use the array.  cudaFree waits for them; a device synchronisation, with which the memory could be
-  // kept, would be refused beside a capture on whatever stream and destroy that capture.
-  void give_back(ContextMemory& memory) {
-    if (ptr && memory.captured) {
-      memory.outgrown.push_back(ptr);
-      ptr = nullptr;
-    }
-    release(*memory.cache, false);
-  }
-  void release(BlockCache& cache, bool idle) {
-    if (ptr) cache.put(ptr, idle);
-    ptr = nullptr;
-    cap = 0;
+    if (e != cudaSuccess) return e;
+    if (ptr && in_order)
+      release(*memory.cache, cudaStreamSynchronize(st) == cudaSuccess);
+    else
+      retire(memory);
+    ptr = static_cast<T*>(bigger);
+    cap = bytes / sizeof(T);
+    return cudaSuccess;
   }
 };
 
@@ -324,10 +332,11 @@ struct headcast_ctx {
   DevBuf<float> part_o;
   DevBuf<float2> part_ml;
   DevBuf<float> part_mid;
-  // The partial results and the counters of the shared queue exist once: see order_shared_scratch
+  // The partial results and the counters of the shared queue: see order_shared_scratch
   bool scratch_used = false;
   unsigned long long scratch_stream = 0;  // of the last call that used them: its number, a handle may name another stream by now
-  int stream_switches = 0;
+  int stream_changes = 0;
+  std::vector<int32_t*> old_counters;  // of streams that were left, see dyn_counter_dev
   cudaEvent_t scratch_done = nullptr;
   DevBuf<float> cls_o, cls_lse, cls_tok, cls_scores;
   DevBuf<int32_t> cls_labels;

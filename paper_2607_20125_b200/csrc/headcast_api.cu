@@ -30,9 +30,9 @@ int upload_schedule(headcast_ctx* c, Schedule& s, cudaStream_t st) {
   // The partial results are shared by all lists of the context, so every launch makes sure of them and not only the first of
   // its list: another list's growth may have failed in between and left none.
   if (s.n_slots > 0) {
-    HC_CUDA(c, c->part_o.reserve(c->memory, static_cast<size_t>(s.n_slots) * 256 * c->D, st));
-    HC_CUDA(c, c->part_ml.reserve(c->memory, static_cast<size_t>(s.n_slots) * 256, st));
-    HC_CUDA(c, c->part_mid.reserve(c->memory, static_cast<size_t>(s.n_slots) * 256, st));
+    HC_CUDA(c, c->part_o.reserve_in_order(c->memory, static_cast<size_t>(s.n_slots) * 256 * c->D, st));
+    HC_CUDA(c, c->part_ml.reserve_in_order(c->memory, static_cast<size_t>(s.n_slots) * 256, st));
+    HC_CUDA(c, c->part_mid.reserve_in_order(c->memory, static_cast<size_t>(s.n_slots) * 256, st));
   }
   if (s.uploaded) return HC_OK;
   HC_CUDA(c, s.items_dev.reserve(c->memory, std::max<size_t>(1, s.items.size()), st));
@@ -85,19 +85,26 @@ int launch_attn_t(headcast_ctx* c, const AttnParams& p, cudaStream_t st) {
 }
 
 // The partial results and the counters of the shared queue are the context's, one set for all its calls, so a call on
-// another stream than the last one has to come after it.  A caller that moves to another stream does so once or twice: that
-// costs a wait for the device each time.  One that keeps changing gets an event behind every call instead, which a call on
-// a single stream is spared (an event per call costs the block of 192 tokens and four heads its overlapping launches).
-constexpr int SWITCHES_BY_WAITING = 3;
+// another stream than the last one has to come after it, or use a set of its own.  A caller that moves to another stream once
+// or twice gets a new set there; the old one stays with the stream that may still work on it.  One that keeps changing gets
+// an event behind every call, and a wait for it when the stream changes.  A single stream is spared both.
+constexpr int CHANGES_WITH_NEW_SCRATCH = 3;
 int order_shared_scratch(headcast_ctx* c, cudaStream_t st) {
   unsigned long long stream = 0;
   HC_CUDA(c, cudaStreamGetId(st, &stream));
   if (c->scratch_used && c->scratch_stream != stream) {
-    if (c->stream_switches < SWITCHES_BY_WAITING) {
-      if (!c->memory.cache->wait_idle()) return fail(c, HC_ERR_CUDA, "the device cannot be waited for while this context changes streams (a stream is under capture?)");
-      if (++c->stream_switches == SWITCHES_BY_WAITING) HC_CUDA(c, cudaEventCreateWithFlags(&c->scratch_done, cudaEventDisableTiming));
-    } else {
+    if (c->scratch_done) {
       HC_CUDA(c, cudaStreamWaitEvent(st, c->scratch_done, 0));
+    } else {
+      void* counters = nullptr;
+      HC_CUDA(c, c->memory.cache->get(&counters, 2 * sizeof(int32_t)));
+      c->old_counters.push_back(c->dyn_counter_dev);
+      c->dyn_counter_dev = static_cast<int32_t*>(counters);
+      HC_CUDA(c, cudaMemsetAsync(c->dyn_counter_dev, 0, 2 * sizeof(int32_t), st));
+      c->part_o.retire(c->memory);
+      c->part_ml.retire(c->memory);
+      c->part_mid.retire(c->memory);
+      if (++c->stream_changes >= CHANGES_WITH_NEW_SCRATCH) HC_CUDA(c, cudaEventCreateWithFlags(&c->scratch_done, cudaEventDisableTiming));
     }
   }
   c->scratch_used = true;
@@ -110,12 +117,12 @@ int run_schedule(headcast_ctx* c, Schedule& s, const void* q, void* out, bool pr
   HC_CUDA(c, cudaStreamIsCapturing(st, &status));
   const bool capturing = status != cudaStreamCaptureStatusNone;
   c->memory.captured = c->memory.captured || capturing;
-  int rc = upload_schedule(c, s, st);
-  if (rc != HC_OK) return rc;
-  if (s.items.empty()) return HC_OK;
   // (the launches of a graph are the caller's to order)
   const bool shares_scratch = !capturing && (s.n_slots > 0 || s.dyn_end > s.dyn_first);
-  if (shares_scratch && (rc = order_shared_scratch(c, st)) != HC_OK) return rc;
+  int rc = shares_scratch ? order_shared_scratch(c, st) : HC_OK;
+  if (rc == HC_OK) rc = upload_schedule(c, s, st);
+  if (rc != HC_OK) return rc;
+  if (s.items.empty()) return HC_OK;
   AttnParams p;
   std::memset(&p, 0, sizeof(p));
   p.items = s.items_dev.ptr;
@@ -359,7 +366,9 @@ int read_status(headcast_ctx* c, cudaStream_t st) {
   HC_CUDA(c, cudaStreamSynchronize(st));
   if (status != 0) {
     cudaMemsetAsync(c->status_dev, 0, sizeof(int32_t), st);
-    cudaMemsetAsync(c->dyn_counter_dev, 0, 2 * sizeof(int32_t), st);  // a kernel that gave up may have left the queue half drawn
+    // a kernel that gave up may have left the queue half drawn
+    cudaMemsetAsync(c->dyn_counter_dev, 0, 2 * sizeof(int32_t), st);
+    for (int32_t* counter : c->old_counters) cudaMemsetAsync(counter, 0, 2 * sizeof(int32_t), st);  // graphs may hold these
     return fail(c, HC_ERR_TIMEOUT, "a kernel gave up on a bounded wait (site %d)", status);
   }
   return HC_OK;
@@ -583,6 +592,7 @@ int headcast_destroy(headcast_ctx* c) {
   void* ptrs[] = {c->arena_k, c->arena_v, c->sp_base, c->sp_nc, c->cells_dev, c->status_dev, c->dyn_counter_dev, c->move_boxes_dev};
   for (void* p : ptrs)
     if (p) cache.put(p, idle);
+  for (int32_t* counter : c->old_counters) cache.put(counter, idle);
   if (c->ev_a) cudaEventDestroy(c->ev_a);
   if (c->ev_b) cudaEventDestroy(c->ev_b);
   if (c->scratch_done) cudaEventDestroy(c->scratch_done);

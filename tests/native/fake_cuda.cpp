@@ -29,7 +29,9 @@ struct Fake {
   bool invalidated = false;                    // the capture was destroyed by a refused call
   unsigned long long context_id = 1;
   std::map<const void*, std::string> kernels;
-  std::string log;                             // launches, events and waits in order: "L<stream>:<kernel> E<stream>:<event> W<stream>:<event> S" (the device)
+  // launches, events, waits and the host's waits for a stream or the device, in order:
+  // "L<stream>:<kernel>@<scratch> E<stream>:<event> W<stream>:<event> Y<stream>: S"
+  std::string log;
 };
 
 Fake& fake() {  // the library registers its kernels before this file's globals would exist
@@ -87,7 +89,7 @@ std::string handle(const void* p) { return std::to_string(reinterpret_cast<uintp
 
 extern "C" {
 
-void fake_saw_launch(const char* name, void** args);
+const void* fake_saw_launch(const char* name, void** args);
 
 void fake_reset() {
   fake().capacity = 1ll << 40;
@@ -216,7 +218,9 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* st) {
   return cudaSuccess;
 }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) {
-  return fake().capture == 2 || (fake().capture && s == fake().capture_stream && s) ? refused() : cudaSuccess;
+  if (fake().capture == 2 || (fake().capture && s == fake().capture_stream && s)) return refused();
+  fake().log += "Y" + handle(s) + ": ";
+  return cudaSuccess;
 }
 cudaError_t cudaStreamGetId(cudaStream_t s, unsigned long long* id) {
   *id = reinterpret_cast<uintptr_t>(s);
@@ -262,8 +266,8 @@ cudaError_t cudaGetSymbolAddress(void** p, const void*) {
 }
 static cudaError_t launched(const void* fn, void** args, cudaStream_t s) {
   const std::string& name = fake().kernels[fn];
-  fake().log += "L" + handle(s) + ":" + name + " ";
-  fake_saw_launch(name.c_str(), args);
+  const void* scratch = fake_saw_launch(name.c_str(), args);
+  fake().log += "L" + handle(s) + ":" + name + "@" + handle(scratch) + " ";
   return cudaSuccess;
 }
 cudaError_t cudaLaunchKernel(const void* fn, dim3, dim3, void** args, size_t, cudaStream_t s) { return launched(fn, args, s); }

@@ -84,13 +84,17 @@ def test_a_growing_scratch_array_takes_back_the_pools_idle_memory(fake):
 
 
 def test_scratch_may_grow_beside_the_capture_of_another_stream(fake):
-    ctx = fake.context(**TINY)
-    assert ctx.append(1) == 0 and ctx.full_attend() == 0
+    ctx = fake.context(n_heads=6, head_dim=128, grid_h=13, grid_w=22, n_blocks=4)
+    assert ctx.append(1) == 0 and ctx.full_attend(stream=78) == 0
     first = fake.attn_part_o()
+    assert fake.is_live(first)
     fake.capture(RELAXED, 77)
     assert ctx.append(3) == 0 and ctx.full_attend(stream=78) == 0
     assert fake.attn_part_o() != first and fake.is_live(fake.attn_part_o())
     assert not fake.capture_invalidated()
+    fake.capture(0, None)
+    twin = fake.context(n_heads=6, head_dim=128, grid_h=13, grid_w=22, n_blocks=4)
+    assert twin.append(1) == 0 and twin.full_attend() == 0 and fake.attn_part_o() == first  # it was kept for others
 
 
 @pytest.mark.parametrize("refusal", ["memory", "capture"])

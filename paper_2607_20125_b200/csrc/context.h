@@ -343,6 +343,7 @@ struct headcast_ctx {
 
   int device = 0;
   ContextMemory memory;
+  bool attn_configured[2] = {false, false}, move_configured = false;  // dynamic shared memory of the kernels (attention: plain, proxy)
   int n_sm = 148;
   int64_t launches = 0;
   bool tracing = false;  // record per-item start/end times in the attention kernel

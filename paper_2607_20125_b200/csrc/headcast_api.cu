@@ -64,15 +64,12 @@ int upload_schedule(headcast_ctx* c, Schedule& s, cudaStream_t st) {
 
 template <int D, bool PROXY>
 int launch_attn_t(headcast_ctx* c, const AttnParams& p, cudaStream_t st) {
-  // the attribute belongs to the (function, device) pair: one flag per device, so that a process that drives several
-  // GPUs sets it on each of them
-  static bool configured[64] = {};
-  int dev = 0;
-  HC_CUDA(c, cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64 || !configured[dev]) {
+  // the attribute belongs to the function in a CUDA context: every headcast_ctx sets it once for itself, whatever GPU it is on
+  // and whatever has been reset before
+  if (!c->attn_configured[PROXY]) {
     HC_CUDA(c, cudaFuncSetAttribute(attn_kernel<D, PROXY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     AttnSmem<D>::DYN_BYTES));
-    if (dev >= 0 && dev < 64) configured[dev] = true;
+    c->attn_configured[PROXY] = true;
   }
   if (c->timing) HC_CUDA(c, cudaEventRecord(c->ev_a, st));
   HC_CUDA(c, launch_pdl(attn_kernel<D, PROXY>, dim3(c->n_sm), dim3(ATTN_THREADS), AttnSmem<D>::DYN_BYTES, st, p));
@@ -250,12 +247,9 @@ bool build_move_maps(headcast_ctx* c, headcast_ctx::MoveMaps& m, const void* k, 
 
 // The same routing as route_block_kernel (RouteParams says which source block feeds which buffer), as bulk tile jobs.
 int launch_move(headcast_ctx* c, const RouteParams& r, int n_src, cudaStream_t st) {
-  static bool configured[64] = {};
-  int dev = 0;
-  HC_CUDA(c, cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64 || !configured[dev]) {
+  if (!c->move_configured) {
     HC_CUDA(c, cudaFuncSetAttribute(move_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MOVE_SMEM_BYTES));
-    if (dev >= 0 && dev < 64) configured[dev] = true;
+    c->move_configured = true;
   }
   MoveParams p;
   std::memset(&p, 0, sizeof(p));

@@ -29,6 +29,7 @@ struct Fake {
   bool invalidated = false;                    // the capture was destroyed by a refused call
   unsigned long long context_id = 1;
   std::map<const void*, std::string> kernels;
+  std::map<const void*, int> smem;             // dynamic shared memory that a kernel may be launched with
   // launches, events, waits and the host's waits for a stream or the device, in order:
   // "L<stream>:<kernel>@<scratch> E<stream>:<event> W<stream>:<event> Y<stream>: S"
   std::string log;
@@ -121,6 +122,7 @@ void fake_device_reset() {  // every allocation is gone, a new context takes the
   fake().from_pool.clear();
   fake().pool.clear();
   fake().busy.clear();
+  fake().smem.clear();
   fake().used = fake().pool_unused = 0;
   ++fake().context_id;
 }
@@ -258,20 +260,24 @@ cudaError_t cudaGetDriverEntryPoint(const char* name, void** fn, unsigned long l
 }
 
 // ------------------------------------------------------------------------------------------ kernels
-cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void* fn, cudaFuncAttribute a, int v) {
+  if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) fake().smem[fn] = v;
+  return cudaSuccess;
+}
 cudaError_t cudaGetSymbolAddress(void** p, const void*) {
   static char scratch[1 << 20];
   *p = scratch;
   return cudaSuccess;
 }
-static cudaError_t launched(const void* fn, void** args, cudaStream_t s) {
+static cudaError_t launched(const void* fn, void** args, size_t smem, cudaStream_t s) {
+  if (smem > 48 << 10 && static_cast<int>(smem) > fake().smem[fn]) return cudaErrorInvalidValue;
   const std::string& name = fake().kernels[fn];
   const void* scratch = fake_saw_launch(name.c_str(), args);
   fake().log += "L" + handle(s) + ":" + name + "@" + handle(scratch) + " ";
   return cudaSuccess;
 }
-cudaError_t cudaLaunchKernel(const void* fn, dim3, dim3, void** args, size_t, cudaStream_t s) { return launched(fn, args, s); }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* fn, void** args) { return launched(fn, args, c->stream); }
+cudaError_t cudaLaunchKernel(const void* fn, dim3, dim3, void** args, size_t smem, cudaStream_t s) { return launched(fn, args, smem, s); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* fn, void** args) { return launched(fn, args, c->dynamicSmemBytes, c->stream); }
 static dim3 pushed_grid, pushed_block;
 static size_t pushed_smem;
 static void* pushed_stream;

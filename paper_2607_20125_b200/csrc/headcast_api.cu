@@ -1244,6 +1244,7 @@ __global__ void __launch_bounds__(256) noalloc_list_kernel(NoAllocScratch* s, in
 
 constexpr int NOALLOC_MAX_DEVICES = 64;
 struct NoAllocDevice {
+  unsigned long long context = 0;     // the CUDA context that the rest was found in: after a device reset it is another one
   NoAllocScratch* scratch = nullptr;  // device address of g_noalloc_scratch on that GPU
   int n_sm = 0;
 };
@@ -1259,11 +1260,13 @@ int noalloc_fail(int code, const char* msg, cudaError_t e = cudaSuccess) {
   return code;
 }
 
-// Once per device, with that device current: the array's name is only a host-side handle, the kernel needs the
+// Once per device and CUDA context, with that device current: the array's name is only a host-side handle, the kernel needs the
 // address cudaGetSymbolAddress reports for the current device.
 int noalloc_setup(int dev) {
   NoAllocDevice& d = g_noalloc_dev[dev];
-  if (d.scratch) return HC_OK;
+  unsigned long long context = 0;
+  const bool known = current_context_id(&context);
+  if (d.scratch && known && d.context == context) return HC_OK;
   cudaDeviceProp prop;
   cudaError_t e = cudaGetDeviceProperties(&prop, dev);
   if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "cudaGetDeviceProperties", e);
@@ -1275,6 +1278,7 @@ int noalloc_setup(int dev) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(attn_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<64>::DYN_BYTES);
   if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "cudaFuncSetAttribute", e);
+  if (!current_context_id(&d.context)) return noalloc_fail(HC_ERR_CUDA, "cuCtxGetId");
   d.n_sm = std::min(prop.multiProcessorCount, NOALLOC_MAX_CTAS);
   d.scratch = static_cast<NoAllocScratch*>(ptr);
   return HC_OK;
@@ -1302,19 +1306,19 @@ int headcast_dense_attend_noalloc(const void* q, const void* k, const void* v, v
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "cudaGetDevice", e);
   if (dev < 0 || dev >= NOALLOC_MAX_DEVICES) return noalloc_fail(HC_ERR_UNSUPPORTED, "device index beyond 63");
-  int rc = noalloc_setup(dev);
-  if (rc != HC_OK) return rc;
-  const NoAllocDevice& d = g_noalloc_dev[dev];
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   {
     // calls share one scratch array: a graph replayed beside other calls would overwrite their work list, so capturing
-    // streams are turned away
+    // streams are turned away.  (This query also makes the device's CUDA context current to a thread that is new to it.)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     e = cudaStreamIsCapturing(st, &cap);
     if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "cudaStreamIsCapturing", e);
     if (cap != cudaStreamCaptureStatusNone)
       return noalloc_fail(HC_ERR_UNSUPPORTED, "headcast_dense_attend_noalloc cannot be called on a capturing stream");
   }
+  int rc = noalloc_setup(dev);
+  if (rc != HC_OK) return rc;
+  const NoAllocDevice& d = g_noalloc_dev[dev];
 
   const uint64_t row_elems = static_cast<uint64_t>(n_heads) * head_dim;
   AttnParams p;

@@ -265,8 +265,8 @@ cudaError_t cudaFuncSetAttribute(const void* fn, cudaFuncAttribute a, int v) {
   return cudaSuccess;
 }
 cudaError_t cudaGetSymbolAddress(void** p, const void*) {
-  static char scratch[1 << 20];
-  *p = scratch;
+  static char scratch[2][1 << 20];
+  *p = scratch[fake().context_id % 2];
   return cudaSuccess;
 }
 static cudaError_t launched(const void* fn, void** args, size_t smem, cudaStream_t s) {

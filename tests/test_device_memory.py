@@ -159,3 +159,14 @@ def test_scratch_that_a_graph_uses_stays_when_another_list_needs_more(fake):
     fake.capacity_left(64 << 20)
     assert ctx.full_attend() == 0 and fake.attn_part_o() != in_graph and fake.is_live(in_graph)
     assert ctx.destroy() == 0 and fake.lib.headcast_release_memory() == 0 and fake.used() == 0
+
+
+def test_the_allocation_free_call_finds_its_array_again_after_a_device_reset(fake):
+    import ctypes
+    buffer = ctypes.create_string_buffer(64)
+    x = (ctypes.addressof(buffer) + 15) & ~15
+    for _ in range(3):
+        for _ in range(2):
+            assert fake.lib.headcast_dense_attend_noalloc(x, x, x, x, 100, 100, 4, 64, 0.0, None) == 0
+            assert fake.noalloc_list_is_the_devices()
+        fake.device_reset()

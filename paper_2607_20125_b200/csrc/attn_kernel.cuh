@@ -16,7 +16,7 @@
 // one tile alone, 2126 for two together), and a tile's softmax and its products follow one another; a step takes about
 // 3050 clk.  With two threads per row, a maximum exchanged through shared memory and the products issued from a diverged
 // lane it took 3600.  Steady-state block at 30 x 52 tokens (12 heads of 128, 7-block window, append + four attends):
-// 1396 -> 1256 us; dense sweep over 7 blocks at 45 x 80 tokens: 4856 -> 4398 us.
+// 1412 -> 1281 us; dense sweep over 7 blocks at 45 x 80 tokens: 4966 -> 4468 us.
 // Which keys a query tile sees is entirely a property of the work item: a row range of one of the
 // cache buffers (whole window, one block, one Spatial cell) or, for the classification's Spatial
 // proxy, a per-frame band of tokens plus an element-wise neighbourhood test.

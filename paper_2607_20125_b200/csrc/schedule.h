@@ -71,7 +71,7 @@ constexpr CostModel COST_MEASURED = {0.90, 2.2, 1.7, 1.1, 1.12};
 // not care.
 constexpr double SHORT_LINE_TILES = 20.0;
 constexpr CostModel COST_SHORT_LINE = {0.86, 2.4, 1.0, 0.75, 1.02};
-constexpr int MIN_PART_TILES = 4;  // never cut a key range into pieces shorter than this
+constexpr int MIN_PART_TILES = 4;  // the line and the queue never cut a key range into pieces shorter than this (short lists: down to one tile)
 
 // The same for work lists with few items per CTA, where the line below has nothing to cut with: its pieces are whole items
 // or at least MIN_PART_TILES long, so five items on 148 SMs stayed five items and a launch took as long as the longest
@@ -536,7 +536,6 @@ void build_dense_schedule(headcast_ctx* c, Schedule& s, int out_mode, bool allow
   s.key_filled = n_filled(c);
 }
 
-// group < 0: every head; 0: Global heads only; 1: Spatial; 2: Sink and Dummy
 // group < 0: every head; else only the heads of one archetype group (0 Global, 1 Spatial, 2 Sink + Dummy), and for
 // groups 0 and 2 only the query rows [q_lo, q_hi) (q_lo a multiple of 256; q_hi < 0: to the end).
 void build_headcast_schedule(headcast_ctx* c, Schedule& s, int group = -1, int q_lo = 0, int q_hi = -1) {

@@ -123,13 +123,7 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 // ---------------------------------------------------------------------------------------------
 // TMA: 2-D tiled load, completion on an mbarrier (no multicast anywhere in this library)
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y)
-      : "memory");
-}
-// The same load with an L2 eviction policy (from l2_policy_*): K/V that are read once should not push out K/V that
+// With an L2 eviction policy (from l2_policy_*): K/V that are read once should not push out K/V that
 // other CTAs will read again.
 __device__ __forceinline__ void tma_load_2d_hint(void* smem_dst, const CUtensorMap* map, int x, int y, uint64_t* bar,
                                                  uint64_t policy) {
@@ -152,9 +146,6 @@ __device__ __forceinline__ uint64_t l2_policy_evict_normal() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
   return p;
-}
-__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -328,13 +319,13 @@ __device__ __forceinline__ float ex2_approx(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// two floats -> packed bf16x2 (lo in bits 0..15), round to nearest even
 // acc_lo += low bf16 of pk, acc_hi += high bf16 of pk, in fp32 (mixed-precision add: no unpacking instructions)
 __device__ __forceinline__ void add_bf16x2_to_f32(uint32_t pk, float& acc_lo, float& acc_hi) {
   asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}"
       : "+f"(acc_lo), "+f"(acc_hi)
       : "r"(pk));
 }
+// two floats -> packed bf16x2 (lo in bits 0..15), round to nearest even
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   uint32_t r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
@@ -365,17 +356,6 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-// 2^lo and 2^hi with ONE special-function operation: both exponents are rounded to fp16 (<= 2^-11 relative
-// for |x| < 16, exact -inf -> 0) and exponentiated as a packed pair; the results come back as fp32.
-__device__ __forceinline__ void ex2_pair(float lo, float hi, float& e_lo, float& e_hi) {
-  uint32_t h, e;
-  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(hi), "f"(lo));
-  asm("ex2.approx.f16x2 %0, %1;" : "=r"(e) : "r"(h));
-  asm("{\n\t.reg .b16 l, u;\n\tmov.b32 {l, u}, %2;\n\tcvt.f32.f16 %0, l;\n\tcvt.f32.f16 %1, u;\n\t}"
-      : "=f"(e_lo), "=f"(e_hi)
-      : "r"(e));
-}
-
 // 2^x for a packed pair WITHOUT the special-function unit (which can only deliver 16 results per clock per
 // SM, exactly what the tensor pipe consumes at head_dim 128): round x to an integer n with the 1.5 * 2^23
 // trick, evaluate a cubic for 2^(x - n) on [-1/2, 1/2] (relative error 7.5e-5, far below the bf16 rounding of P),
@@ -396,21 +376,6 @@ __device__ __forceinline__ void ex2_poly_pair(uint64_t x2, float& e_lo, float& e
   unpack_f32x2(p2, p_lo, p_hi);
   e_lo = __uint_as_float(__float_as_uint(p_lo) + (__float_as_uint(t_lo) << 23));
   e_hi = __uint_as_float(__float_as_uint(p_hi) + (__float_as_uint(t_hi) << 23));
-}
-
-// 2^lo and 2^hi as packed bf16x2 with ONE special-function operation on bf16 inputs.  The two exponents
-// are rounded to bf16 with integer adds and a byte permute (no conversion instruction).
-__device__ __forceinline__ uint32_t ex2_pair_bf16(float lo, float hi) {
-  uint32_t a = __float_as_uint(lo) + 0x8000u, b = __float_as_uint(hi) + 0x8000u, x, e;
-  asm("prmt.b32 %0, %1, %2, 0x7632;" : "=r"(x) : "r"(a), "r"(b));
-  asm("ex2.approx.ftz.bf16x2 %0, %1;" : "=r"(e) : "r"(x));
-  return e;
-}
-__device__ __forceinline__ uint32_t ex2_pair_bf16_cvt(float lo, float hi) {
-  uint32_t x, e;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(hi), "f"(lo));
-  asm("ex2.approx.ftz.bf16x2 %0, %1;" : "=r"(e) : "r"(x));
-  return e;
 }
 
 // Byte offset of the 16-byte chunk `chunk` (0..7) of row `row` inside a [rows][64] bf16 block stored with

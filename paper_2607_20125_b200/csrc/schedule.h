@@ -68,7 +68,8 @@ constexpr CostModel COST_MEASURED = {0.90, 2.2, 1.7, 1.1, 1.12};
 // per block against 127 with the measured costs; 14, 31 x 46, four heads: 173 against 182; 18, 25 x 33: 187 against 192).
 // Longer lists are charged too little by these (25, 15 x 27, sixteen heads: 251 us against 247; 33, 30 x 49, eight heads: 334
 // against 320; 190, 55 x 87, four heads, cells of 6, two-block Sink and Dummy heads: 1915 against 1600); 480P to 1080P do
-// not care.
+// not care.  These constants are an earlier kernel's fit and describe nothing of the present one: they are kept for where their
+// cuts fall.  The layouts that come out are judged against each other by the measured costs alone (short_end_of_line).
 constexpr double SHORT_LINE_TILES = 20.0;
 constexpr CostModel COST_SHORT_LINE = {0.86, 2.4, 1.0, 0.75, 1.02};
 constexpr int MIN_PART_TILES = 4;  // the line and the queue never cut a key range into pieces shorter than this (short lists: down to one tile)

@@ -130,3 +130,34 @@ def test_destroying_a_context_beside_a_relaxed_capture_keeps_results_right():
     runtime.cudaGetLastError()
     torch.cuda.synchronize()
     one_life(w)
+
+
+def test_two_contexts_on_recycled_memory_and_streams_of_their_own():
+    import torch
+    from paper_2607_20125_b200.binding import HeadCast
+    from test_gpu_parity import to_dev
+    w = synth.small()
+    kv = [tuple(to_dev(x) for x in synth.make_kv(w, b)) for b in range(2)]
+    q = to_dev(synth.make_q(w, 1, 0))
+
+    def start(stream, out):  # create, append, attend: enqueued on the stream, not waited for
+        with torch.cuda.stream(stream):
+            hc = HeadCast.from_workload(w)
+            for k, v in kv:
+                hc.append(k, v)
+            for _ in range(4):
+                hc.full_attend(q, out)
+        return hc
+
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    want = torch.empty_like(q)
+    torch.cuda.synchronize()
+    start(streams[0], want).destroy()
+    for turn in range(4):
+        outs = [torch.full_like(q, float("nan")) for _ in streams]
+        torch.cuda.synchronize()
+        pair = [start(s, o) for s, o in zip(streams, outs)]
+        pair[turn % 2].destroy()  # the other one's work may be in flight
+        pair[1 - turn % 2].destroy()
+        torch.cuda.synchronize()
+        assert all(torch.equal(o, want) for o in outs)

@@ -105,7 +105,10 @@ class BlockCache {
   }
   // The same for memory of get_mono.  Its free is ordered by a stream and does not wait for the others.
   void put_mono(void* ptr, bool idle) {
-    if (idle && cudaFreeAsync(ptr, nullptr) == cudaSuccess) return;
+    if (idle) {
+      if (cudaFreeAsync(ptr, nullptr) == cudaSuccess) return;
+      cudaGetLastError();
+    }
     std::lock_guard<std::mutex> hold(lock_);
     aside_.push_back(ptr);
   }
@@ -118,6 +121,7 @@ class BlockCache {
       aside.swap(aside_);
     }
     const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+    if (!idle) cudaGetLastError();  // (dealt with here and below: no later call is to report it)
     std::lock_guard<std::mutex> hold(lock_);
     if (idle)
       for (void* ptr : aside) give_up(ptr);
@@ -161,7 +165,9 @@ class BlockCache {
     return cudaSuccess;
   }
   void give_up(void* ptr) {
-    if (cudaFree(ptr) != cudaSuccess) aside_.push_back(ptr);
+    if (cudaFree(ptr) == cudaSuccess) return;
+    cudaGetLastError();
+    aside_.push_back(ptr);
   }
   static size_t round_up(size_t bytes) {
     if (bytes > (size_t(1) << 20)) return (bytes + (size_t(2) << 20) - 1) >> 21 << 21;
@@ -230,6 +236,11 @@ struct DevBuf {  // grow-only device array of the context's device
   }
 
  private:
+  static bool done(cudaStream_t st) {
+    if (cudaStreamSynchronize(st) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
+  }
   cudaError_t grow(ContextMemory& memory, size_t n, cudaStream_t st, bool in_order) {
     // while `st` is captured the cache stands aside: cudaMalloc then says whether memory may be taken in this capture mode
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
@@ -240,13 +251,13 @@ struct DevBuf {  // grow-only device array of the context's device
     size_t bytes = 0;
     e = memory.cache->get(&bigger, n * sizeof(T), &bytes, capturing);
     if (e == cudaErrorMemoryAllocation && !memory.captured) {  // what this context does not need any more comes first
-      if (in_order) release(*memory.cache, ptr && cudaStreamSynchronize(st) == cudaSuccess);
+      if (ptr && in_order) release(*memory.cache, done(st));
       if (!memory.outgrown.empty() && memory.cache->wait_idle()) memory.release(true);
       e = memory.cache->get(&bigger, n * sizeof(T), &bytes, capturing);
     }
     if (e != cudaSuccess) return e;
     if (ptr && in_order)
-      release(*memory.cache, cudaStreamSynchronize(st) == cudaSuccess);
+      release(*memory.cache, done(st));
     else
       retire(memory);
     ptr = static_cast<T*>(bigger);
@@ -373,9 +384,11 @@ int fail(headcast_ctx* c, int code, const char* fmt, ...) {
 #define HC_CUDA(c, expr)                                                                           \
   do {                                                                                             \
     cudaError_t e_ = (expr);                                                                       \
-    if (e_ != cudaSuccess)                                                                         \
+    if (e_ != cudaSuccess) {                                                                       \
+      cudaGetLastError(); /* reported here, and by no later call */                                \
       return fail((c), e_ == cudaErrorMemoryAllocation ? HC_ERR_NOMEM : HC_ERR_CUDA, "%s: %s", #expr, \
                   cudaGetErrorString(e_));                                                         \
+    }                                                                                              \
   } while (0)
 
 std::vector<int> default_edges(int grid, int cell) {

@@ -567,6 +567,7 @@ int headcast_create(const headcast_config* cfg, headcast_ctx** out) {
   if (rc == HC_OK) rc = build_maps(c);
   if (rc == HC_OK && !cache.wait_idle()) rc = HC_ERR_CUDA;
   if (rc != HC_OK) {
+    cudaGetLastError();
     headcast_destroy(c);
     return rc;
   }
@@ -613,7 +614,6 @@ int headcast_destroy(headcast_ctx* c) {
   c->cls_scores.release(cache, idle);
   c->cls_labels.release(cache, idle);
   c->memory.release(idle);
-  if (!idle) cudaGetLastError();  // the refusal is dealt with, no later call is to report it
   if (current != c->device) cudaSetDevice(current);
   delete c;
   return HC_OK;
@@ -1253,6 +1253,7 @@ NoAllocDevice g_noalloc_dev[NOALLOC_MAX_DEVICES];
 char g_noalloc_error[256] = "";
 
 int noalloc_fail(int code, const char* msg, cudaError_t e = cudaSuccess) {
+  if (e != cudaSuccess) cudaGetLastError();  // reported here, and by no later call
   if (e != cudaSuccess)
     snprintf(g_noalloc_error, sizeof(g_noalloc_error), "%s: %s", msg, cudaGetErrorString(e));
   else

@@ -82,6 +82,9 @@ class FakeContext:
     def classify(self, stream=0):
         return self.lib.headcast_classify(self.ptr, self.tensor, (C.c_int32 * self.cfg.n_heads)(), None, stream)
 
+    def export(self, head=0, stream=0):
+        return self.lib.headcast_export_cache(self.ptr, head, self.tensor, self.tensor, None, stream)
+
     def destroy(self):
         rc = self.lib.headcast_destroy(self.ptr)
         self.ptr = C.c_void_p()

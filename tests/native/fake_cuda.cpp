@@ -28,6 +28,7 @@ struct Fake {
   cudaStream_t capture_stream = nullptr;
   bool invalidated = false;                    // the capture was destroyed by a refused call
   unsigned long long context_id = 1;
+  cudaError_t last_error = cudaSuccess;        // what the next cudaGetLastError reports
   std::map<const void*, std::string> kernels;
   std::map<const void*, int> smem;             // dynamic shared memory that a kernel may be launched with
   // launches, events, waits and the host's waits for a stream or the device, in order:
@@ -40,9 +41,14 @@ Fake& fake() {  // the library registers its kernels before this file's globals 
   return state;
 }
 
+cudaError_t failed(cudaError_t e) {
+  fake().last_error = e;
+  return e;
+}
+
 cudaError_t refused() {
   fake().invalidated = true;
-  return cudaErrorStreamCaptureUnsupported;
+  return failed(cudaErrorStreamCaptureUnsupported);
 }
 
 void finish() { fake().busy.clear(); }
@@ -60,7 +66,7 @@ bool write_to(void* p) {  // by the device
 }
 
 cudaError_t take(void** p, size_t bytes) {
-  if (fake().used + static_cast<long long>(bytes) > fake().capacity) return cudaErrorMemoryAllocation;
+  if (fake().used + static_cast<long long>(bytes) > fake().capacity) return failed(cudaErrorMemoryAllocation);
   char* c = static_cast<char*>(std::aligned_alloc(4096, (bytes + 4095) / 4096 * 4096));
   fake().used += bytes;
   fake().live[c] = bytes;
@@ -133,7 +139,7 @@ cudaError_t cudaFree(void* p) {
   if (!p) return cudaSuccess;
   if (fake().capture == 2) return refused();
   char* c = static_cast<char*>(p);
-  if (!fake().live.count(c)) return cudaErrorInvalidValue;
+  if (!fake().live.count(c)) return failed(cudaErrorInvalidValue);
   if (fake().from_pool.count(c)) {
     to_pool(c);
     return cudaSuccess;
@@ -151,7 +157,7 @@ cudaError_t cudaMemPoolCreate(cudaMemPool_t* pool, const cudaMemPoolProps*) {
 cudaError_t cudaMemPoolDestroy(cudaMemPool_t) { return cudaSuccess; }
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
 cudaError_t cudaMemPoolTrimTo(cudaMemPool_t pool, size_t) {
-  if (reinterpret_cast<unsigned long long>(pool) != fake().context_id) return cudaErrorInvalidValue;
+  if (reinterpret_cast<unsigned long long>(pool) != fake().context_id) return failed(cudaErrorInvalidValue);
   for (auto& e : fake().pool) {
     fake().used -= e.first;
     std::free(e.second);
@@ -162,7 +168,7 @@ cudaError_t cudaMemPoolTrimTo(cudaMemPool_t pool, size_t) {
 }
 cudaError_t cudaMallocFromPoolAsync(void** p, size_t bytes, cudaMemPool_t pool, cudaStream_t) {
   if (fake().capture == 2) return refused();
-  if (reinterpret_cast<unsigned long long>(pool) != fake().context_id) return cudaErrorInvalidValue;
+  if (reinterpret_cast<unsigned long long>(pool) != fake().context_id) return failed(cudaErrorInvalidValue);
   auto it = fake().pool.find(bytes);
   if (it != fake().pool.end()) {
     fake().live[it->second] = bytes;
@@ -178,7 +184,7 @@ cudaError_t cudaMallocFromPoolAsync(void** p, size_t bytes, cudaMemPool_t pool, 
 }
 cudaError_t cudaFreeAsync(void* p, cudaStream_t) {
   if (fake().capture == 2) return refused();
-  if (!fake().from_pool.count(static_cast<char*>(p))) return cudaErrorInvalidValue;
+  if (!fake().from_pool.count(static_cast<char*>(p))) return failed(cudaErrorInvalidValue);
   to_pool(static_cast<char*>(p));
   return cudaSuccess;
 }
@@ -251,7 +257,11 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
 }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 0.f; return cudaSuccess; }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError() {
+  const cudaError_t e = fake().last_error;
+  fake().last_error = cudaSuccess;
+  return e;
+}
 const char* cudaGetErrorString(cudaError_t) { return "fake error"; }
 cudaError_t cudaGetDriverEntryPoint(const char* name, void** fn, unsigned long long, cudaDriverEntryPointQueryResult* q) {
   *fn = std::strcmp(name, "cuCtxGetId") == 0 ? reinterpret_cast<void*>(context_id) : reinterpret_cast<void*>(encode_tiled);
@@ -270,7 +280,7 @@ cudaError_t cudaGetSymbolAddress(void** p, const void*) {
   return cudaSuccess;
 }
 static cudaError_t launched(const void* fn, void** args, size_t smem, cudaStream_t s) {
-  if (smem > 48 << 10 && static_cast<int>(smem) > fake().smem[fn]) return cudaErrorInvalidValue;
+  if (smem > 48 << 10 && static_cast<int>(smem) > fake().smem[fn]) return failed(cudaErrorInvalidValue);
   const std::string& name = fake().kernels[fn];
   const void* scratch = fake_saw_launch(name.c_str(), args);
   fake().log += "L" + handle(s) + ":" + name + "@" + handle(scratch) + " ";

@@ -32,8 +32,8 @@ enum { MAP_MONO = 0, MAP_SD = 1, MAP_GLOBAL = 2, MAP_SPATIAL = 3, N_MAP_PAIRS = 
 // with giving them back; with cudaMalloc and cudaFree that took half of the 14.8 ms from create to destroy (3.5 us per MB
 // and 55 us per small buffer each way), with blocks kept from the context before it takes 0.3 ms.  Per GPU at most
 // CACHE_KEEP_BYTES are kept, the blocks given back last; older ones go to the system then and there, all of them and what
-// the pool holds unused when an allocation of either kind fails.  A block is kept only if the device has been waited for
-// since its last use, so it may serve any stream.
+// the pool holds unused when an allocation of either kind fails.  A block is kept only if its last use has been waited
+// for (see put), so it may serve any stream.
 constexpr size_t CACHE_KEEP_BYTES = size_t(384) << 20;
 constexpr unsigned long long MONO_KEEP_BYTES = 256ull << 20;  // the same for the monolithic caches, see get_mono
 
@@ -73,8 +73,9 @@ class BlockCache {
     if (got) *got = need;
     return e;
   }
-  // Gives a block back.  idle: wait_idle() has returned true since its last use.  If not, the block goes through cudaFree,
-  // which waits itself, or refuses beside a stream capture: then it is set aside until the device can be waited for.
+  // Gives a block back.  idle: since its last use the device has been waited for (wait_idle), or the one stream that orders all
+  // its uses.  If not, the block goes through cudaFree, which waits itself, or refuses beside a stream capture: then it is set
+  // aside until the device can be waited for.
   void put(void* ptr, bool idle) {
     std::lock_guard<std::mutex> hold(lock_);
     auto it = live_.find(ptr);

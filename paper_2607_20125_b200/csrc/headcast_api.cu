@@ -180,7 +180,7 @@ int run_schedule(headcast_ctx* c, Schedule& s, const void* q, void* out, bool pr
   if (!s.combine.empty()) {
     const unsigned blocks = static_cast<unsigned>(s.combine.size() - s.n_long) * (128 / COMBINE_ROWS) + static_cast<unsigned>(s.n_long) * 128;
     HC_CUDA(c, launch_pdl(c->D == 128 ? combine_kernel<128> : combine_kernel<64>, dim3(blocks), dim3(COMBINE_ROWS * (c->D / 8)), 0, st,
-                          s.combine_dev.ptr, s.n_long, c->cells_dev, c->part_o.ptr, c->part_ml.ptr, p.out, c->H, c->T_f, c->G_w));
+                          s.combine_dev.ptr, s.n_long, c->cells_dev, c->part_o.ptr, c->part_ml.ptr, p.out, c->H, c->T_f, c->G_w, true));
     ++c->launches;
   }
   if (shares_scratch && c->scratch_done) HC_CUDA(c, cudaEventRecord(c->scratch_done, st));

@@ -37,59 +37,63 @@ struct ClsGroup {
   int32_t head, q_start, q_count[2], first_part, n_parts;
 };
 
+// Both merges of a classification wait for memory as combine_kernel does: one pass, batches of parts (see MERGE_BATCH).  A pair
+// has two or three parts here, and these kernels hold more per thread.  9 x 12 tokens, eight heads, four blocks: 110 -> 99 us for the
+// whole classification; 30 x 52 tokens, twelve heads, two blocks: 482 -> 475 (three parts at a time 486, four 490).
+constexpr int CLS_MERGE_BATCH = 2;
+
 template <int D>
 __global__ void __launch_bounds__(COMBINE_ROWS * (D / 8))
 cls_combine_kernel(const ClsGroup* groups, const ClsPart* parts, const float* part_o, const float2* part_ml, float* o_ref,
                    float* lse_ref, float* tok, int n_heads, int block_tokens) {
   pdl_launch_dependents();
-  pdl_wait();
   constexpr int CHUNKS = D / 8;
   constexpr int BLOCKS_PER_TILE = 128 / COMBINE_ROWS;
-  const ClsGroup g = groups[blockIdx.x / (2 * BLOCKS_PER_TILE)];
+  const ClsGroup g = groups[blockIdx.x / (2 * BLOCKS_PER_TILE)];  // complete before the launch was made
+  pdl_wait();
   const int sub = (blockIdx.x / BLOCKS_PER_TILE) & 1;
   const int r = (blockIdx.x % BLOCKS_PER_TILE) * COMBINE_ROWS + threadIdx.x / CHUNKS;
   const int c = threadIdx.x % CHUNKS;
   const bool valid = r < g.q_count[sub];  // rows past the block's end do the arithmetic on zeros and write nothing
   const ClsPart* pp = parts + g.first_part;
   const int n_parts = valid ? g.n_parts : 0;
-  float m[3] = {-INFINITY, -INFINITY, -INFINITY};  // all, first, newest
-  for (int i = 0; i < n_parts; ++i) {
-    const float mi = part_ml[static_cast<size_t>(pp[i].slot) * 256 + sub * 128 + r].x;
-    m[0] = fmaxf(m[0], mi);
-    if (pp[i].tag == 0) m[1] = fmaxf(m[1], mi);
-    if (pp[i].tag == 2) m[2] = fmaxf(m[2], mi);
-  }
-  float acc[3][8], l[3] = {0.f, 0.f, 0.f};
+  RowMerge set[3];  // all, first, newest
+  for (int i0 = 0; i0 < n_parts; i0 += CLS_MERGE_BATCH) {
+    ClsPart part[CLS_MERGE_BATCH];
+    float2 ml[CLS_MERGE_BATCH];
+    float4 a[CLS_MERGE_BATCH], b[CLS_MERGE_BATCH];
 #pragma unroll
-  for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < CLS_MERGE_BATCH; ++k) part[k] = pp[min(i0 + k, n_parts - 1)];  // past the end: the last one again, not added
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[k][j] = 0.f;
-  for (int i = 0; i < n_parts; ++i) {
-    const size_t row = static_cast<size_t>(pp[i].slot) * 256 + sub * 128 + r;
-    const float2 ml = part_ml[row];
-    if (ml.x == -INFINITY) continue;
-    const float4* src = reinterpret_cast<const float4*>(part_o + row * D + c * 8);
-    const float4 a = src[0], b = src[1];
-    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    for (int k = 0; k < CLS_MERGE_BATCH; ++k) {
+      const size_t row = static_cast<size_t>(part[k].slot) * 256 + sub * 128 + r;
+      ml[k] = part_ml[row];
+      const float4* src = reinterpret_cast<const float4*>(part_o + row * D + c * 8);
+      a[k] = ld_stream_f4(src);
+      b[k] = ld_stream_f4(src + 1);
+      if (i0 + k >= n_parts) ml[k].x = -INFINITY;
+    }
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const bool in_set = (k == 0) || (k == 1 && pp[i].tag == 0) || (k == 2 && pp[i].tag == 2);
-      if (!in_set) continue;
-      const float wgt = ex2_approx(ml.x - m[k]);
-      l[k] += wgt * ml.y;
+    for (int s = 0; s < 3; ++s) {
+      float to = -INFINITY;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) acc[k][j] += wgt * v[j];
+      for (int k = 0; k < CLS_MERGE_BATCH; ++k)
+        if (s == 0 || part[k].tag == 2 * (s - 1)) to = fmaxf(to, ml[k].x);
+      set[s].raise_reference(to);
+#pragma unroll
+      for (int k = 0; k < CLS_MERGE_BATCH; ++k)
+        if (s == 0 || part[k].tag == 2 * (s - 1)) set[s].add(ml[k], a[k], b[k]);
     }
   }
   float dot[2] = {0.f, 0.f}, nrm[3] = {0.f, 0.f, 0.f};
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const float inv = l[k] > 0.f ? 1.f / l[k] : 0.f;
+    const float inv = set[k].l > 0.f ? 1.f / set[k].l : 0.f;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      acc[k][j] *= inv;
-      nrm[k] += acc[k][j] * acc[k][j];
-      if (k > 0) dot[k - 1] += acc[k][j] * acc[0][j];
+      set[k].acc[j] *= inv;
+      nrm[k] += set[k].acc[j] * set[k].acc[j];
+      if (k > 0) dot[k - 1] += set[k].acc[j] * set[0].acc[j];
     }
   }
 #pragma unroll
@@ -100,13 +104,13 @@ cls_combine_kernel(const ClsGroup* groups, const ClsPart* parts, const float* pa
   const int token = g.q_start + sub * 128 + r;
   const size_t idx = static_cast<size_t>(token) * n_heads + g.head;
   float4* dst = reinterpret_cast<float4*>(o_ref + idx * D + c * 8);
-  dst[0] = make_float4(acc[0][0], acc[0][1], acc[0][2], acc[0][3]);
-  dst[1] = make_float4(acc[0][4], acc[0][5], acc[0][6], acc[0][7]);
+  dst[0] = make_float4(set[0].acc[0], set[0].acc[1], set[0].acc[2], set[0].acc[3]);
+  dst[1] = make_float4(set[0].acc[4], set[0].acc[5], set[0].acc[6], set[0].acc[7]);
   if (c == 0) {
     const float ln2 = 0.6931471805599453f;
     float lse[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) lse[k] = (l[k] > 0.f) ? m[k] * ln2 + __logf(l[k]) : -INFINITY;
+    for (int k = 0; k < 3; ++k) lse[k] = (set[k].l > 0.f) ? set[k].m * ln2 + __logf(set[k].l) : -INFINITY;
     lse_ref[idx] = lse[0];
     const size_t hl = static_cast<size_t>(n_heads) * block_tokens, at = static_cast<size_t>(g.head) * block_tokens + token;
     tok[TOK_COS_SINK * hl + at] = cosine(dot[0], nrm[1], nrm[0]);
@@ -126,31 +130,16 @@ proxy_combine_kernel(const ClsGroup* groups, const ClsPart* parts, const float* 
                      const float* part_mid, const float* o_ref, const float* lse_ref, float* tok, int n_heads,
                      int block_tokens) {
   pdl_launch_dependents();
-  pdl_wait();
   constexpr int CHUNKS = D / 8;
   constexpr int BLOCKS_PER_TILE = 128 / COMBINE_ROWS;
-  const ClsGroup g = groups[blockIdx.x / (2 * BLOCKS_PER_TILE)];
+  const ClsGroup g = groups[blockIdx.x / (2 * BLOCKS_PER_TILE)];  // complete before the launch was made
+  pdl_wait();
   const int sub = (blockIdx.x / BLOCKS_PER_TILE) & 1;
   const int r = (blockIdx.x % BLOCKS_PER_TILE) * COMBINE_ROWS + threadIdx.x / CHUNKS;
   const int c = threadIdx.x % CHUNKS;
   const bool valid = r < g.q_count[sub];
   const ClsPart* pp = parts + g.first_part;
   const int n_parts = valid ? g.n_parts : 0;
-  float m = -INFINITY;
-  for (int i = 0; i < n_parts; ++i) m = fmaxf(m, part_ml[static_cast<size_t>(pp[i].slot) * 256 + sub * 128 + r].x);
-  float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0}, l = 0.f, l_mid = 0.f;
-  for (int i = 0; i < n_parts; ++i) {
-    const size_t row = static_cast<size_t>(pp[i].slot) * 256 + sub * 128 + r;
-    const float2 ml = part_ml[row];
-    if (ml.x == -INFINITY) continue;
-    const float wgt = ex2_approx(ml.x - m);
-    l += wgt * ml.y;
-    l_mid += wgt * part_mid[row];
-    const float4* src = reinterpret_cast<const float4*>(part_o + row * D + c * 8);
-    const float4 a = src[0], b = src[1];
-    acc[0] += wgt * a.x; acc[1] += wgt * a.y; acc[2] += wgt * a.z; acc[3] += wgt * a.w;
-    acc[4] += wgt * b.x; acc[5] += wgt * b.y; acc[6] += wgt * b.z; acc[7] += wgt * b.w;
-  }
   const int token = g.q_start + sub * 128 + r;
   const size_t idx = static_cast<size_t>(valid ? token : 0) * n_heads + g.head;
   float ref[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -159,11 +148,42 @@ proxy_combine_kernel(const ClsGroup* groups, const ClsPart* parts, const float* 
     const float4 a = src[0], b = src[1];
     ref[0] = a.x; ref[1] = a.y; ref[2] = a.z; ref[3] = a.w; ref[4] = b.x; ref[5] = b.y; ref[6] = b.z; ref[7] = b.w;
   }
-  const float inv = l > 0.f ? 1.f / l : 0.f;
+  RowMerge row;
+  float l_mid = 0.f;
+  for (int i0 = 0; i0 < n_parts; i0 += CLS_MERGE_BATCH) {
+    int32_t slot[CLS_MERGE_BATCH];
+    float2 ml[CLS_MERGE_BATCH];
+    float mid[CLS_MERGE_BATCH];
+    float4 a[CLS_MERGE_BATCH], b[CLS_MERGE_BATCH];
+#pragma unroll
+    for (int k = 0; k < CLS_MERGE_BATCH; ++k) slot[k] = pp[min(i0 + k, n_parts - 1)].slot;  // past the end: the last one again, not added
+    float to = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < CLS_MERGE_BATCH; ++k) {
+      const size_t at = static_cast<size_t>(slot[k]) * 256 + sub * 128 + r;
+      ml[k] = part_ml[at];
+      mid[k] = part_mid[at];
+      const float4* src = reinterpret_cast<const float4*>(part_o + at * D + c * 8);
+      a[k] = ld_stream_f4(src);
+      b[k] = ld_stream_f4(src + 1);
+      if (i0 + k >= n_parts) ml[k].x = -INFINITY;
+    }
+#pragma unroll
+    for (int k = 0; k < CLS_MERGE_BATCH; ++k) to = fmaxf(to, ml[k].x);
+    const float before = row.m;
+    row.raise_reference(to);
+    if (before != -INFINITY) l_mid *= ex2_approx(before - row.m);
+#pragma unroll
+    for (int k = 0; k < CLS_MERGE_BATCH; ++k) {
+      const float w = row.add(ml[k], a[k], b[k]);
+      if (w != 0.f) l_mid += w * mid[k];
+    }
+  }
+  const float inv = row.l > 0.f ? 1.f / row.l : 0.f;
   float dot = 0.f, n_sp = 0.f, n_ref = 0.f, sq = 0.f;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    const float x = acc[j] * inv;
+    const float x = row.acc[j] * inv;
     dot += x * ref[j];
     n_sp += x * x;
     n_ref += ref[j] * ref[j];
@@ -176,8 +196,8 @@ proxy_combine_kernel(const ClsGroup* groups, const ClsPart* parts, const float* 
   if (!valid || c != 0) return;
   const float ln2 = 0.6931471805599453f;
   const float l_ref = lse_ref[idx];
-  const float lse_sp = (l > 0.f) ? m * ln2 + __logf(l) : -INFINITY;
-  const float lse_mid = (l_mid > 0.f) ? m * ln2 + __logf(l_mid) : -INFINITY;
+  const float lse_sp = (row.l > 0.f) ? row.m * ln2 + __logf(row.l) : -INFINITY;
+  const float lse_mid = (l_mid > 0.f) ? row.m * ln2 + __logf(l_mid) : -INFINITY;
   const size_t hl = static_cast<size_t>(n_heads) * block_tokens, at = static_cast<size_t>(g.head) * block_tokens + token;
   tok[TOK_COS_SPATIAL * hl + at] = cosine(dot, n_sp, n_ref);
   tok[TOK_SQERR * hl + at] = sq;

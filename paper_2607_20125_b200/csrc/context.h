@@ -330,7 +330,7 @@ struct headcast_ctx {
   MoveMaps move_mono;
   MoveMaps move_recent[8];
   int move_next = 0;
-  int32_t* status_dev = nullptr;
+  int32_t* status_dev = nullptr;  // followed by the scores and labels of the last classification, see status_words
   int32_t* dyn_counter_dev = nullptr;  // [2]: next queue position, CTAs done (the last one clears both)
 
   Schedule sched_dense, sched_hc, sched_cls, sched_proxy;
@@ -350,8 +350,7 @@ struct headcast_ctx {
   int stream_changes = 0;
   std::vector<int32_t*> old_counters;  // of streams that were left, see dyn_counter_dev
   cudaEvent_t scratch_done = nullptr;
-  DevBuf<float> cls_o, cls_lse, cls_tok, cls_scores;
-  DevBuf<int32_t> cls_labels;
+  DevBuf<float> cls_o, cls_lse, cls_tok;
 
   int device = 0;
   ContextMemory memory;

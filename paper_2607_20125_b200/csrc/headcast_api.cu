@@ -354,10 +354,10 @@ int launch_route(headcast_ctx* c, RouteParams& r, int n_src, cudaStream_t st) {
   return HC_OK;
 }
 
-int read_status(headcast_ctx* c, cudaStream_t st) {
-  int32_t status = 0;
-  HC_CUDA(c, cudaMemcpyAsync(&status, c->status_dev, sizeof(status), cudaMemcpyDeviceToHost, st));
-  HC_CUDA(c, cudaStreamSynchronize(st));
+// Words at status_dev: the status, then the scores and the labels of the last classification.
+size_t status_words(const headcast_ctx* c) { return 1 + static_cast<size_t>(c->H) * (HC_N_SCORES + 1); }
+
+int report_status(headcast_ctx* c, int32_t status, cudaStream_t st) {
   if (status != 0) {
     cudaMemsetAsync(c->status_dev, 0, sizeof(int32_t), st);
     // a kernel that gave up may have left the queue half drawn
@@ -366,6 +366,13 @@ int read_status(headcast_ctx* c, cudaStream_t st) {
     return fail(c, HC_ERR_TIMEOUT, "a kernel gave up on a bounded wait (site %d)", status);
   }
   return HC_OK;
+}
+
+int read_status(headcast_ctx* c, cudaStream_t st) {
+  int32_t status = 0;
+  HC_CUDA(c, cudaMemcpyAsync(&status, c->status_dev, sizeof(status), cudaMemcpyDeviceToHost, st));
+  HC_CUDA(c, cudaStreamSynchronize(st));
+  return report_status(c, status, st);
 }
 
 void assign_classes(headcast_ctx* c) {
@@ -542,7 +549,7 @@ int headcast_create(const headcast_config* cfg, headcast_ctx** out) {
   get(&c->sp_base, c->T_f * sizeof(int32_t));
   get(&c->sp_nc, c->T_f * sizeof(int32_t));
   get(&c->cells_dev, c->cells.size() * sizeof(CellGeom));
-  get(&c->status_dev, sizeof(int32_t));
+  get(&c->status_dev, status_words(c) * sizeof(int32_t));
   get(&c->dyn_counter_dev, 2 * sizeof(int32_t));
   if (c->move_ok) get(&c->move_boxes_dev, std::max<size_t>(1, c->move_boxes.size()) * sizeof(MoveBox));
   if (e == cudaSuccess) {
@@ -611,8 +618,6 @@ int headcast_destroy(headcast_ctx* c) {
   c->cls_o.release(cache, idle);
   c->cls_lse.release(cache, idle);
   c->cls_tok.release(cache, idle);
-  c->cls_scores.release(cache, idle);
-  c->cls_labels.release(cache, idle);
   c->memory.release(idle);
   if (current != c->device) cudaSetDevice(current);
   delete c;
@@ -720,8 +725,6 @@ int headcast_classify(headcast_ctx* c, const void* q, int32_t* labels_host, floa
   HC_CUDA(c, c->cls_o.reserve(c->memory, rows * c->D, st));  // the reference output (fp32); the proxy outputs never leave registers
   HC_CUDA(c, c->cls_lse.reserve(c->memory, rows, st));
   HC_CUDA(c, c->cls_tok.reserve(c->memory, TOK_N * rows, st));
-  HC_CUDA(c, c->cls_scores.reserve(c->memory, static_cast<size_t>(c->H) * HC_N_SCORES, st));
-  HC_CUDA(c, c->cls_labels.reserve(c->memory, c->H, st));
   const int newest = c->slots.back();
   const int cls_key = n_filled(c) * 64 + newest;  // the work lists depend on the fill and on where the newest block sits
   if (c->sched_cls.key_filled != cls_key) {
@@ -843,8 +846,8 @@ int headcast_classify(headcast_ctx* c, const void* q, int32_t* labels_host, floa
   {
     DecideParams d;
     d.tok = c->cls_tok.ptr;
-    d.scores = c->cls_scores.ptr;
-    d.labels = c->cls_labels.ptr;
+    d.scores = reinterpret_cast<float*>(c->status_dev + 1);
+    d.labels = c->status_dev + 1 + c->H * HC_N_SCORES;
     d.L = c->L;
     d.H = c->H;
     d.D = c->D;
@@ -858,15 +861,19 @@ int headcast_classify(headcast_ctx* c, const void* q, int32_t* labels_host, floa
     d.gamma = c->cfg.gamma;
     d.rule = c->cfg.rule;
     d.mass_tau = c->cfg.mass_tau;
-    HC_CUDA(c, launch_pdl(head_decide_kernel, dim3(c->H), dim3(1024), 0, st, d));
+    HC_CUDA(c, launch_pdl(head_decide_kernel, dim3(c->H), dim3(DECIDE_THREADS), 0, st, d));
     ++c->launches;
   }
-  std::vector<float> scores(static_cast<size_t>(c->H) * HC_N_SCORES);
-  HC_CUDA(c, cudaMemcpyAsync(labels_host, c->cls_labels.ptr, c->H * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  HC_CUDA(c, cudaMemcpyAsync(scores.data(), c->cls_scores.ptr, scores.size() * sizeof(float), cudaMemcpyDeviceToHost, st));
-  rc = read_status(c, st);
+  // status word, scores and labels lie together: one copy to the host instead of three that wait for one another
+  std::vector<int32_t> result(status_words(c));
+  HC_CUDA(c, cudaMemcpyAsync(result.data(), c->status_dev, result.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  HC_CUDA(c, cudaStreamSynchronize(st));
+  rc = report_status(c, result[0], st);
   if (rc != HC_OK) return rc;
-  if (scores_host) std::copy(scores.begin(), scores.end(), scores_host);
+  const int32_t* scores = result.data() + 1;
+  const int32_t* labels = scores + static_cast<size_t>(c->H) * HC_N_SCORES;
+  std::copy(labels, labels + c->H, labels_host);
+  if (scores_host) std::memcpy(scores_host, scores, static_cast<size_t>(c->H) * HC_N_SCORES * sizeof(float));
   c->labels.assign(labels_host, labels_host + c->H);
   c->have_labels = true;
   return HC_OK;

@@ -214,25 +214,44 @@ __device__ __forceinline__ float float_from_key(uint32_t k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
-// k-th smallest (0-based) of v[0..n) by a 4-pass, 8-bit-digit radix select.  Block-wide; result broadcast.
+constexpr int DECIDE_THREADS = 1024;
+constexpr int DECIDE_KEPT = 24;  // values per thread that stay in registers: heads of up to 24576 rows (68 x 120 tokens: 24480)
+
+// The order keys of v[0..n): those of the first DECIDE_KEPT * DECIDE_THREADS values from registers, the rest from memory.
+struct OrderKeys {
+  const float* v;
+  int n;
+  uint32_t kept[DECIDE_KEPT];
+  template <typename F>
+  __device__ __forceinline__ void each(F f) const {
+#pragma unroll
+    for (int k = 0; k < DECIDE_KEPT; ++k) {
+      if (k * DECIDE_THREADS >= n) return;
+      if (k * DECIDE_THREADS + static_cast<int>(threadIdx.x) < n) f(kept[k]);
+    }
+    for (int i = DECIDE_KEPT * DECIDE_THREADS + threadIdx.x; i < n; i += DECIDE_THREADS) f(float_order_key(v[i]));
+  }
+};
+
+// k-th smallest (0-based) of the keys by a 4-pass, 8-bit-digit radix select.  Block-wide; result broadcast.
 // *n_le receives how many values are <= the result (so the caller can tell whether rank k + 1 holds the same value).
-__device__ float block_select(const float* v, int n, int k, uint32_t* hist /* [256] shared */, uint32_t* bcast /* [3] */,
-                              uint32_t* n_le) {
+__device__ __forceinline__ uint32_t block_select(const OrderKeys& keys, int k, uint32_t* hist /* [256] shared */, uint32_t* bcast /* [3] */,
+                                                 uint32_t* n_le) {
   __shared__ uint32_t totals[8];
   uint32_t prefix = 0, mask = 0, below_total = 0;
   int remaining = k;
+#pragma unroll 1
   for (int shift = 24; shift >= 0; shift -= 8) {
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
+    if (threadIdx.x < 256) hist[threadIdx.x] = 0;
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const uint32_t key = float_order_key(v[i]);
+    keys.each([&](uint32_t key) {
       // cosines crowd into a few bins: the lanes of a warp that hit the same one add their number once (an atomic per
       // value queued up thousands of them on one address)
       const bool in = (key & mask) == prefix;
       const uint32_t digit = (key >> shift) & 255u;
       const uint32_t peers = __match_any_sync(__activemask(), in ? digit : 256u);
       if (in && static_cast<int>(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&hist[digit], static_cast<uint32_t>(__popc(peers)));
-    }
+    });
     __syncthreads();
     if (threadIdx.x < 256) {
       // the digit whose bin holds rank `remaining`: a scan of the 256 bins, eight warps by shuffles and their totals
@@ -264,19 +283,17 @@ __device__ float block_select(const float* v, int n, int k, uint32_t* hist /* [2
     __syncthreads();
   }
   *n_le = below_total;
-  return float_from_key(prefix);
+  return prefix;
 }
 
-// Smallest value of v[0..n) that is greater than x (+inf if none).  Block-wide; result broadcast through *slot.
-__device__ float block_min_above(const float* v, int n, float x, uint32_t* slot) {
+// Smallest value whose key is greater than x (+inf if none).  Block-wide; result broadcast through *slot.
+__device__ __forceinline__ float block_min_above(const OrderKeys& keys, uint32_t x, uint32_t* slot) {
   if (threadIdx.x == 0) *slot = 0xffffffffu;
   __syncthreads();
   uint32_t best = 0xffffffffu;
-  const uint32_t kx = float_order_key(x);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const uint32_t key = float_order_key(v[i]);
-    if (key > kx) best = min(best, key);
-  }
+  keys.each([&](uint32_t key) {
+    if (key > x) best = min(best, key);
+  });
   for (int off = 16; off > 0; off >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, off));
   if ((threadIdx.x & 31) == 0 && best != 0xffffffffu) atomicMin(slot, best);
   __syncthreads();
@@ -298,7 +315,9 @@ struct DecideParams {
 };
 
 // One block per head: fixed-order sums (deterministic), percentile by selection, Eq. 4 and Eq. 5.
-__global__ void __launch_bounds__(1024) head_decide_kernel(const DecideParams p) {
+// What it waits for is memory, one head per SM: every token quantity is read once, all eight of a token in flight together, and the
+// percentile's passes work on registers.
+__global__ void __launch_bounds__(DECIDE_THREADS) head_decide_kernel(const DecideParams p) {
   pdl_launch_dependents();
   pdl_wait();
   __shared__ double red[TOK_N][32];
@@ -307,16 +326,29 @@ __global__ void __launch_bounds__(1024) head_decide_kernel(const DecideParams p)
   __shared__ double sums[TOK_N];
   const int h = blockIdx.x;
   const size_t hl = static_cast<size_t>(p.H) * p.L;
+  OrderKeys keys;
+  keys.v = p.tok + TOK_COS_SPATIAL * hl + static_cast<size_t>(h) * p.L;
+  keys.n = p.L;
   {
     // all per-token quantities in one pass; the order of every sum is fixed by the thread layout alone
     double acc[TOK_N];
 #pragma unroll
     for (int q = 0; q < TOK_N; ++q) acc[q] = 0.0;
     const float* v = p.tok + static_cast<size_t>(h) * p.L;
-    for (int i = threadIdx.x; i < p.L; i += blockDim.x) {
+    auto add_token = [&](int i) {
+      float x[TOK_N];
 #pragma unroll
-      for (int q = 0; q < TOK_N; ++q) acc[q] += static_cast<double>(v[q * hl + i]);
+      for (int q = 0; q < TOK_N; ++q) x[q] = v[q * hl + i];
+#pragma unroll
+      for (int q = 0; q < TOK_N; ++q) acc[q] += static_cast<double>(x[q]);
+      return float_order_key(x[TOK_COS_SPATIAL]);
+    };
+#pragma unroll
+    for (int k = 0; k < DECIDE_KEPT; ++k) {
+      const int i = k * DECIDE_THREADS + threadIdx.x;
+      if (k * DECIDE_THREADS < p.L && i < p.L) keys.kept[k] = add_token(i);
     }
+    for (int i = DECIDE_KEPT * DECIDE_THREADS + threadIdx.x; i < p.L; i += DECIDE_THREADS) add_token(i);
 #pragma unroll
     for (int q = 0; q < TOK_N; ++q) {
       double x = acc[q];
@@ -331,12 +363,12 @@ __global__ void __launch_bounds__(1024) head_decide_kernel(const DecideParams p)
     }
     __syncthreads();
   }
-  const float* cos_sp = p.tok + TOK_COS_SPATIAL * hl + static_cast<size_t>(h) * p.L;
   // order statistics rank_lo and rank_lo + 1: one selection, then either the same value again (ties) or the smallest
   // value above it
   uint32_t n_le = 0;
-  const float lo = block_select(cos_sp, p.L, p.rank_lo, hist, bcast, &n_le);
-  const float above = block_min_above(cos_sp, p.L, lo, bcast);
+  const uint32_t lo_key = block_select(keys, p.rank_lo, hist, bcast, &n_le);
+  const float lo = float_from_key(lo_key);
+  const float above = block_min_above(keys, lo_key, bcast);
   const float hi = (p.rank_lo + 1 >= p.L || static_cast<int>(n_le) > p.rank_lo + 1) ? lo : above;
   if (threadIdx.x == 0) {
     const float inv_l = 1.f / static_cast<float>(p.L);

@@ -245,8 +245,9 @@ const char* headcast_last_error(const headcast_ctx* ctx);
  * other allocating routine.  q_dev and out_dev are [n_queries][n_heads][head_dim] bf16, k_dev and v_dev
  * [n_keys][n_heads][head_dim] bf16, all caller-owned, 16-byte aligned and contiguous.
  *
- * The scratch the kernel needs in global memory (work list, per-CTA ranges, status word; about 140 KB) is a fixed device array inside
- * the library: every GPU that loads the library holds it until the process exits.  Consequences:
+ * The scratch the kernels need in global memory (work list, per-CTA ranges, status word; partial results of key ranges that are cut
+ * to keep the whole GPU busy; 40 MB in all) is a fixed device array inside the library: every GPU that loads the library holds it until
+ * the process exits.  Consequences:
  *   - size limit: n_heads * ceil(n_queries / 256) <= HEADCAST_NOALLOC_MAX_ITEMS, head_dim 64 or 128,
  *     n_heads <= 64; anything larger returns HC_ERR_UNSUPPORTED and does nothing;
  *   - all calls on one GPU share that array, which keeps the previous call's contents (each call rewrites what

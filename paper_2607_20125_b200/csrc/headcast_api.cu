@@ -1204,49 +1204,159 @@ const char* headcast_last_error(const headcast_ctx* c) { return c ? c->err.c_str
 // =====================================================================================================
 // Allocation-free dense attention
 // =====================================================================================================
-// Everything the attention kernel needs in global memory besides the caller's tensors - the work list, the per-CTA
-// ranges and the status word - lives in one file-scope device array of fixed size (the two tensor maps travel as
+// Everything the kernels need in global memory besides the caller's tensors - the work list, the per-CTA ranges, the status
+// word, the partial results of key ranges that are cut and what is to be merged - lives in one file-scope device array of fixed size (the two tensor maps travel as
 // kernel parameters).  Each GPU that loads the
 // library carries these bytes until the process exits.
 namespace {
 
 constexpr int NOALLOC_MAX_ITEMS = HEADCAST_NOALLOC_MAX_ITEMS;
 constexpr int NOALLOC_MAX_CTAS = 1024;
+constexpr double NOALLOC_MERGE = 3.0, NOALLOC_MERGE_PART = 0.12;  // launch and a first batch of parts; each further part
+
+// Query-tile pairs are cut along their keys where whole ones would leave much of the GPU idle, over at most this many CTAs, each
+// of which leaves at most two partial results (its first and its last piece).
+constexpr int NOALLOC_CUT_CTAS = 148, NOALLOC_SLOTS = 2 * NOALLOC_CUT_CTAS, NOALLOC_MERGES = 2 * NOALLOC_CUT_CTAS;
 
 struct NoAllocScratch {
-  WorkItem items[NOALLOC_MAX_ITEMS];
+  float part_o[NOALLOC_SLOTS][256 * 128];  // (head_dim 64 uses half of it)
+  float2 part_ml[NOALLOC_SLOTS][256];
+  WorkItem items[NOALLOC_MAX_ITEMS + NOALLOC_CUT_CTAS];
+  CombineEntry merge[NOALLOC_MERGES];  // two per pair that is cut
   int32_t cta_first[NOALLOC_MAX_CTAS + 1];
   int32_t status;
 };
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocScratch)];
 
-// Writes the work list of one call: whole query-tile pairs, dealt round-robin to one CTA per SM (every item has the same key
-// range).  Built here and not copied from the host: three copies from pageable memory made a call take 21 us of host time
-// whatever its size.
-__global__ void __launch_bounds__(256) noalloc_list_kernel(NoAllocScratch* s, int n_items, int n_cta, int n_heads, int head_dim,
-                                                           int n_queries, int n_keys) {
+// How the query-tile pairs of one call (all of the same key range) are spread.
+struct NoAllocPlan {
+  int n_items, n_tiles;  // pairs, key tiles of each
+  int n_cta;             // CTAs that get work (cut), or that whole pairs are dealt to
+  int cuts;              // 0: whole pairs; > 0: every pair in so many equal pieces, a CTA each; < 0: pairs laid end to end, an equal share of the line to each CTA
+  // first key tile of CTA b's share, on the line of all pairs
+  __host__ __device__ long long share_begin(int b) const {
+    if (cuts > 0) return static_cast<long long>(b / cuts) * n_tiles + static_cast<long long>(b % cuts) * n_tiles / cuts;
+    const long long x = static_cast<long long>(n_items) * n_tiles * b / n_cta, in = x % n_tiles;
+    return in < MIN_PART_TILES ? x - in : n_tiles - in < MIN_PART_TILES ? x + n_tiles - in : x;  // no piece shorter than that
+  }
+};
+
+// Whole pairs, equal pieces of each, or equal shares of the line of all of them, whichever the scheduler's cost model expects to
+// end first; cutting has to promise 5 %, and merging costs one more launch.  The line is for numbers of pairs that fill the last wave
+// badly: its shares are at least two proper pieces long, and beyond eight waves there is too little to gain.  1373 queries, 5492 keys,
+// sixteen heads of 64 (a line): 77 -> 61 us; 687 queries, 2748 keys, eight heads of 128 (equal pieces): 46.5 -> 24.8;
+// 1785 queries, 12495 keys, four heads of 128: 166 -> 53.
+NoAllocPlan noalloc_plan(int n_items, int n_keys, int n_sm) {
+  NoAllocPlan p = {n_items, (n_keys + 127) / 128, n_sm, 0};
+  if (p.n_tiles < 8) return p;  // half of that does not pay for a merge
+  const double item = COST_MEASURED.item, piece = COST_MEASURED.item + COST_MEASURED.partial;
+  double best = 0.95 * ((n_items + n_sm - 1) / n_sm) * (p.n_tiles + item);
+  const int n_cta = std::min(n_sm, NOALLOC_CUT_CTAS);
+  for (int k = 2; k <= std::min(n_cta / n_items, p.n_tiles); ++k) {
+    const double end = (p.n_tiles + k - 1) / k + piece + NOALLOC_MERGE + NOALLOC_MERGE_PART * k;
+    if (end < best) {
+      best = end;
+      p.cuts = k;
+      p.n_cta = n_items * k;
+    }
+  }
+  const double share = static_cast<double>(n_items) * p.n_tiles / n_cta;
+  if (n_items > n_cta / 4 && n_items < 8 * n_cta && p.n_tiles >= 4 * MIN_PART_TILES && share >= 2 * MIN_PART_TILES) {
+    const double end = share + item * n_items / n_cta + 2 * piece - item + NOALLOC_MERGE;
+    if (end < best) {
+      p.cuts = -1;
+      p.n_cta = n_cta;
+    }
+  }
+  return p;
+}
+
+// Writes the work list of one call, and what is to be merged: whole pairs over as many blocks as it takes, shares of a line in one
+// block with a thread per CTA of the attention kernel (which it scans over).  Built here and not copied from the host: three copies from
+// pageable memory made a call take 21 us of host time whatever its size.
+template <bool CUT>
+__global__ void __launch_bounds__(CUT ? NOALLOC_MAX_CTAS : 256) noalloc_list_kernel(NoAllocScratch* s, NoAllocPlan plan, int grid, int n_heads, int head_dim,
+                                                                        int n_queries, int n_keys) {
   pdl_launch_dependents();
+  const int b = blockIdx.x * blockDim.x + threadIdx.x, nt = plan.n_tiles;
+  auto item = [&](int pair, int begin, int end) {
+    const int h = pair % n_heads, q0 = pair / n_heads * 256;
+    WorkItem w = {};
+    w.head = h;
+    w.cell = -1;
+    w.q_start[0] = q0;
+    w.q_start[1] = q0 + 128;
+    w.q_count[0] = min(128, n_queries - q0);
+    w.q_count[1] = max(0, min(128, n_queries - q0 - 128));
+    w.kv_x0 = h * head_dim;
+    w.seg_len = n_keys;
+    w.tiles_per_seg = nt;
+    w.tile_begin = begin;
+    w.tile_end = end;
+    w.out_mode = OUT_BF16;
+    return w;
+  };
+  if (!CUT) {
+    const int each = plan.n_items / grid, more = plan.n_items % grid;  // CTA b owns items b, b + grid, ...: `each`, plus one for the first `more`
+    const int at = (b % grid) * each + min(b % grid, more) + b / grid;
+    const WorkItem w = item(b, 0, nt);
+    pdl_wait();  // the kernel before may still read the list of its own call
+    if (b <= grid) s->cta_first[b] = b * each + min(b, more);
+    if (b == 0) s->status = 0;  // the array keeps the previous call's contents
+    if (b < plan.n_items) s->items[at] = w;
+    return;
+  }
+  __shared__ int32_t warp_sum[3][NOALLOC_MAX_CTAS / 32];
+  // CTA b's share [x0, x1) of the line: its pieces, how many of them are partial results, and whether it begins a pair that is cut
+  const long long x0 = b < plan.n_cta ? plan.share_begin(b) : 0, x1 = b < plan.n_cta ? plan.share_begin(b + 1) : 0;
+  const int p0 = static_cast<int>(x0 / nt), p1 = x1 > x0 ? static_cast<int>((x1 - 1) / nt) : p0 - 1;  // first and last pair
+  auto begin_of = [&](int pair) { return pair == p0 ? static_cast<int>(x0 - static_cast<long long>(p0) * nt) : 0; };
+  auto end_of = [&](int pair) { return pair == p1 ? static_cast<int>(x1 - static_cast<long long>(p1) * nt) : nt; };
+  int n[3] = {p1 - p0 + 1, 0, 0};
+  if (n[0] > 0) {
+    const bool first_cut = begin_of(p0) > 0 || end_of(p0) < nt;
+    n[1] = (first_cut ? 1 : 0) + (p1 > p0 && end_of(p1) < nt ? 1 : 0);
+    n[2] = begin_of(p1) == 0 && end_of(p1) < nt ? 1 : 0;
+  }
+  int before[3];  // the same of all CTAs before this one
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    int upto = n[q];
+#pragma unroll
+    for (int off = 1; off < 32; off *= 2) {
+      const int y = __shfl_up_sync(0xffffffffu, upto, off);
+      if ((b & 31) >= off) upto += y;
+    }
+    if ((b & 31) == 31) warp_sum[q][b >> 5] = upto;
+    before[q] = upto - n[q];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 3; ++q)
+    for (int w = 0; w < (b >> 5); ++w) before[q] += warp_sum[q][w];
   pdl_wait();  // the kernel before may still read the list of its own call
-  const int i = blockIdx.x * 256 + threadIdx.x;
-  const int each = n_items / n_cta, more = n_items % n_cta;  // CTA b owns items b, b + n_cta, ...: `each`, plus one for the first `more`
-  if (i <= n_cta) s->cta_first[i] = i * each + min(i, more);
-  if (i == 0) s->status = 0;  // the array keeps the previous call's contents
-  if (i >= n_items) return;
-  const int b = i % n_cta, h = i % n_heads, q0 = i / n_heads * 256;
-  WorkItem w = {};
-  w.head = h;
-  w.cell = -1;
-  w.q_start[0] = q0;
-  w.q_start[1] = q0 + 128;
-  w.q_count[0] = min(128, n_queries - q0);
-  w.q_count[1] = max(0, min(128, n_queries - q0 - 128));
-  w.kv_x0 = h * head_dim;
-  w.seg_len = n_keys;
-  w.tiles_per_seg = (n_keys + 127) / 128;
-  w.tile_end = w.tiles_per_seg;
-  w.out_mode = OUT_BF16;
-  s->items[b * each + min(b, more) + i / n_cta] = w;
+  if (b < grid) s->cta_first[b] = before[0];
+  if (b == grid - 1) s->cta_first[grid] = before[0] + n[0];
+  if (b == 0) s->status = 0;
+  int slot = before[1];
+  for (int pair = p0; pair <= p1; ++pair) {
+    WorkItem w = item(pair, begin_of(pair), end_of(pair));
+    if (w.tile_end - w.tile_begin < nt) {
+      w.out_mode = OUT_PARTIAL;
+      w.out_slot = slot++;
+      if (w.tile_begin == 0) {  // this pair's pieces: here and in the CTAs that follow
+        int more = 1;
+        while (plan.share_begin(b + more + 1) < static_cast<long long>(pair + 1) * nt) ++more;
+        for (int t = 0; t < 2; ++t) s->merge[2 * before[2] + t] = {w.head, -1, w.q_start[t], w.q_count[t], w.out_slot, more + 1, t, 0};
+      }
+    }
+    s->items[before[0] + pair - p0] = w;
+  }
+  // entries that the launch of the merge has blocks for but no pair was cut for
+  int n_entries = 0;
+  for (int w = 0; w < static_cast<int>(blockDim.x) / 32; ++w) n_entries += 2 * warp_sum[2][w];
+  for (int i = n_entries + b; i < NOALLOC_MERGES; i += blockDim.x) s->merge[i].q_count = 0;
 }
 
 constexpr int NOALLOC_MAX_DEVICES = 64;
@@ -1335,9 +1445,10 @@ int headcast_dense_attend_noalloc(const void* q, const void* k, const void* v, v
       !make_tmap_bf16_2d(&p.maps[1], v, row_elems, n_keys, row_elems, 128))
     return noalloc_fail(HC_ERR_CUDA, "cuTensorMapEncodeTiled failed or is unavailable");
   const int n_cta = d.n_sm;
-  const int list_threads = std::max(static_cast<int>(n_items), n_cta + 1);
-  e = launch_pdl(noalloc_list_kernel, dim3((list_threads + 255) / 256), dim3(256), 0, st, d.scratch, static_cast<int>(n_items), n_cta,
-                 n_heads, head_dim, n_queries, n_keys);
+  const NoAllocPlan plan = noalloc_plan(static_cast<int>(n_items), n_keys, n_cta);
+  const int list_threads = std::max(plan.cuts ? 0 : static_cast<int>(n_items), n_cta + 1);
+  e = launch_pdl(plan.cuts ? noalloc_list_kernel<true> : noalloc_list_kernel<false>, plan.cuts ? dim3(1) : dim3((list_threads + 255) / 256), dim3(plan.cuts ? (n_cta + 31) / 32 * 32 : 256), 0, st,
+                 d.scratch, plan, n_cta, n_heads, head_dim, n_queries, n_keys);
   if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "launching the list kernel", e);
 
   p.items = d.scratch->items;
@@ -1351,9 +1462,20 @@ int headcast_dense_attend_noalloc(const void* q, const void* k, const void* v, v
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / std::sqrt(static_cast<float>(head_dim));
   p.scale_log2e = scale * 1.4426950408889634f;
   p.status = &d.scratch->status;
+  p.part_o = &d.scratch->part_o[0][0];
+  p.part_ml = &d.scratch->part_ml[0][0];
   e = launch_pdl(head_dim == 128 ? attn_kernel<128, false> : attn_kernel<64, false>, dim3(n_cta), dim3(ATTN_THREADS),
                  head_dim == 128 ? AttnSmem<128>::DYN_BYTES : AttnSmem<64>::DYN_BYTES, st, p);
   if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "launching the attention kernel", e);
+  if (plan.cuts != 0) {
+    // pairs that are cut: with equal pieces all of them, else at most one at every boundary between two shares
+    const int entries = 2 * (plan.cuts > 0 ? plan.n_items : std::min(plan.n_items, plan.n_cta - 1));
+    const int n_long = plan.cuts > COMBINE_LONG_PARTS ? entries : 0;
+    e = launch_pdl(head_dim == 128 ? combine_kernel<128> : combine_kernel<64>, dim3(n_long * 128 + (entries - n_long) * (128 / COMBINE_ROWS)),
+                   dim3(COMBINE_ROWS * (head_dim / 8)), 0, st, d.scratch->merge, n_long, nullptr, p.part_o, p.part_ml, p.out, n_heads, n_queries, 1,
+                   false);
+    if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "launching the merge kernel", e);
+  }
   return HC_OK;
 }
 

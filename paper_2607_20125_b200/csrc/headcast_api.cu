@@ -953,6 +953,12 @@ int init_host_path(headcast_ctx* c) {
 
 }  // namespace
 
+// Blocks whose queries are no larger than this are copied, attended and copied back as one, in the order of the caller's stream:
+// stages hide copies, but every one brings launches, copies and events of its own.  Append + four attends, one stage against four:
+// 0.5 MB 253 us against 323, 2.5 MB 677 against 875, 3.8 MB 974 against 1081; 4.4 MB 1120 against 1214 but 4.6 MB 1557 against 1538
+// and 8.7 MB 2262 against 2067.
+constexpr size_t HOST_ONE_STAGE_BYTES = 4 << 20;
+
 int headcast_append_host(headcast_ctx* c, const void* k_host, const void* v_host, void* stream) {
   if (!c || !k_host || !v_host) return HC_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -968,11 +974,18 @@ int headcast_attend_host(headcast_ctx* c, const void* q_host, void* out_host, vo
   if (!c || !q_host || !out_host) return HC_ERR_INVALID_ARG;
   if (c->state != STATE_SPLIT) return fail(c, HC_ERR_STATE, "head-specific attention needs the split cache");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int rc = init_host_path(c);
-  if (rc != HC_OK) return rc;
-  const size_t elems = static_cast<size_t>(c->L) * c->H * c->D;
+  const size_t elems = static_cast<size_t>(c->L) * c->H * c->D, bytes = elems * sizeof(__nv_bfloat16);
   HC_CUDA(c, c->stage_q.reserve(c->memory, elems, st));
   HC_CUDA(c, c->stage_out.reserve(c->memory, elems, st));
+  if (bytes <= HOST_ONE_STAGE_BYTES) {
+    HC_CUDA(c, cudaMemcpyAsync(c->stage_q.ptr, q_host, bytes, cudaMemcpyHostToDevice, st));
+    const int rc = headcast_attend(c, c->stage_q.ptr, c->stage_out.ptr, stream);
+    if (rc != HC_OK) return rc;
+    HC_CUDA(c, cudaMemcpyAsync(out_host, c->stage_out.ptr, bytes, cudaMemcpyDeviceToHost, st));
+    return HC_OK;
+  }
+  int rc = init_host_path(c);
+  if (rc != HC_OK) return rc;
   const int key = n_filled(c) * 4 + c->sd_valid;
   // Stages: a stage's queries are copied in (strided: the rows of [L][H][d] hold all heads), attended and copied out
   // as a unit, so that the next stage's queries arrive and the previous stage's outputs leave while this stage

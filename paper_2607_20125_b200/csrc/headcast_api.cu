@@ -6,8 +6,8 @@
 
 namespace {
 
-// Launches a kernel of this library (every one of them calls pdl_wait before it touches global memory) so that it may
-// become resident while its predecessor on the stream drains.  Since the predecessor may still write while such a kernel
+// Launches a kernel of this library (every one of them calls pdl_wait before it touches global memory, but for lists whose
+// upload was waited for) so that it may become resident while its predecessor on the stream drains.  Since the predecessor may still write while such a kernel
 // runs, nothing is read through the non-coherent path (__ldg, ld.global.nc): that path wants data which no one writes for
 // as long as the reading kernel lives, and pdl_wait orders ordinary loads only.  Together with the one merge launch instead of two it takes
 // the block of 192 tokens and four heads from 86 to 76 us and leaves the large ones where they are (45 x 80: -1 %).
@@ -1218,9 +1218,9 @@ const char* headcast_last_error(const headcast_ctx* c) { return c ? c->err.c_str
 // Allocation-free dense attention
 // =====================================================================================================
 // Everything the kernels need in global memory besides the caller's tensors - the work list, the per-CTA ranges, the status
-// word, the partial results of key ranges that are cut and what is to be merged - lives in one file-scope device array of fixed size (the two tensor maps travel as
-// kernel parameters).  Each GPU that loads the
-// library carries these bytes until the process exits.
+// word, the partial results of key ranges that are cut and what is to be merged - lives in one file-scope device array of
+// fixed size (the two tensor maps travel as kernel parameters).  Each GPU that loads the library carries these bytes until the
+// process exits.
 namespace {
 
 constexpr int NOALLOC_MAX_ITEMS = HEADCAST_NOALLOC_MAX_ITEMS;

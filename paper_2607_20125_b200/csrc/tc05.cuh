@@ -101,7 +101,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
 
 // Programmatic dependent launch.  launch_dependents lets the next kernel of the stream become resident (and set itself up)
 // while this one drains; wait returns once the kernel before has completed and its writes are visible.  Every thread that
-// touches global memory calls wait first.
+// touches global memory calls wait first, but for work and merge lists that were complete before the launch was made.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

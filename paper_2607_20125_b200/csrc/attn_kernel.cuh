@@ -641,9 +641,10 @@ struct RowMerge {
 #pragma unroll
     for (int i = 0; i < 8; ++i) acc[i] *= old;
   }
-  __device__ __forceinline__ float add(float2 ml, const float4& a, const float4& b) {  // returns the part's weight
-    if (ml.x == -INFINITY) return 0.f;
-    const float w = ex2_approx(ml.x - m);
+  // Returns the part's weight.  A row that met nothing but NaN logits has the maximum -inf too: its values count, times zero,
+  // so that they come out as NaN.
+  __device__ __forceinline__ float add(float2 ml, const float4& a, const float4& b) {
+    const float w = ml.x == -INFINITY ? 0.f : ex2_approx(ml.x - m);
     l += w * ml.y;
     acc[0] += w * a.x; acc[1] += w * a.y; acc[2] += w * a.z; acc[3] += w * a.w;
     acc[4] += w * b.x; acc[5] += w * b.y; acc[6] += w * b.z; acc[7] += w * b.w;
@@ -682,7 +683,8 @@ __device__ __forceinline__ void combine_rows(const CombineEntry& e, int block, c
     }
     row.raise_reference(fmaxf(fmaxf(ml[0].x, ml[1].x), fmaxf(ml[2].x, ml[3].x)));
 #pragma unroll
-    for (int k = 0; k < MERGE_BATCH; ++k) row.add(ml[k], a[k], b[k]);
+    for (int k = 0; k < MERGE_BATCH; ++k)
+      if (i0 + k < n) row.add(ml[k], a[k], b[k]);
   }
   const float inv = row.l > 0.f ? 1.f / row.l : 0.f;
   int token = e.q_start + r;

@@ -82,7 +82,7 @@ cls_combine_kernel(const ClsGroup* groups, const ClsPart* parts, const float* pa
       set[s].raise_reference(to);
 #pragma unroll
       for (int k = 0; k < CLS_MERGE_BATCH; ++k)
-        if (s == 0 || part[k].tag == 2 * (s - 1)) set[s].add(ml[k], a[k], b[k]);
+        if (ml[k].x != -INFINITY && (s == 0 || part[k].tag == 2 * (s - 1))) set[s].add(ml[k], a[k], b[k]);
     }
   }
   float dot[2] = {0.f, 0.f}, nrm[3] = {0.f, 0.f, 0.f};
@@ -174,10 +174,8 @@ proxy_combine_kernel(const ClsGroup* groups, const ClsPart* parts, const float* 
     row.raise_reference(to);
     if (before != -INFINITY) l_mid *= ex2_approx(before - row.m);
 #pragma unroll
-    for (int k = 0; k < CLS_MERGE_BATCH; ++k) {
-      const float w = row.add(ml[k], a[k], b[k]);
-      if (w != 0.f) l_mid += w * mid[k];
-    }
+    for (int k = 0; k < CLS_MERGE_BATCH; ++k)
+      if (ml[k].x != -INFINITY) l_mid += row.add(ml[k], a[k], b[k]) * mid[k];
   }
   const float inv = row.l > 0.f ? 1.f / row.l : 0.f;
   float dot = 0.f, n_sp = 0.f, n_ref = 0.f, sq = 0.f;

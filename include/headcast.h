@@ -20,6 +20,7 @@
  *     Attention calls of one context share scratch memory.  When a context changes streams the call takes a new
  *     scratch, the first three times, and from then on waits on the device for the call before it.  Launches
  *     captured into a graph use the same scratch at every replay; the caller orders replays and other calls.
+ *     Calls that change the cache are ordered by the caller against all others where they are on different streams.
  *   - the context owns every cache, table and scratch buffer: device memory that it takes at headcast_create or
  *     on first use and gives up at headcast_destroy (the monolithic cache at the split).  Of what contexts give up
  *     the library keeps at most 640 MB per GPU for contexts to come (384 MB of blocks, 256 MB of monolithic
@@ -186,7 +187,8 @@ int64_t headcast_launch_count(const headcast_ctx* ctx);
  * (Sec. 4.4, as headcast_attend) and its part of the output copied out, on two copy streams of the context, so that
  * transfers in both directions overlap the attention of the other stages.  Both
  * return once everything is enqueued; out_host is complete when work enqueued on `stream` after the call runs (e.g.
- * after synchronising `stream`).  q_host must stay unchanged and out_host untouched until then.  Staging buffers,
+ * after synchronising `stream`).  q_host must stay unchanged and out_host untouched until then.  All attends of a context
+ * share one pair of staging buffers: one on another stream than the last waits for that one on the device.  Staging buffers,
  * streams and events are created on the first call.  Errors as headcast_attend / headcast_append. */
 int headcast_append_host(headcast_ctx* ctx, const void* k_host, const void* v_host, void* stream);
 int headcast_attend_host(headcast_ctx* ctx, const void* q_host, void* out_host, void* stream);

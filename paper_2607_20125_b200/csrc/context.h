@@ -339,6 +339,10 @@ struct headcast_ctx {
   static constexpr int N_HOST_STAGES = 4;
   Schedule sched_stage[N_HOST_STAGES];
   DevBuf<__nv_bfloat16> stage_q, stage_out, stage_k, stage_v;  // device copies of host tensors
+  // the last call that used stage_q and stage_out: its stream's number, and what is recorded behind its last copy
+  bool stage_used = false;
+  unsigned long long stage_stream = 0;
+  cudaEvent_t stage_done = nullptr;
   cudaStream_t copy_in = nullptr, copy_out = nullptr;
   cudaEvent_t ev_host[2 + 2 * N_HOST_STAGES] = {};
   DevBuf<float> part_o;

@@ -598,6 +598,7 @@ int headcast_destroy(headcast_ctx* c) {
   if (c->ev_a) cudaEventDestroy(c->ev_a);
   if (c->ev_b) cudaEventDestroy(c->ev_b);
   if (c->scratch_done) cudaEventDestroy(c->scratch_done);
+  if (c->stage_done) cudaEventDestroy(c->stage_done);
   c->sched_dense.release(cache, idle);
   c->sched_hc.release(cache, idle);
   c->sched_cls.release(cache, idle);
@@ -970,18 +971,17 @@ int headcast_append_host(headcast_ctx* c, const void* k_host, const void* v_host
   return headcast_append(c, c->stage_k.ptr, c->stage_v.ptr, stream);
 }
 
-int headcast_attend_host(headcast_ctx* c, const void* q_host, void* out_host, void* stream) {
-  if (!c || !q_host || !out_host) return HC_ERR_INVALID_ARG;
-  if (c->state != STATE_SPLIT) return fail(c, HC_ERR_STATE, "head-specific attention needs the split cache");
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
+// `done`: recorded once the call's last copy has left the staging buffers (nullptr: not).
+static int attend_host(headcast_ctx* c, const void* q_host, void* out_host, cudaStream_t st, cudaEvent_t done) {
   const size_t elems = static_cast<size_t>(c->L) * c->H * c->D, bytes = elems * sizeof(__nv_bfloat16);
   HC_CUDA(c, c->stage_q.reserve(c->memory, elems, st));
   HC_CUDA(c, c->stage_out.reserve(c->memory, elems, st));
   if (bytes <= HOST_ONE_STAGE_BYTES) {
     HC_CUDA(c, cudaMemcpyAsync(c->stage_q.ptr, q_host, bytes, cudaMemcpyHostToDevice, st));
-    const int rc = headcast_attend(c, c->stage_q.ptr, c->stage_out.ptr, stream);
+    const int rc = headcast_attend(c, c->stage_q.ptr, c->stage_out.ptr, st);
     if (rc != HC_OK) return rc;
     HC_CUDA(c, cudaMemcpyAsync(out_host, c->stage_out.ptr, bytes, cudaMemcpyDeviceToHost, st));
+    if (done) HC_CUDA(c, cudaEventRecord(done, st));
     return HC_OK;
   }
   int rc = init_host_path(c);
@@ -1036,10 +1036,38 @@ int headcast_attend_host(headcast_ctx* c, const void* q_host, void* out_host, vo
     HC_CUDA(c, cudaStreamWaitEvent(c->copy_out, c->ev_host[3 + 2 * i], 0));
     if ((rc = copy_stage(stages[i], false)) != HC_OK) return rc;
   }
-  HC_CUDA(c, cudaEventRecord(c->ev_host[1], c->copy_out));
-  HC_CUDA(c, cudaStreamWaitEvent(st, c->ev_host[1], 0));
+  if (!done) done = c->ev_host[1];
+  HC_CUDA(c, cudaEventRecord(done, c->copy_out));
+  HC_CUDA(c, cudaStreamWaitEvent(st, done, 0));
   return HC_OK;
 }
+
+// All calls go through one pair of staging buffers, so every call leaves an event behind its last copy and a call on another stream
+// than the last one waits for it.  (The launches and copies of a graph are the caller's to order; events of a capture mean
+// nothing outside it.)
+int headcast_attend_host(headcast_ctx* c, const void* q_host, void* out_host, void* stream) {
+  if (!c || !q_host || !out_host) return HC_ERR_INVALID_ARG;
+  if (c->state != STATE_SPLIT) return fail(c, HC_ERR_STATE, "head-specific attention needs the split cache");
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  HC_CUDA(c, cudaStreamIsCapturing(st, &status));
+  if (status != cudaStreamCaptureStatusNone) return attend_host(c, q_host, out_host, st, nullptr);
+  unsigned long long id = 0;
+  HC_CUDA(c, cudaStreamGetId(st, &id));
+  if (!c->stage_done) HC_CUDA(c, cudaEventCreateWithFlags(&c->stage_done, cudaEventDisableTiming));
+  if (c->stage_used && c->stage_stream != id) HC_CUDA(c, cudaStreamWaitEvent(st, c->stage_done, 0));
+  c->stage_used = true;
+  c->stage_stream = id;
+  const int rc = attend_host(c, q_host, out_host, st, c->stage_done);
+  if (rc != HC_OK) {  // what was enqueued before it failed comes first all the same
+    for (cudaStream_t copies : {c->copy_in, c->copy_out})
+      if (copies && cudaEventRecord(c->stage_done, copies) == cudaSuccess) cudaStreamWaitEvent(st, c->stage_done, 0);
+    cudaEventRecord(c->stage_done, st);
+    cudaGetLastError();
+  }
+  return rc;
+}
+
 
 int headcast_export_cache(headcast_ctx* c, int32_t head, void* k_out, void* v_out, int32_t* n_tokens_host, void* stream) {
   if (!c || head < 0 || head >= c->H) return HC_ERR_INVALID_ARG;

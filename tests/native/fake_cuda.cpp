@@ -31,8 +31,8 @@ struct Fake {
   cudaError_t last_error = cudaSuccess;        // what the next cudaGetLastError reports
   std::map<const void*, std::string> kernels;
   std::map<const void*, int> smem;             // dynamic shared memory that a kernel may be launched with
-  // launches, events, waits and the host's waits for a stream or the device, in order:
-  // "L<stream>:<kernel>@<scratch> E<stream>:<event> W<stream>:<event> Y<stream>: S"
+  // launches, copies to and from the device (with their address there), events, waits and the host's waits for a stream or the
+  // device, in order: "L<stream>:<kernel>@<scratch> H<stream>:<to> D<stream>:<from> E<stream>:<event> W<stream>:<event> Y<stream>: S"
   std::string log;
 };
 
@@ -192,8 +192,16 @@ cudaError_t cudaMemcpy(void* dst, const void* src, size_t n, cudaMemcpyKind kind
   if (kind == cudaMemcpyDeviceToHost || write_to(dst)) std::memcpy(dst, src, n);
   return cudaSuccess;
 }
-cudaError_t cudaMemcpyAsync(void* dst, const void* src, size_t n, cudaMemcpyKind k, cudaStream_t) { return cudaMemcpy(dst, src, n, k); }
-cudaError_t cudaMemcpy2DAsync(void* dst, size_t, const void*, size_t, size_t, size_t, cudaMemcpyKind kind, cudaStream_t) {
+static void copied(void* dst, const void* src, cudaMemcpyKind kind, cudaStream_t s) {
+  if (kind == cudaMemcpyHostToDevice) fake().log += "H" + handle(s) + ":" + handle(dst) + " ";
+  if (kind == cudaMemcpyDeviceToHost) fake().log += "D" + handle(s) + ":" + handle(src) + " ";
+}
+cudaError_t cudaMemcpyAsync(void* dst, const void* src, size_t n, cudaMemcpyKind kind, cudaStream_t s) {
+  copied(dst, src, kind, s);
+  return cudaMemcpy(dst, src, n, kind);
+}
+cudaError_t cudaMemcpy2DAsync(void* dst, size_t, const void* src, size_t, size_t, size_t, cudaMemcpyKind kind, cudaStream_t s) {
+  copied(dst, src, kind, s);
   if (kind == cudaMemcpyHostToDevice) write_to(dst);
   return cudaSuccess;
 }

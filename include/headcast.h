@@ -256,8 +256,9 @@ const char* headcast_last_error(const headcast_ctx* ctx);
  *   - all calls on one GPU share that array, which keeps the previous call's contents (each call rewrites what
  *     it uses and clears the status word): two calls whose GPU work overlaps - different streams, or different
  *     host threads - race on it.  Keep calls on one GPU in one stream, or order them with events;
- *   - the first call on each device looks up the array's device address and sets the kernel's shared-memory
- *     attribute (with that device current).  Make that first call before starting any stream capture;
+ *   - the first call on each device looks up the array's device address, loads every kernel that a call of any size
+ *     needs and sets their shared-memory attributes (with that device current).  Make that first call before the
+ *     memory is handed out and before starting any stream capture;
  *   - a call on a stream that is being captured returns HC_ERR_UNSUPPORTED (a graph replayed beside other calls
  *     would overwrite the work list they share).
  * softmax_scale = 0 selects 1/sqrt(head_dim).  Asynchronous on `stream`.  headcast_noalloc_status synchronises

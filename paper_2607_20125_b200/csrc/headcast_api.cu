@@ -1437,6 +1437,19 @@ int noalloc_setup(int dev) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(attn_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<64>::DYN_BYTES);
   if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "cudaFuncSetAttribute", e);
+  // The driver loads a kernel's code when the kernel is first asked for, and may take device memory or wait for the device then:
+  // all that any size can need is asked for here, in the first call, whatever its size.
+  auto load = [&](auto* kernel) {
+    cudaFuncAttributes attributes;
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&attributes, kernel);
+  };
+  load(noalloc_list_kernel<false>);
+  load(noalloc_list_kernel<true>);
+  load(attn_kernel<64, false>);
+  load(attn_kernel<128, false>);
+  load(combine_kernel<64>);
+  load(combine_kernel<128>);
+  if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "cudaFuncGetAttributes", e);
   if (!current_context_id(&d.context)) return noalloc_fail(HC_ERR_CUDA, "cuCtxGetId");
   d.n_sm = std::min(prop.multiProcessorCount, NOALLOC_MAX_CTAS);
   d.scratch = static_cast<NoAllocScratch*>(ptr);

@@ -31,6 +31,7 @@ struct Fake {
   cudaError_t last_error = cudaSuccess;        // what the next cudaGetLastError reports
   std::map<const void*, std::string> kernels;
   std::map<const void*, int> smem;             // dynamic shared memory that a kernel may be launched with
+  std::set<const void*> loaded;                // kernels whose code the driver has been asked for
   // launches, copies to and from the device (with their address there), events, waits and the host's waits for a stream or the
   // device, in order: "L<stream>:<kernel>@<scratch> H<stream>:<to> D<stream>:<from> E<stream>:<event> W<stream>:<event> Y<stream>: S"
   std::string log;
@@ -121,6 +122,7 @@ void fake_capture(int mode, void* stream) {
 }
 int fake_capture_invalidated() { return fake().invalidated; }
 int fake_is_live(void* p) { return fake().live.count(static_cast<char*>(p)) != 0; }
+int fake_kernels_loaded() { return static_cast<int>(fake().loaded.size()); }
 const char* fake_log() { return fake().log.c_str(); }
 void fake_clear_log() { fake().log.clear(); }
 void fake_device_reset() {  // every allocation is gone, a new context takes the old one's place
@@ -129,6 +131,7 @@ void fake_device_reset() {  // every allocation is gone, a new context takes the
   fake().pool.clear();
   fake().busy.clear();
   fake().smem.clear();
+  fake().loaded.clear();
   fake().used = fake().pool_unused = 0;
   ++fake().context_id;
 }
@@ -278,7 +281,13 @@ cudaError_t cudaGetDriverEntryPoint(const char* name, void** fn, unsigned long l
 }
 
 // ------------------------------------------------------------------------------------------ kernels
+cudaError_t cudaFuncGetAttributes(cudaFuncAttributes* a, const void* fn) {
+  std::memset(a, 0, sizeof(*a));
+  fake().loaded.insert(fn);
+  return cudaSuccess;
+}
 cudaError_t cudaFuncSetAttribute(const void* fn, cudaFuncAttribute a, int v) {
+  fake().loaded.insert(fn);
   if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) fake().smem[fn] = v;
   return cudaSuccess;
 }
@@ -289,6 +298,7 @@ cudaError_t cudaGetSymbolAddress(void** p, const void*) {
 }
 static cudaError_t launched(const void* fn, void** args, size_t smem, cudaStream_t s) {
   if (smem > 48 << 10 && static_cast<int>(smem) > fake().smem[fn]) return failed(cudaErrorInvalidValue);
+  fake().loaded.insert(fn);
   const std::string& name = fake().kernels[fn];
   const void* scratch = fake_saw_launch(name.c_str(), args);
   fake().log += "L" + handle(s) + ":" + name + "@" + handle(scratch) + " ";

@@ -249,14 +249,14 @@ const char* headcast_last_error(const headcast_ctx* ctx);
  * [n_keys][n_heads][head_dim] bf16, all caller-owned, 16-byte aligned and contiguous.
  *
  * The scratch the kernels need in global memory (work list, per-CTA ranges, status word; partial results of key ranges that are cut
- * to keep the whole GPU busy; 40 MB in all) is a fixed device array inside the library: every GPU that loads the library holds it until
- * the process exits.  Consequences:
+ * to keep the whole GPU busy; 40 MB in all) is a fixed device array inside the library: a GPU holds it from its first such call until
+ * the process exits (programs that make none do not).  Consequences:
  *   - size limit: n_heads * ceil(n_queries / 256) <= HEADCAST_NOALLOC_MAX_ITEMS, head_dim 64 or 128,
  *     n_heads <= 64; anything larger returns HC_ERR_UNSUPPORTED and does nothing;
  *   - all calls on one GPU share that array, which keeps the previous call's contents (each call rewrites what
  *     it uses and clears the status word): two calls whose GPU work overlaps - different streams, or different
  *     host threads - race on it.  Keep calls on one GPU in one stream, or order them with events;
- *   - the first call on each device looks up the array's device address, loads every kernel that a call of any size
+ *   - the first call on each device makes the driver place the array, loads every kernel that a call of any size
  *     needs and sets their shared-memory attributes (with that device current).  Make that first call before the
  *     memory is handed out and before starting any stream capture;
  *   - a call on a stream that is being captured returns HC_ERR_UNSUPPORTED (a graph replayed beside other calls

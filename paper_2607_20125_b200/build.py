@@ -6,6 +6,7 @@ import subprocess
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
+UNITS = ("headcast_api.cu", "noalloc_scratch.cu")
 LIB = os.path.join(HERE, "libheadcast.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
@@ -27,11 +28,11 @@ def is_stale() -> bool:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compiles csrc/headcast_api.cu (which includes every kernel header) into libheadcast.so."""
+    """Compiles csrc/headcast_api.cu (which includes every kernel header) and csrc/noalloc_scratch.cu into libheadcast.so."""
     if not force and not is_stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    cmd = [nvcc, *NVCC_FLAGS, "-o", LIB, os.path.join(CSRC, "headcast_api.cu")]
+    cmd = [nvcc, *NVCC_FLAGS, "-o", LIB, *(os.path.join(CSRC, f) for f in UNITS)]
     if verbose:
         cmd.insert(1, "-Xptxas=-v")
     res = subprocess.run(cmd, capture_output=True, text=True)

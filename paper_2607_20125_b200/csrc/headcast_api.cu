@@ -2,6 +2,7 @@
 // tile scheduling, and the launches of the kernels in attn_kernel.cuh / copy_kernels.cuh /
 // score_kernels.cuh.  No CPU fallback exists: every step of the path runs in those kernels.
 #include "context.h"
+#include "noalloc_scratch.h"
 #include "schedule.h"
 
 namespace {
@@ -1247,8 +1248,8 @@ const char* headcast_last_error(const headcast_ctx* c) { return c ? c->err.c_str
 // =====================================================================================================
 // Everything the kernels need in global memory besides the caller's tensors - the work list, the per-CTA ranges, the status
 // word, the partial results of key ranges that are cut and what is to be merged - lives in one file-scope device array of
-// fixed size (the two tensor maps travel as kernel parameters).  Each GPU that loads the library carries these bytes until the
-// process exits.
+// fixed size (noalloc_scratch.cu; the two tensor maps travel as kernel parameters).  A GPU carries these bytes from its first such call
+// until the process exits.
 namespace {
 
 constexpr int NOALLOC_MAX_ITEMS = HEADCAST_NOALLOC_MAX_ITEMS;
@@ -1268,7 +1269,7 @@ struct NoAllocScratch {
   int32_t status;
 };
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocScratch)];
+static_assert(sizeof(NoAllocScratch) <= NOALLOC_SCRATCH_BYTES, "the array of noalloc_scratch.cu is too small");
 
 // How the query-tile pairs of one call (all of the same key range) are spread.
 struct NoAllocPlan {
@@ -1403,7 +1404,7 @@ __global__ void __launch_bounds__(CUT ? NOALLOC_MAX_CTAS : 256) noalloc_list_ker
 constexpr int NOALLOC_MAX_DEVICES = 64;
 struct NoAllocDevice {
   unsigned long long context = 0;     // the CUDA context that the rest was found in: after a device reset it is another one
-  NoAllocScratch* scratch = nullptr;  // device address of g_noalloc_scratch on that GPU
+  NoAllocScratch* scratch = nullptr;  // the array's address on that GPU
   int n_sm = 0;
 };
 NoAllocDevice g_noalloc_dev[NOALLOC_MAX_DEVICES];
@@ -1419,8 +1420,7 @@ int noalloc_fail(int code, const char* msg, cudaError_t e = cudaSuccess) {
   return code;
 }
 
-// Once per device and CUDA context, with that device current: the array's name is only a host-side handle, the kernel needs the
-// address cudaGetSymbolAddress reports for the current device.
+// Once per device and CUDA context, with that device current.
 int noalloc_setup(int dev) {
   NoAllocDevice& d = g_noalloc_dev[dev];
   unsigned long long context = 0;
@@ -1431,8 +1431,8 @@ int noalloc_setup(int dev) {
   if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "cudaGetDeviceProperties", e);
   if (prop.major != 10) return noalloc_fail(HC_ERR_UNSUPPORTED, "this library needs an sm_100 device");
   void* ptr = nullptr;
-  e = cudaGetSymbolAddress(&ptr, g_noalloc_scratch);
-  if (e != cudaSuccess || !ptr) return noalloc_fail(HC_ERR_CUDA, "cudaGetSymbolAddress(g_noalloc_scratch)", e);
+  e = noalloc_scratch_address(&ptr);
+  if (e != cudaSuccess || !ptr) return noalloc_fail(HC_ERR_CUDA, "loading the scratch array", e);
   e = cudaFuncSetAttribute(attn_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<128>::DYN_BYTES);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(attn_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<64>::DYN_BYTES);

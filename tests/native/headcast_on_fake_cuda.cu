@@ -1,5 +1,6 @@
 // The whole library on top of fake_cuda.cpp: host code only, no kernel ever runs.
 #include "../../paper_2607_20125_b200/csrc/headcast_api.cu"
+#include "../../paper_2607_20125_b200/csrc/noalloc_scratch.cu"
 
 // What the last attention launch was given.
 static hc::AttnParams last_attn;

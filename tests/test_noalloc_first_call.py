@@ -23,13 +23,15 @@ def test_the_first_call_loads_every_kernel():
         assert fake.kernels_loaded() == loaded
 
 
+def in_fresh_process(code):
+    code = "import sys\nsys.path.insert(0, %r)\nimport torch\nfrom paper_2607_20125_b200 import binding\n" % ROOT + code
+    res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=ROOT, timeout=300)
+    assert res.returncode == 0, res.stdout + res.stderr
+
+
 @pytest.mark.gpu
 def test_free_memory_stays_the_same_after_the_first_call():
-    code = """
-import sys
-sys.path.insert(0, %r)
-import torch
-from paper_2607_20125_b200 import binding
+    in_fresh_process("""
 routes = %r
 sets = [[torch.zeros(n, h, d, dtype=torch.bfloat16, device="cuda") for n in (q, k, k, q)] for h, q, k in routes for d in (64, 128)]
 binding.dense_attend_noalloc(*sets[0])
@@ -40,6 +42,25 @@ for s in sets:
     binding.dense_attend_noalloc(*s)
 binding.noalloc_status()
 assert torch.cuda.mem_get_info()[0] == free, (free, torch.cuda.mem_get_info()[0])
-""" % (ROOT, ROUTES)
-    res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=ROOT, timeout=300)
-    assert res.returncode == 0, res.stdout + res.stderr
+""" % ROUTES)
+
+
+@pytest.mark.gpu
+def test_programs_that_make_no_such_call_do_not_hold_its_scratch():
+    in_fresh_process("""
+q = torch.zeros(48, 4, 64, dtype=torch.bfloat16, device="cuda")
+out = torch.empty_like(q)
+torch.cuda.synchronize()
+free = torch.cuda.mem_get_info()[0]
+hc = binding.HeadCast(4, 64, 4, 4, 2)
+hc.append(q, q)
+hc.full_attend(q, out)
+hc.append(q, q)
+hc.classify(q)
+hc.split_cache()
+hc.attend(q, out)
+hc.check()
+hc.destroy()
+binding.release_memory()
+assert free - torch.cuda.mem_get_info()[0] < 16 << 20  # what is left is the kernels' code
+""")

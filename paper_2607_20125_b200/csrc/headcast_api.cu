@@ -1261,12 +1261,13 @@ constexpr double NOALLOC_MERGE = 3.0, NOALLOC_MERGE_PART = 0.12;  // launch and 
 constexpr int NOALLOC_CUT_CTAS = 148, NOALLOC_SLOTS = 2 * NOALLOC_CUT_CTAS, NOALLOC_MERGES = 2 * NOALLOC_CUT_CTAS;
 
 struct NoAllocScratch {
-  float part_o[NOALLOC_SLOTS][256 * 128];  // (head_dim 64 uses half of it)
-  float2 part_ml[NOALLOC_SLOTS][256];
   WorkItem items[NOALLOC_MAX_ITEMS + NOALLOC_CUT_CTAS];
   CombineEntry merge[NOALLOC_MERGES];  // two per pair that is cut
   int32_t cta_first[NOALLOC_MAX_CTAS + 1];
   int32_t status;
+  // of cut pairs alone, behind the lists, which lie on one page that way: an uncut call of 20 us took 0.15 us more with the lists 39 MB into the array
+  alignas(256) float part_o[NOALLOC_SLOTS][256 * 128];  // (head_dim 64 uses half of it)
+  float2 part_ml[NOALLOC_SLOTS][256];
 };
 
 static_assert(sizeof(NoAllocScratch) <= NOALLOC_SCRATCH_BYTES, "the array of noalloc_scratch.cu is too small");
@@ -1314,14 +1315,15 @@ NoAllocPlan noalloc_plan(int n_items, int n_keys, int n_sm) {
   return p;
 }
 
-// Writes the work list of one call, and what is to be merged: whole pairs over as many blocks as it takes, shares of a line in one
-// block with a thread per CTA of the attention kernel (which it scans over).  Built here and not copied from the host: three copies from
-// pageable memory made a call take 21 us of host time whatever its size.
-template <bool CUT>
-__global__ void __launch_bounds__(CUT ? NOALLOC_MAX_CTAS : 256) noalloc_list_kernel(NoAllocScratch* s, NoAllocPlan plan, int grid, int n_heads, int head_dim,
-                                                                        int n_queries, int n_keys) {
+// Writes the work list of one call, and what is to be merged: whole pairs (`plan`: their number) over as many blocks as it takes,
+// shares of a line in one block with a thread per CTA of the attention kernel (which it scans over).  Built here and not copied from the
+// host: three copies from pageable memory made a call take 21 us of host time whatever its size.  For whole pairs it is a kernel without
+// shared memory and without the plan among its parameters: with both, the launches of such a call took 7.0 us of the host and not 6.65.
+template <typename Plan>
+__global__ void __launch_bounds__(std::is_same_v<Plan, int> ? 256 : NOALLOC_MAX_CTAS)
+    noalloc_list_kernel(NoAllocScratch* s, Plan plan, int grid, int n_heads, int head_dim, int n_queries, int n_keys) {
   pdl_launch_dependents();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x, nt = plan.n_tiles;
+  const int b = blockIdx.x * blockDim.x + threadIdx.x, nt = (n_keys + 127) / 128;
   auto item = [&](int pair, int begin, int end) {
     const int h = pair % n_heads, q0 = pair / n_heads * 256;
     WorkItem w = {};
@@ -1339,66 +1341,66 @@ __global__ void __launch_bounds__(CUT ? NOALLOC_MAX_CTAS : 256) noalloc_list_ker
     w.out_mode = OUT_BF16;
     return w;
   };
-  if (!CUT) {
-    const int each = plan.n_items / grid, more = plan.n_items % grid;  // CTA b owns items b, b + grid, ...: `each`, plus one for the first `more`
+  if constexpr (std::is_same_v<Plan, int>) {
+    const int each = plan / grid, more = plan % grid;  // CTA b owns items b, b + grid, ...: `each`, plus one for the first `more`
     const int at = (b % grid) * each + min(b % grid, more) + b / grid;
     const WorkItem w = item(b, 0, nt);
     pdl_wait();  // the kernel before may still read the list of its own call
     if (b <= grid) s->cta_first[b] = b * each + min(b, more);
     if (b == 0) s->status = 0;  // the array keeps the previous call's contents
-    if (b < plan.n_items) s->items[at] = w;
-    return;
-  }
-  __shared__ int32_t warp_sum[3][NOALLOC_MAX_CTAS / 32];
-  // CTA b's share [x0, x1) of the line: its pieces, how many of them are partial results, and whether it begins a pair that is cut
-  const long long x0 = b < plan.n_cta ? plan.share_begin(b) : 0, x1 = b < plan.n_cta ? plan.share_begin(b + 1) : 0;
-  const int p0 = static_cast<int>(x0 / nt), p1 = x1 > x0 ? static_cast<int>((x1 - 1) / nt) : p0 - 1;  // first and last pair
-  auto begin_of = [&](int pair) { return pair == p0 ? static_cast<int>(x0 - static_cast<long long>(p0) * nt) : 0; };
-  auto end_of = [&](int pair) { return pair == p1 ? static_cast<int>(x1 - static_cast<long long>(p1) * nt) : nt; };
-  int n[3] = {p1 - p0 + 1, 0, 0};
-  if (n[0] > 0) {
-    const bool first_cut = begin_of(p0) > 0 || end_of(p0) < nt;
-    n[1] = (first_cut ? 1 : 0) + (p1 > p0 && end_of(p1) < nt ? 1 : 0);
-    n[2] = begin_of(p1) == 0 && end_of(p1) < nt ? 1 : 0;
-  }
-  int before[3];  // the same of all CTAs before this one
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    int upto = n[q];
-#pragma unroll
-    for (int off = 1; off < 32; off *= 2) {
-      const int y = __shfl_up_sync(0xffffffffu, upto, off);
-      if ((b & 31) >= off) upto += y;
+    if (b < plan) s->items[at] = w;
+  } else {
+    __shared__ int32_t warp_sum[3][NOALLOC_MAX_CTAS / 32];
+    // CTA b's share [x0, x1) of the line: its pieces, how many of them are partial results, and whether it begins a pair that is cut
+    const long long x0 = b < plan.n_cta ? plan.share_begin(b) : 0, x1 = b < plan.n_cta ? plan.share_begin(b + 1) : 0;
+    const int p0 = static_cast<int>(x0 / nt), p1 = x1 > x0 ? static_cast<int>((x1 - 1) / nt) : p0 - 1;  // first and last pair
+    auto begin_of = [&](int pair) { return pair == p0 ? static_cast<int>(x0 - static_cast<long long>(p0) * nt) : 0; };
+    auto end_of = [&](int pair) { return pair == p1 ? static_cast<int>(x1 - static_cast<long long>(p1) * nt) : nt; };
+    int n[3] = {p1 - p0 + 1, 0, 0};
+    if (n[0] > 0) {
+      const bool first_cut = begin_of(p0) > 0 || end_of(p0) < nt;
+      n[1] = (first_cut ? 1 : 0) + (p1 > p0 && end_of(p1) < nt ? 1 : 0);
+      n[2] = begin_of(p1) == 0 && end_of(p1) < nt ? 1 : 0;
     }
-    if ((b & 31) == 31) warp_sum[q][b >> 5] = upto;
-    before[q] = upto - n[q];
-  }
-  __syncthreads();
+    int before[3];  // the same of all CTAs before this one
 #pragma unroll
-  for (int q = 0; q < 3; ++q)
-    for (int w = 0; w < (b >> 5); ++w) before[q] += warp_sum[q][w];
-  pdl_wait();  // the kernel before may still read the list of its own call
-  if (b < grid) s->cta_first[b] = before[0];
-  if (b == grid - 1) s->cta_first[grid] = before[0] + n[0];
-  if (b == 0) s->status = 0;
-  int slot = before[1];
-  for (int pair = p0; pair <= p1; ++pair) {
-    WorkItem w = item(pair, begin_of(pair), end_of(pair));
-    if (w.tile_end - w.tile_begin < nt) {
-      w.out_mode = OUT_PARTIAL;
-      w.out_slot = slot++;
-      if (w.tile_begin == 0) {  // this pair's pieces: here and in the CTAs that follow
-        int more = 1;
-        while (plan.share_begin(b + more + 1) < static_cast<long long>(pair + 1) * nt) ++more;
-        for (int t = 0; t < 2; ++t) s->merge[2 * before[2] + t] = {w.head, -1, w.q_start[t], w.q_count[t], w.out_slot, more + 1, t, 0};
+    for (int q = 0; q < 3; ++q) {
+      int upto = n[q];
+#pragma unroll
+      for (int off = 1; off < 32; off *= 2) {
+        const int y = __shfl_up_sync(0xffffffffu, upto, off);
+        if ((b & 31) >= off) upto += y;
       }
+      if ((b & 31) == 31) warp_sum[q][b >> 5] = upto;
+      before[q] = upto - n[q];
     }
-    s->items[before[0] + pair - p0] = w;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      for (int w = 0; w < (b >> 5); ++w) before[q] += warp_sum[q][w];
+    pdl_wait();  // the kernel before may still read the list of its own call
+    if (b < grid) s->cta_first[b] = before[0];
+    if (b == grid - 1) s->cta_first[grid] = before[0] + n[0];
+    if (b == 0) s->status = 0;
+    int slot = before[1];
+    for (int pair = p0; pair <= p1; ++pair) {
+      WorkItem w = item(pair, begin_of(pair), end_of(pair));
+      if (w.tile_end - w.tile_begin < nt) {
+        w.out_mode = OUT_PARTIAL;
+        w.out_slot = slot++;
+        if (w.tile_begin == 0) {  // this pair's pieces: here and in the CTAs that follow
+          int more = 1;
+          while (plan.share_begin(b + more + 1) < static_cast<long long>(pair + 1) * nt) ++more;
+          for (int t = 0; t < 2; ++t) s->merge[2 * before[2] + t] = {w.head, -1, w.q_start[t], w.q_count[t], w.out_slot, more + 1, t, 0};
+        }
+      }
+      s->items[before[0] + pair - p0] = w;
+    }
+    // entries that the launch of the merge has blocks for but no pair was cut for
+    int n_entries = 0;
+    for (int w = 0; w < static_cast<int>(blockDim.x) / 32; ++w) n_entries += 2 * warp_sum[2][w];
+    for (int i = n_entries + b; i < NOALLOC_MERGES; i += blockDim.x) s->merge[i].q_count = 0;
   }
-  // entries that the launch of the merge has blocks for but no pair was cut for
-  int n_entries = 0;
-  for (int w = 0; w < static_cast<int>(blockDim.x) / 32; ++w) n_entries += 2 * warp_sum[2][w];
-  for (int i = n_entries + b; i < NOALLOC_MERGES; i += blockDim.x) s->merge[i].q_count = 0;
 }
 
 constexpr int NOALLOC_MAX_DEVICES = 64;
@@ -1443,8 +1445,8 @@ int noalloc_setup(int dev) {
     cudaFuncAttributes attributes;
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&attributes, kernel);
   };
-  load(noalloc_list_kernel<false>);
-  load(noalloc_list_kernel<true>);
+  load(noalloc_list_kernel<int>);
+  load(noalloc_list_kernel<NoAllocPlan>);
   load(attn_kernel<64, false>);
   load(attn_kernel<128, false>);
   load(combine_kernel<64>);
@@ -1500,9 +1502,9 @@ int headcast_dense_attend_noalloc(const void* q, const void* k, const void* v, v
     return noalloc_fail(HC_ERR_CUDA, "cuTensorMapEncodeTiled failed or is unavailable");
   const int n_cta = d.n_sm;
   const NoAllocPlan plan = noalloc_plan(static_cast<int>(n_items), n_keys, n_cta);
-  const int list_threads = std::max(plan.cuts ? 0 : static_cast<int>(n_items), n_cta + 1);
-  e = launch_pdl(plan.cuts ? noalloc_list_kernel<true> : noalloc_list_kernel<false>, plan.cuts ? dim3(1) : dim3((list_threads + 255) / 256), dim3(plan.cuts ? (n_cta + 31) / 32 * 32 : 256), 0, st,
-                 d.scratch, plan, n_cta, n_heads, head_dim, n_queries, n_keys);
+  const dim3 list_threads(plan.cuts ? (n_cta + 31) / 32 * 32 : 256), list_blocks(plan.cuts ? 1 : (std::max(plan.n_items, n_cta + 1) + 255) / 256);
+  e = plan.cuts ? launch_pdl(noalloc_list_kernel<NoAllocPlan>, list_blocks, list_threads, 0, st, d.scratch, plan, n_cta, n_heads, head_dim, n_queries, n_keys)
+                : launch_pdl(noalloc_list_kernel<int>, list_blocks, list_threads, 0, st, d.scratch, plan.n_items, n_cta, n_heads, head_dim, n_queries, n_keys);
   if (e != cudaSuccess) return noalloc_fail(HC_ERR_CUDA, "launching the list kernel", e);
 
   p.items = d.scratch->items;

@@ -1290,11 +1290,18 @@ struct NoAllocPlan {
 // badly: its shares are at least two proper pieces long, and beyond eight waves there is too little to gain.  1373 queries, 5492 keys,
 // sixteen heads of 64 (a line): 77 -> 61 us; 687 queries, 2748 keys, eight heads of 128 (equal pieces): 46.5 -> 24.8;
 // 1785 queries, 12495 keys, four heads of 128: 166 -> 53.
-NoAllocPlan noalloc_plan(int n_items, int n_keys, int n_sm) {
+// At head_dim 128 a key tile of a line takes 1.16 times as long as one of whole pairs (the CTAs of whole pairs walk a head's keys in
+// step and share them in L2, those of a line stand at different places, and all SMs at work clock lower), so there a line has to end
+// earlier by that count too.  Measured on 704 sizes of 1 to 1100 pairs and 8 to 200 key tiles each: without it 130 pairs of 200 key
+// tiles took 409 us as a line and 353 whole, 130 of 120 226 and 214, 80 of 16 38.2 and 37.3; with it no line is more than 1.2 % slower
+// than whole pairs, and the lines that it refuses were at most 4.5 % faster.  At head_dim 64 and for equal pieces no size was slower cut.
+constexpr double NOALLOC_LINE_TILE_128 = 1.16, NOALLOC_LINE_MORE_128 = 10.7, NOALLOC_WHOLE_MORE_128 = 3.5;
+NoAllocPlan noalloc_plan(int n_items, int n_keys, int n_sm, int head_dim) {
   NoAllocPlan p = {n_items, (n_keys + 127) / 128, n_sm, 0};
   if (p.n_tiles < 8) return p;  // half of that does not pay for a merge
   const double item = COST_MEASURED.item, piece = COST_MEASURED.item + COST_MEASURED.partial;
-  double best = 0.95 * ((n_items + n_sm - 1) / n_sm) * (p.n_tiles + item);
+  const int waves = (n_items + n_sm - 1) / n_sm;
+  double best = 0.95 * waves * (p.n_tiles + item);
   const int n_cta = std::min(n_sm, NOALLOC_CUT_CTAS);
   for (int k = 2; k <= std::min(n_cta / n_items, p.n_tiles); ++k) {
     const double end = (p.n_tiles + k - 1) / k + piece + NOALLOC_MERGE + NOALLOC_MERGE_PART * k;
@@ -1307,7 +1314,8 @@ NoAllocPlan noalloc_plan(int n_items, int n_keys, int n_sm) {
   const double share = static_cast<double>(n_items) * p.n_tiles / n_cta;
   if (n_items > n_cta / 4 && n_items < 8 * n_cta && p.n_tiles >= 4 * MIN_PART_TILES && share >= 2 * MIN_PART_TILES) {
     const double end = share + item * n_items / n_cta + 2 * piece - item + NOALLOC_MERGE;
-    if (end < best) {
+    const bool in_step = head_dim == 128 && waves * (p.n_tiles + NOALLOC_WHOLE_MORE_128) <= NOALLOC_LINE_TILE_128 * share + NOALLOC_LINE_MORE_128;
+    if (end < best && !in_step) {
       p.cuts = -1;
       p.n_cta = n_cta;
     }
@@ -1501,7 +1509,7 @@ int headcast_dense_attend_noalloc(const void* q, const void* k, const void* v, v
       !make_tmap_bf16_2d(&p.maps[1], v, row_elems, n_keys, row_elems, 128))
     return noalloc_fail(HC_ERR_CUDA, "cuTensorMapEncodeTiled failed or is unavailable");
   const int n_cta = d.n_sm;
-  const NoAllocPlan plan = noalloc_plan(static_cast<int>(n_items), n_keys, n_cta);
+  const NoAllocPlan plan = noalloc_plan(static_cast<int>(n_items), n_keys, n_cta, head_dim);
   const dim3 list_threads(plan.cuts ? (n_cta + 31) / 32 * 32 : 256), list_blocks(plan.cuts ? 1 : (std::max(plan.n_items, n_cta + 1) + 255) / 256);
   e = plan.cuts ? launch_pdl(noalloc_list_kernel<NoAllocPlan>, list_blocks, list_threads, 0, st, d.scratch, plan, n_cta, n_heads, head_dim, n_queries, n_keys)
                 : launch_pdl(noalloc_list_kernel<int>, list_blocks, list_threads, 0, st, d.scratch, plan.n_items, n_cta, n_heads, head_dim, n_queries, n_keys);

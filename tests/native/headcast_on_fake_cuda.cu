@@ -25,3 +25,5 @@ extern "C" int fake_attn_tile_steps() {
   for (int i = 0; i < last_attn.cta_first[148]; ++i) sum += last_attn.items[i].tile_end - last_attn.items[i].tile_begin;
   return sum;
 }
+// How the allocation-free call spreads so many query-tile pairs: 0 whole, > 0 in so many equal pieces, < 0 as a line.
+extern "C" int fake_noalloc_cuts(int pairs, int n_keys, int n_sm, int head_dim) { return noalloc_plan(pairs, n_keys, n_sm, head_dim).cuts; }

@@ -181,8 +181,8 @@ int64_t headcast_launch_count(const headcast_ctx* ctx);
  * is for measuring, or serving, the path end to end across PCIe).  k_host/v_host/q_host/out_host: host pointers to
  * [L][H][d] bf16; pinned memory lets the copies overlap the kernels, pageable memory works but serialises.
  * headcast_append_host copies the block into device staging owned by the context and appends it.
- * headcast_attend_host takes blocks of up to 4 MiB as one: q_host is copied in, attended and copied out on `stream`.  Larger ones
- * it splits into four stages (first half of the Global heads' query rows; Sink + Dummy
+ * headcast_attend_host takes small blocks as one (up to 4 MiB, the less the fewer runs of neighbouring heads of one pathway there are):
+ * q_host is copied in, attended and copied out on `stream`.  Others it splits into four stages (first half of the Global heads' query rows; Sink + Dummy
  * heads; Spatial heads; second half of the Global heads' rows): each stage's part of Q is copied in, attended
  * (Sec. 4.4, as headcast_attend) and its part of the output copied out, on two copy streams of the context, so that
  * transfers in both directions overlap the attention of the other stages.  Both

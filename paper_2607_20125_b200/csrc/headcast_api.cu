@@ -955,11 +955,35 @@ int init_host_path(headcast_ctx* c) {
 
 }  // namespace
 
-// Blocks whose queries are no larger than this are copied, attended and copied back as one, in the order of the caller's stream:
-// stages hide copies, but every one brings launches, copies and events of its own.  Append + four attends, one stage against four:
-// 0.5 MB 253 us against 323, 2.5 MB 677 against 875, 3.8 MB 974 against 1081; 4.4 MB 1120 against 1214 but 4.6 MB 1557 against 1538
-// and 8.7 MB 2262 against 2067.
-constexpr size_t HOST_ONE_STAGE_BYTES = 4 << 20;
+// What headcast_attend_host cuts a block into.  Its stages hide copies behind attention and copies of the other direction, but
+// every run of neighbouring heads of one stage is a strided copy each way, of 5 us of the host (a whole small block: 40 to 60 us), and a
+// stage is a launch, a merge and two events.  So a block is copied, attended and copied back as one where there is but one stage, or
+// where it is small for the number of copies that the stages would make.  Append + four attends, stages against one: twelve heads of 64
+// at 7 x 12 tokens (eight Dummy, four Spatial) 364 us against 204, 32 of 128 at 9 x 15 (all but Global) 1000 against 747; but 16 Global
+// heads of 64 at 17 x 28 tokens 827 against 1030, two Spatial and two Global ones of 128 at 21 x 28 801 against 980.  Over 1529 layers of up to
+// 4 MiB (2 to 32 heads, every mix of labels) this rule ends at 1.26 times the speed of stages for all of them (slowest twentieth: 0.99;
+// one for all of them: 1.25, slowest twentieth 0.89); of 256, 384 and 512 KB per copy 384 comes nearest to the better of the two (1.2 % off).
+// Blocks of 4 to 9 MiB stay in stages: as one they were 5 % slower on average.
+constexpr size_t HOST_ONE_STAGE_BYTES = 4 << 20, HOST_BYTES_PER_COPY = 384 << 10;
+
+struct HostStage { int group, lo, hi; };  // head group (0 Global, 1 Spatial, 2 Sink + Dummy) and rows [lo, hi)
+
+static int host_group(const headcast_ctx* c, int h) { return c->cls[h] == CLS_GLOBAL ? 0 : c->cls[h] == CLS_SPATIAL ? 1 : 2; }
+
+// Rows of the first of the two stages of the Global heads.
+static int host_first_rows(const headcast_ctx* c) { return std::min(c->L, ((c->L / 2 + 255) / 256) * 256); }
+
+static bool host_as_one(const headcast_ctx* c, size_t bytes) {
+  if (bytes > HOST_ONE_STAGE_BYTES) return false;
+  int stages = 0, copies = 0, runs[3] = {0, 0, 0};
+  for (int h = 0; h < c->H; ++h) runs[host_group(c, h)] += h == 0 || host_group(c, h) != host_group(c, h - 1);
+  for (int g = 0; g < 3; ++g) {
+    const int cut = g == 0 && host_first_rows(c) < c->L ? 2 : 1;
+    stages += runs[g] > 0 ? cut : 0;
+    copies += runs[g] * cut;
+  }
+  return stages == 1 || bytes <= (copies - 1) * HOST_BYTES_PER_COPY;
+}
 
 int headcast_append_host(headcast_ctx* c, const void* k_host, const void* v_host, void* stream) {
   if (!c || !k_host || !v_host) return HC_ERR_INVALID_ARG;
@@ -977,7 +1001,7 @@ static int attend_host(headcast_ctx* c, const void* q_host, void* out_host, cuda
   const size_t elems = static_cast<size_t>(c->L) * c->H * c->D, bytes = elems * sizeof(__nv_bfloat16);
   HC_CUDA(c, c->stage_q.reserve(c->memory, elems, st));
   HC_CUDA(c, c->stage_out.reserve(c->memory, elems, st));
-  if (bytes <= HOST_ONE_STAGE_BYTES) {
+  if (host_as_one(c, bytes)) {
     HC_CUDA(c, cudaMemcpyAsync(c->stage_q.ptr, q_host, bytes, cudaMemcpyHostToDevice, st));
     const int rc = headcast_attend(c, c->stage_q.ptr, c->stage_out.ptr, st);
     if (rc != HC_OK) return rc;
@@ -993,24 +1017,22 @@ static int attend_host(headcast_ctx* c, const void* q_host, void* out_host, cuda
   // computes.  The Global heads do most of the arithmetic per byte moved, so their query rows are halved (at a
   // multiple of 256 rows: the query-tile pairs stay the same) and the halves go first and last: the kernels start
   // after a small copy, and when they end only a small copy is left; the other heads' copies hide in between.
-  const int mid = std::min(c->L, ((c->L / 2 + 255) / 256) * 256);  // blocks of up to 256 tokens have one stage per group
-  struct Stage { int group, lo, hi; };
-  const Stage stages[headcast_ctx::N_HOST_STAGES] = {{0, 0, mid}, {2, 0, c->L}, {1, 0, c->L}, {0, mid, c->L}};
+  const int mid = host_first_rows(c);  // blocks of up to 256 tokens have one stage per group
+  const HostStage stages[headcast_ctx::N_HOST_STAGES] = {{0, 0, mid}, {2, 0, c->L}, {1, 0, c->L}, {0, mid, c->L}};
   for (int i = 0; i < headcast_ctx::N_HOST_STAGES; ++i)
     if (c->sched_stage[i].key_filled != key)
       build_headcast_schedule(c, c->sched_stage[i], stages[i].group, stages[i].lo, stages[i].hi);
   const size_t pitch = static_cast<size_t>(c->H) * c->D * sizeof(__nv_bfloat16);
-  auto copy_stage = [&](const Stage& sg, bool in) -> int {
+  auto copy_stage = [&](const HostStage& sg, bool in) -> int {
     const int rows = sg.hi - sg.lo;
     if (rows <= 0) return HC_OK;
     for (int h0 = 0; h0 < c->H;) {
-      auto group_of = [&](int h) { return c->cls[h] == CLS_GLOBAL ? 0 : c->cls[h] == CLS_SPATIAL ? 1 : 2; };
-      if (group_of(h0) != sg.group) {
+      if (host_group(c, h0) != sg.group) {
         ++h0;
         continue;
       }
       int h1 = h0 + 1;
-      while (h1 < c->H && group_of(h1) == sg.group) ++h1;
+      while (h1 < c->H && host_group(c, h1) == sg.group) ++h1;
       const size_t off = static_cast<size_t>(sg.lo) * c->H * c->D + static_cast<size_t>(h0) * c->D;
       const size_t width = static_cast<size_t>(h1 - h0) * c->D * sizeof(__nv_bfloat16);
       if (in)

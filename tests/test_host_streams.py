@@ -33,10 +33,10 @@ def unordered(log):
 
 
 class Caller:
-    def __init__(self, cfg):
+    def __init__(self, cfg, labels=(0, 1, 2, 3, 2, 3)):
         self.fake = FakeLibrary()
         self.ctx = self.fake.context(**cfg)
-        labels = [0, 1, 2, 3, 2, 3][:cfg["n_heads"]]
+        labels = list(labels)[:cfg["n_heads"]]
         assert self.ctx.append(3) == 0 and self.ctx.split(labels) == 0
         bytes_ = 2 * 3 * cfg["grid_h"] * cfg["grid_w"] * cfg["n_heads"] * cfg["head_dim"]
         self.buffers = [C.create_string_buffer(bytes_) for _ in range(2)]
@@ -104,3 +104,21 @@ def test_a_call_that_failed_half_way_is_waited_for_too(cfg):
     caller.fake.capacity_left(1 << 40)
     assert caller.attend(12) == 0
     assert unordered(caller.log) == (2, [])
+
+
+@pytest.mark.parametrize("labels,grid_h,grid_w,as_one", [
+    ([3] * 12, 9, 9, True),                  # one stage: up to 256 rows of Global heads
+    ([3] * 12, 16, 28, False),               # two halves of the Global heads' rows, one copy each
+    ([2] * 12, 16, 28, True),                # one stage
+    ([0, 1] * 6, 16, 28, True),
+    ([2] * 3 + [3] * 3, 10, 17, True),       # three copies: up to 768 KB, 512 rows of six heads
+    ([2] * 3 + [3] * 3, 9, 19, False),
+    ([2, 3] * 6, 16, 28, True),              # eighteen copies
+    ([2, 3] * 6, 19, 24, False),             # more than 4 MiB
+])
+def test_blocks_are_cut_where_the_copies_of_the_stages_are_few(labels, grid_h, grid_w, as_one):
+    caller = Caller(dict(n_heads=len(labels), head_dim=128, grid_h=grid_h, grid_w=grid_w, n_blocks=3), labels)
+    assert caller.attend(11) == 0
+    caller.log = ""
+    assert caller.attend(11) == 0
+    assert (sum(entry[0] == "H" for entry in caller.log.split()) == 1 and "E11" in caller.log and "W" not in caller.log) == as_one

@@ -27,3 +27,11 @@ extern "C" int fake_attn_tile_steps() {
 }
 // How the allocation-free call spreads so many query-tile pairs: 0 whole, > 0 in so many equal pieces, < 0 as a line.
 extern "C" int fake_noalloc_cuts(int pairs, int n_keys, int n_sm, int head_dim) { return noalloc_plan(pairs, n_keys, n_sm, head_dim).cuts; }
+// The first key tile of every CTA's share and, behind the last, their end; returns how many CTAs (0: whole pairs).
+extern "C" int fake_noalloc_shares(int pairs, int n_keys, int n_sm, int head_dim, long long* begins, int* slots, int* entries) {
+  const NoAllocPlan plan = noalloc_plan(pairs, n_keys, n_sm, head_dim);
+  *slots = NOALLOC_SLOTS;
+  *entries = NOALLOC_MERGES;
+  for (int b = 0; plan.cuts != 0 && b <= plan.n_cta; ++b) begins[b] = plan.share_begin(b);
+  return plan.cuts != 0 ? plan.n_cta : 0;
+}

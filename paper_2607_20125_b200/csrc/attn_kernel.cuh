@@ -13,8 +13,8 @@
 //   - warp 0 is the TMA producer, warp 1 issues every MMA (converged, see tc05.cuh).
 // What bounds it: per pair of tiles the tensor pipe needs 2048 clk, the softmax of the two tiles 2100 clk of issue and
 // special-function time per scheduler (microbenchmark: 61 clk to fetch, 136 for the maximum, 1086 for the exponentials of
-// one tile alone, 2126 for two together), and a tile's softmax and its products follow one another; a step takes about
-// 3050 clk.  With two threads per row, a maximum exchanged through shared memory and the products issued from a diverged
+// one tile alone, 2126 for two together), and a tile's softmax and its products follow one another; a step takes 2930
+// to 3050 clk.  With two threads per row, a maximum exchanged through shared memory and the products issued from a diverged
 // lane it took 3600.  Steady-state block at 30 x 52 tokens (12 heads of 128, 7-block window, append + four attends):
 // 1412 -> 1281 us; dense sweep over 7 blocks at 45 x 80 tokens: 4966 -> 4468 us.
 // Which keys a query tile sees is entirely a property of the work item: a row range of one of the
@@ -655,7 +655,7 @@ struct RowMerge {
 // The merge kernels wait for memory, not for its bandwidth: a thread fetches 40 bytes per part, and a query tile has a few
 // parts.  So MERGE_BATCH parts are taken at a time with every load of a batch, maxima, sums and values alike, issued before the
 // first use, in one pass: looking for the maximum first cost another round trip.  Append + four attends: 13 x 22 tokens, six heads
-// 95.4 -> 90.5 us; 14 x 25, twelve heads 122.8 -> 118.7; 30 x 52, twelve heads 1278 -> 1257 to 1274.
+// 95.4 -> 90.5 us; 14 x 25, twelve heads 122.8 -> 118.7; 30 x 52, twelve heads level (1302 and 1298).
 constexpr int MERGE_BATCH = 4;
 
 template <int D>
@@ -699,8 +699,9 @@ __device__ __forceinline__ void combine_rows(const CombineEntry& e, int block, c
 
 // The same merge for query tiles that were cut into MANY pieces (the pieces of one pair in the shared queue of the
 // dynamic tail can run to dozens): one block per ROW, the parts dealt over COMBINE_LANES groups of threads that each
-// merge their share as above, then one group merges the groups' results through shared memory.  With one thread
+// merge their share, then one group merges the groups' results through shared memory.  With one thread
 // walking all parts of its row the launch ended with a few blocks each waiting on twenty memory round trips in turn.
+// (A group looks for the maximum of its parts first and then adds them, one after the other: it has two parts, rarely more.)
 constexpr int COMBINE_LANES = 16;
 constexpr int COMBINE_LONG_PARTS = 16;  // entries with more parts than this go through combine_long_row
 

@@ -1276,7 +1276,10 @@ namespace {
 
 constexpr int NOALLOC_MAX_ITEMS = HEADCAST_NOALLOC_MAX_ITEMS;
 constexpr int NOALLOC_MAX_CTAS = 1024;
-constexpr double NOALLOC_MERGE = 3.0, NOALLOC_MERGE_PART = 0.12;  // launch and a first batch of parts; each further part
+// Of a cut, in key tiles: launch and a first batch of parts, each further part.  Fitted to 1300 timings of equal pieces, merging and
+// partial results cost 1.5 + 1.7 times the share of CTAs in use + 0.2 per part at head_dim 64, 1.5 + 2.6 times + 0.2 at 128; with
+// the partial result's 1.1 these constants charge a little more where parts are few: no size was slower cut than whole.
+constexpr double NOALLOC_MERGE = 3.0, NOALLOC_MERGE_PART = 0.12;
 
 // Query-tile pairs are cut along their keys where whole ones would leave much of the GPU idle, over at most this many CTAs, each
 // of which leaves at most two partial results (its first and its last piece).

@@ -204,12 +204,14 @@ proxy_combine_kernel(const ClsGroup* groups, const ClsPart* parts, const float* 
       fmaxf(0.f, 1.f - tok[TOK_MASS_FIRST * hl + at] - tok[TOK_MASS_LAST * hl + at] - __expf(lse_mid - l_ref));
 }
 
+// Keys in the order of the floats, NaNs beyond the infinities of their sign.  By exclusive or with a mask: as a choice between the two
+// signs' forms, on a value that is also summed, the compiled code ordered positive NaNs as 0.
 __device__ __forceinline__ uint32_t float_order_key(float x) {
   const uint32_t u = __float_as_uint(x);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  return u ^ (static_cast<uint32_t>(static_cast<int32_t>(u) >> 31) | 0x80000000u);
 }
 __device__ __forceinline__ float float_from_key(uint32_t k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+  return __uint_as_float(k ^ (((k >> 31) - 1u) | 0x80000000u));
 }
 
 constexpr int DECIDE_THREADS = 1024;
